@@ -1,138 +1,266 @@
 // Step 2 — rank allocation (Sec. 3.2: min-max normalisation, Eq. 4 water-filling, Algorithm 1's
-// water level) for every (sequence, layer), one CTA each.
+// water level) for every (sequence, layer), one thread-block cluster each.
 //
-// All float arithmetic is IEEE fp32 with explicit round-to-nearest intrinsics (no contraction
-// into FMA), so the ranks are a deterministic function of the salience bits:
+// All float arithmetic is IEEE fp32 with explicitly rounded intrinsics (no contraction into FMA),
+// so the ranks are a deterministic function of the salience bits:
 //   s_hat = (s - min) / (max - min)            (1 if max == min, or in UNIFORM mode)
 //   x     = fl(fl(lambda * s_hat) + r_min)
 //   rank  = r_max if x >= r_max else max(r_min, floor(x))
-// lambda is the largest finite fp32 value >= 0 whose ranks sum to at most B_c, found by bisection
-// over the fp32 bit patterns (the sum is non-decreasing in lambda): 31 block-wide counts.
+// lambda is the largest finite fp32 value >= 0 whose ranks sum to at most B_c, searched over the
+// fp32 bit patterns (the sum is non-decreasing in lambda).
+//
+// What bounds it: the chain of sums over all tokens, one after another. So each CTA of the cluster
+// takes a contiguous share of the tokens, normalises it once into shared memory (the division is
+// what a pass over the salience costs most), and each pass sums the ranks at 15 water levels at
+// once, with one cluster barrier, instead of halving the bracket.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace vr {
 
 namespace {
 
-constexpr int kThreads = 1024;
-
-__device__ __forceinline__ int rank_of(float lam, float sh, int r_min, int r_max) {
-  const float x = __fadd_rn(__fmul_rn(lam, sh), (float)r_min);
-  if (x >= (float)r_max) return r_max;          // also catches x = +inf
-  const int f = (int)floorf(x);
-  return f < r_min ? r_min : f;
-}
+constexpr int kThreads = 256;          // few warps: each pass ends in 15 warp sums and two barriers
+constexpr int kWarps = kThreads / 32;
+constexpr int kCand = 15;              // water levels per pass
+constexpr int kMaxCluster = 8;         // portable cluster size
+constexpr int64_t kMaxCached = 49152;  // normalised saliences kept in shared memory (192 KB)
 
 __device__ __forceinline__ float shat_of(float s, float mn, float den, bool flat) {
-  return flat ? 1.0f : __fdiv_rn(__fsub_rn(s, mn), den);
+  const float v = flat ? 1.0f : __fdiv_rn(__fsub_rn(s, mn), den);
+  return v == v ? v : 0.f;   // NaN salience: rank r_min, as x = r_min gives
 }
 
-// Block-wide sum of one int64 per thread, result returned to every thread.
-__device__ int64_t block_sum(int64_t v, int64_t* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// floor(min(x, r_max)) + 0x4B000000 as an integer, x = fl(fl(lam * sh) + r_min) in [r_min, inf]: adding
+// 2^23 with rounding toward minus infinity leaves floor(x) in the mantissa (x <= 128).
+__device__ __forceinline__ uint32_t rank_bits(float lam, float sh, float r_min, float r_max) {
+  const float x = fminf(__fadd_rn(__fmul_rn(lam, sh), r_min), r_max);
+  return __float_as_uint(__fadd_rd(x, 8388608.f));
+}
+constexpr uint32_t kRankBias = 0x4B000000u;
+
+__device__ __forceinline__ void warp_stats(float& mn, float& mx, float& sum) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    int64_t x = lane < (int)(blockDim.x >> 5) ? red[lane] : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) red[32] = x;
+  for (int o = 16; o > 0; o >>= 1) {
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
-  __syncthreads();
-  return red[32];
 }
 
+// Offset of the k-th of kCand levels around a guess whose error is expected within `reach` (in units of
+// the bit pattern): none at the guess, then factors of four (two near the ends) on both sides.
+__device__ __forceinline__ int64_t spread(int k, int64_t reach) {
+  const int m = k - kCand / 2;
+  const int a = m < 0 ? -m : m;
+  const int64_t d = a == 0 ? 0 : reach >> (2 * (kCand / 2 - a));
+  return m < 0 ? -d : d;
+}
+
+struct AllocSmem {
+  float mm[kMaxCluster][3];                        // every CTA's min, max and sum
+  long long tot[2][kMaxCluster][kCand + 1];        // every CTA's sums, by pass parity
+  unsigned long long wsum[kCand][kWarps + 1];
+  float fred[3][kWarps];
+};
+
+// grid (C B L) in clusters of C CTAs, one cluster for each (sequence, layer); CTA `rank` of it takes
+// `share` tokens, the first `cached` of them held in the dynamic shared memory.
 __global__ void __launch_bounds__(kThreads)
 allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
-                int64_t* __restrict__ realized, int32_t* __restrict__ dev_status, Shape s) {
-  __shared__ int64_t red[33];
-  __shared__ float fred[2][32];
-  const int64_t bl = blockIdx.x;
+                int64_t* __restrict__ realized, int32_t* __restrict__ dev_status, Shape s,
+                int64_t share, int64_t cached) {
+  extern __shared__ float sh_cache[];
+  __shared__ AllocSmem sm;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int64_t bl = blockIdx.x / C;
   const int64_t n = s.n_coded;
   const float* sl = sal ? sal + bl * n : nullptr;
   uint8_t* rk = ranks + bl * s.N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t t0 = min(n, rank * share), cnt = min(n, t0 + share) - t0;   // this CTA's tokens
 
   // exact set: full rank
-  for (int64_t t = n + tid; t < s.N; t += blockDim.x) rk[t] = (uint8_t)s.r_max;
+  if (rank == 0)
+    for (int64_t t = n + tid; t < s.N; t += kThreads) rk[t] = (uint8_t)s.r_max;
 
-  // min / max over the coded set (exact in any order)
-  float mn = INFINITY, mx = -INFINITY;
-  const bool uniform = (s.mode == VARRATE_UNIFORM) || sl == nullptr;
-  if (!uniform) {
-    for (int64_t t = tid; t < n; t += blockDim.x) {
-      const float v = sl[t];
-      mn = fminf(mn, v);
-      mx = fmaxf(mx, v);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    if (lane == 0) { fred[0][warp] = mn; fred[1][warp] = mx; }
-    __syncthreads();
-    mn = INFINITY; mx = -INFINITY;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) { mn = fminf(mn, fred[0][i]); mx = fmaxf(mx, fred[1][i]); }
-  }
-  const bool flat = uniform || !(mx > mn);
-  const float den = flat ? 1.0f : __fsub_rn(mx, mn);
-
-  int mode_fixed = -1;    // -1: bisection, otherwise every coded token gets this rank
+  int mode_fixed = -1;    // -1: search, otherwise every coded token gets this rank
   if (n == 0) {
     mode_fixed = s.r_max;
   } else if ((int64_t)s.r_min * n > s.Bc) {
     mode_fixed = s.r_min;
-    if (tid == 0) raise_status(dev_status, VARRATE_FLOOR_BINDS);
+    if (rank == 0 && tid == 0) raise_status(dev_status, VARRATE_FLOOR_BINDS);
   } else if (s.Bc >= (int64_t)s.r_max * n) {
     mode_fixed = s.r_max;
   }
+  if (mode_fixed >= 0) {   // uniform over the cluster: no barrier is skipped by part of it
+    for (int64_t i = tid; i < cnt; i += kThreads) rk[t0 + i] = (uint8_t)mode_fixed;
+    if (rank == 0 && tid == 0 && realized) realized[bl] = (int64_t)mode_fixed * n;
+    return;
+  }
 
-  float lam = 0.f;
-  if (mode_fixed < 0) {
-    auto total = [&](uint32_t bits) -> int64_t {
-      const float l = __uint_as_float(bits);
-      int64_t acc = 0;
-      for (int64_t t = tid; t < n; t += blockDim.x)
-        acc += rank_of(l, shat_of(sl ? sl[t] : 0.f, mn, den, flat), s.r_min, s.r_max);
-      return block_sum(acc, red);
-    };
-    uint32_t lo;
-    if (total(0x7F7FFFFFu) <= s.Bc) {
-      lo = 0x7F7FFFFFu;
-    } else {
-      lo = 0;
-      uint32_t hi = 0x7F7FFFFFu;
-      while (hi - lo > 1) {
-        const uint32_t mid = lo + (hi - lo) / 2;
-        if (total(mid) <= s.Bc) lo = mid; else hi = mid;
+  // min / max over the coded set (exact in any order), and the sum, which only places the first levels
+  float mn = INFINITY, mx = -INFINITY, sum = 0.f;
+  const bool uniform = (s.mode == VARRATE_UNIFORM) || sl == nullptr;
+  if (!uniform) {
+    for (int64_t i = tid; i < cnt; i += kThreads) {
+      const float v = sl[t0 + i];
+      if (i < cached) sh_cache[i] = v;
+      mn = fminf(mn, v);
+      mx = fmaxf(mx, v);
+      sum += v;
+    }
+    warp_stats(mn, mx, sum);
+    if (lane == 0) { sm.fred[0][warp] = mn; sm.fred[1][warp] = mx; sm.fred[2][warp] = sum; }
+    __syncthreads();
+    if (warp == 0) {
+      mn = lane < kWarps ? sm.fred[0][lane] : INFINITY;
+      mx = lane < kWarps ? sm.fred[1][lane] : -INFINITY;
+      sum = lane < kWarps ? sm.fred[2][lane] : 0.f;
+      warp_stats(mn, mx, sum);
+      if (lane < C) {
+        float* peer = cluster.map_shared_rank(&sm.mm[0][0], lane) + 3 * rank;
+        peer[0] = mn;
+        peer[1] = mx;
+        peer[2] = sum;
       }
     }
-    lam = __uint_as_float(lo);
+  }
+  cluster.sync();
+  if (!uniform) {
+    mn = INFINITY; mx = -INFINITY; sum = 0.f;
+    for (int c = 0; c < C; ++c) {
+      mn = fminf(mn, sm.mm[c][0]);
+      mx = fmaxf(mx, sm.mm[c][1]);
+      sum += sm.mm[c][2];
+    }
+  }
+  const bool flat = uniform || !(mx > mn);
+  const float den = flat ? 1.0f : __fsub_rn(mx, mn);
+  // a thread normalises, and reads in every pass, the entries it loaded itself
+  for (int64_t i = tid; i < min(cnt, cached); i += kThreads)
+    sh_cache[i] = shat_of(uniform ? 0.f : sh_cache[i], mn, den, flat);
+  auto shat = [&](int64_t i) {
+    return i < cached ? sh_cache[i] : shat_of(uniform ? 0.f : sl[t0 + i], mn, den, flat);
+  };
+  const float fmin_r = (float)s.r_min, fmax_r = (float)s.r_max;
+  const bool wide = share >= (int64_t(1) << 24);   // a warp's sum may pass 32 bits
+
+  // The answer is the largest b with total(b) <= B_c: total(lo) <= B_c < total(hi), where lo = 0 and the
+  // pattern after the largest finite value stand in at the start. Any levels that bracket it closer give
+  // the same answer. The first pass spreads them around the level that would spend the budget if no
+  // rank met r_max; then the totals at both ends interpolate a guess (the total is close to linear in
+  // a narrow bracket), and every other pass cuts the bracket evenly, to a sixteenth, which bounds the
+  // number of passes whatever the salience looks like.
+  uint32_t lo = 0, hi = 0x7F800000u;
+  long long tot_lo = (long long)s.r_min * n, tot_hi = (long long)s.r_max * n;
+  const float mean = flat ? 1.f : (sum / (float)n - mn) / den;
+  const float first = ((float)((double)s.Bc / (double)n) - fmin_r + 0.5f) / mean;
+  for (int pass = 0; hi - lo > 1; ++pass) {
+    const uint32_t span = hi - lo, step = (span + kCand) / (kCand + 1);
+    const bool even = span <= kCand + 1 || (pass == 0 ? !(first > 0.f && first < 3e38f) : pass % 3 == 0);
+    int64_t guess, reach;
+    if (pass == 0) {
+      guess = __float_as_uint(first);
+      reach = 1 << 26;                       // eight octaves either way
+    } else {
+      guess = lo + (int64_t)((float)span * ((float)(s.Bc - tot_lo) / (float)(tot_hi - tot_lo)));
+      reach = max(span / 4, 1u);
+    }
+    // level k of this pass, in (lo, hi), not decreasing in k
+    auto level = [&](int k) -> uint32_t {
+      if (even) return min(lo + step * (k + 1), hi - 1);
+      const int64_t b = guess + spread(k, reach) + (k - kCand / 2);
+      return (uint32_t)max((int64_t)lo + 1, min(b, (int64_t)hi - 1));
+    };
+    float lam[kCand];
+    uint32_t acc[kCand];
+#pragma unroll
+    for (int k = 0; k < kCand; ++k) {
+      lam[k] = __uint_as_float(level(k));
+      acc[k] = 0;
+    }
+    uint32_t seen = 0;
+    for (int64_t i = tid; i < cnt; i += kThreads) {
+      const float sh = shat(i);
+#pragma unroll
+      for (int k = 0; k < kCand; ++k) acc[k] += rank_bits(lam[k], sh, fmin_r, fmax_r);
+      ++seen;
+    }
+#pragma unroll
+    for (int k = 0; k < kCand; ++k) {
+      const uint32_t v = acc[k] - seen * kRankBias;   // modulo 2^32: the sum itself
+      unsigned long long w;
+      if (wide) {
+        w = v;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      } else {
+        w = __reduce_add_sync(0xffffffffu, v);
+      }
+      if (lane == 0) sm.wsum[k][warp] = w;
+    }
+    __syncthreads();
+    if (tid < kCand * C) {   // thread (candidate, peer)
+      const int k = tid % kCand, c = tid / kCand;
+      unsigned long long w = 0;
+#pragma unroll
+      for (int i = 0; i < kWarps; ++i) w += sm.wsum[k][i];
+      *cluster.map_shared_rank(&sm.tot[pass & 1][rank][k], c) = (long long)w;
+    }
+    cluster.sync();   // also orders this pass's reads of wsum before the next pass's writes
+    long long total = 0;
+    if (lane < kCand)
+      for (int c = 0; c < C; ++c) total += sm.tot[pass & 1][c][lane];
+    // the levels do not decrease, so those that fit come first
+    const int m = __popc(__ballot_sync(0xffffffffu, lane < kCand && total <= s.Bc));
+    const uint32_t below = m > 0 ? level(m - 1) : lo, above = m < kCand ? level(m) : hi;
+    if (m > 0) tot_lo = __shfl_sync(0xffffffffu, total, m - 1);
+    if (m < kCand) tot_hi = __shfl_sync(0xffffffffu, total, m);
+    lo = below;
+    hi = above;
   }
 
-  int64_t acc = 0;
-  for (int64_t t = tid; t < n; t += blockDim.x) {
-    const int r = mode_fixed >= 0 ? mode_fixed
-                                  : rank_of(lam, shat_of(sl ? sl[t] : 0.f, mn, den, flat), s.r_min, s.r_max);
-    rk[t] = (uint8_t)r;
-    acc += r;
-  }
-  const int64_t sum = block_sum(acc, red);
-  if (tid == 0 && realized) realized[bl] = sum;
+  const float lam = __uint_as_float(lo);
+  for (int64_t i = tid; i < cnt; i += kThreads)
+    rk[t0 + i] = (uint8_t)(rank_bits(lam, shat(i), fmin_r, fmax_r) - kRankBias);
+  if (rank == 0 && tid == 0 && realized) realized[bl] = tot_lo;
 }
 
 }  // namespace
 
 int launch_allocate(const Shape& s, const float* sal, uint8_t* ranks, int64_t* realized,
-                    int32_t* dev_status, cudaStream_t st) {
-  allocate_kernel<<<s.B * s.L, kThreads, 0, st>>>(s.mode == VARRATE_UNIFORM ? nullptr : sal, ranks,
-                                                  realized, dev_status, s);
-  return 1;
+                    int32_t* dev_status, int num_sms, cudaStream_t st) {
+  // One CTA for every 2048 tokens or so (eight per thread), at most 8 to a pair, and no more than two CTAs
+  // an SM over all pairs: a second wave would double the time.
+  const int64_t pairs = (int64_t)s.B * s.L;
+  int C = 1;
+  while (C < kMaxCluster && (int64_t)C * 2048 < s.n_coded && C * pairs <= num_sms) C *= 2;
+  const int64_t share = (s.n_coded + C - 1) / C;
+  const int64_t cached = share < kMaxCached ? share : kMaxCached;
+  const size_t smem = (size_t)cached * sizeof(float);
+  if (smem > 32768 &&
+      cudaFuncSetAttribute(allocate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(kMaxCached * sizeof(float))) != cudaSuccess)
+    return -1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(pairs * C));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = C; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  const float* sp = s.mode == VARRATE_UNIFORM ? nullptr : sal;
+  return cudaLaunchKernelEx(&cfg, allocate_kernel, sp, ranks, realized, dev_status, s, share, cached) == cudaSuccess
+             ? 1 : -1;
 }
 
 }  // namespace vr

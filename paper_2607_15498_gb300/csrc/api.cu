@@ -188,7 +188,8 @@ varrate_status varrate_allocate(const varrate_config* cfg, const float* sal, uin
     return VARRATE_ERR_ARG;
   if (!aligned16({sal, ranks, realized_sum, dev_status})) return VARRATE_ERR_ARG;
   const Shape s = make_shape(cfg, cap_elems(cfg));
-  vr::launch_allocate(s, sal, ranks, realized_sum, dev_status, (cudaStream_t)stream);
+  if (vr::launch_allocate(s, sal, ranks, realized_sum, dev_status, num_sms(), (cudaStream_t)stream) < 0)
+    return VARRATE_ERR_CUDA;
   return launched();
 }
 
@@ -231,7 +232,7 @@ varrate_status varrate_encode(const varrate_config* cfg, const void* q_win, cons
       : reinterpret_cast<int64_t*>(w + sal_ws + align256((size_t)s.B * s.L * s.n_coded * sizeof(float)));
   if (cfg->mode == VARRATE_SALIENCE && vr::launch_salience(s, q_win, k, sal, w, dev_status, sms, cs) < 0)
     return VARRATE_ERR_CUDA;
-  vr::launch_allocate(s, sal, out->ranks, realized, dev_status, cs);
+  if (vr::launch_allocate(s, sal, out->ranks, realized, dev_status, sms, cs) < 0) return VARRATE_ERR_CUDA;
   if (vr::launch_pack(s, k, v, basis_k, basis_v, *out, dev_status, sms, cs) < 0) return VARRATE_ERR_CUDA;
   return launched();
 }

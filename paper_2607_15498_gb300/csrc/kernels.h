@@ -31,7 +31,7 @@ int launch_salience_tc(const Shape& s, const void* q_win, const void* k, float* 
 
 // ---- step 2: allocation
 int launch_allocate(const Shape& s, const float* sal, uint8_t* ranks, int64_t* realized,
-                    int32_t* dev_status, cudaStream_t st);
+                    int32_t* dev_status, int num_sms, cudaStream_t st);
 
 // ---- step 3: tables + projection
 // Host-side checks of what launch_pack builds before its first launch (bf16: the TMA tensor maps
