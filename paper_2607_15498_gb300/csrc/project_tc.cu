@@ -90,6 +90,13 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constant_
   const uint32_t tmem = sm.tmem_base;
 
   __nv_bfloat16* out = coef + ((bl * s.G + g) * 2 + kv) * s.cap;
+  // zero the padding of each bucket of this stream: in row j they are the end of the last 8-slot group
+  for (int i = blockIdx.x * blockDim.x + tid; i < (kMaxR + 1) * kHeadDim; i += gridDim.x * blockDim.x) {
+    const int r = i / kHeadDim, j = i % kHeadDim;
+    if (r < s.r_min || j >= r) continue;
+    for (int p = bucket_count[bl * (kMaxR + 1) + r]; p < sm.n8[r]; ++p)
+      out[sm.base[r] + coef_offset(r, sm.n8[r], p, j)] = __float2bfloat16_rn(0.f);
+  }
   const int64_t t_begin = blockIdx.x * chunk;
   const int64_t t_end = min(s.N, t_begin + chunk);
   const int n_tiles = (int)((t_end - t_begin + TM - 1) / TM);
