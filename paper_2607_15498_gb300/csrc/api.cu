@@ -296,7 +296,7 @@ varrate_status varrate_quantize(const varrate_config* cfg, const varrate_packed*
   if (!aligned16({dev_status})) return VARRATE_ERR_ARG;
   const Shape s = make_shape(cfg, in->cap_elems);
   if ((int64_t)s.B * s.L > 65535) return VARRATE_ERR_UNSUPPORTED;   // grid.y of the quantize kernel
-  vr::launch_quantize(s, *in, *out, dev_status, (cudaStream_t)stream);
+  vr::launch_quantize(s, *in, *out, dev_status, num_sms(), (cudaStream_t)stream);
   return launched();
 }
 

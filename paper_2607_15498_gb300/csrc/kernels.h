@@ -81,7 +81,7 @@ int launch_decode_window(const Shape& s, const varrate_packed& c, const void* ba
 
 // ---- quantized coefficients (quant.cu)
 int launch_quantize(const Shape& s, const varrate_packed& in, const varrate_qpacked& out,
-                    int32_t* dev_status, cudaStream_t st);
+                    int32_t* dev_status, int num_sms, cudaStream_t st);
 // Fused decode on a group-quantized cache (decode_q.cu): the bf16 kernel's work split with the
 // codes dequantized in each warp's ring. Workspace: that of the bf16 fused decode (header, then
 // the partials). Shapes it does not take run the general kernels on x^ (launch_decode_q,
