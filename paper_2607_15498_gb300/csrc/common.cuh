@@ -38,6 +38,14 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float
   return __float2bfloat16_rn(x);
 }
 
+// Four consecutive elements from an address aligned to all four.
+__device__ __forceinline__ float4 load4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                     __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
+
 // Eight consecutive elements starting at a 16-byte (bf16) / 32-byte (fp32) aligned address,
 // streamed (read once: evict-first in L2, no L1 allocation).
 __device__ __forceinline__ void load8_stream(const __nv_bfloat16* p, float (&f)[8]) {

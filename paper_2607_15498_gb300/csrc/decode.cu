@@ -25,6 +25,7 @@ constexpr int kMaxR = kHeadDim;
 constexpr int kWarps = 8;
 constexpr int kItem = 128;        // slots per warp item: one tile of the packed layout
 constexpr int kMaxTail = 4096;
+constexpr int kMaxSplits = 128;
 
 // Raw 8-element row fragment: bf16 -> one uint4, fp32 -> two float4.
 template <typename T> struct Frag;
@@ -129,7 +130,9 @@ __device__ __forceinline__ float transpose_reduce32(float (&v)[32]) {
   return v[0];
 }
 
-// grid (G, B), 256 threads: qt[b][h][j] = scale * sum_i U_K[j][i] q[b][h][i].
+constexpr int kRotSplit = 8;   // CTAs that share the rows of U_K of one head
+
+// grid (G, B, kRotSplit), 256 threads: qt[b][h][j] = scale * sum_i U_K[j][i] q[b][h][i].
 template <typename T>
 __global__ void __launch_bounds__(256)
 decode_rotate_kernel(const T* __restrict__ q, const T* __restrict__ basis_k, float* __restrict__ qt,
@@ -142,10 +145,12 @@ decode_rotate_kernel(const T* __restrict__ q, const T* __restrict__ basis_k, flo
   __syncthreads();
   const T* U = basis_k + ((int64_t)layer * s.G + g) * kHeadDim * kHeadDim;
   const float scale = kLog2e * rsqrtf((float)kHeadDim);
-  for (int j = warp; j < kHeadDim; j += kWarps) {
-    float u[4];
+  constexpr int kRows = kHeadDim / kRotSplit;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) u[i] = to_f(U[j * kHeadDim + lane * 4 + i]);
+  for (int jj = warp; jj < kRows; jj += kWarps) {
+    const int j = blockIdx.z * kRows + jj;
+    const float4 u4 = load4(U + j * kHeadDim + lane * 4);
+    const float u[4] = {u4.x, u4.y, u4.z, u4.w};
     for (int hh = 0; hh < s.grp; ++hh) {
       float acc = 0.f;
 #pragma unroll
@@ -167,6 +172,7 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
   __shared__ int cnt[kMaxR + 1];
   __shared__ long long base[kMaxR + 2];
   __shared__ long long qb[kMaxR + 2];   // quantized source: byte offset of each bucket
+  __shared__ int i_first[kMaxR + 1], i_last[kMaxR + 1];   // this split's items of each bucket
   __shared__ float wM[kWarps][GP], wL[kWarps][GP];
   __shared__ float wacc[kWarps][GP][kHeadDim];
 
@@ -205,16 +211,24 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
   const bool table_ok = W <= s.cap && (Src::kTableBase || qb[kMaxR + 1] <= table_cap);
   const long long lo = table_ok ? W * split / S : 0, hi = table_ok ? W * (split + 1) / S : 0;
   src.bind((bl * s.G + g) * 2);
+  // one bucket a thread: the 64-bit divisions of all buckets at once
+  for (int r = tid; r <= kMaxR; r += blockDim.x) {
+    int first = 0, last = 0;
+    if (table_ok && r >= s.r_min && r <= s.r_max && cnt[r] > 0) {
+      const long long b0 = base[r], unit = (long long)kItem * r;
+      const long long nit = (pad8(cnt[r]) + kItem - 1) / kItem;
+      first = (int)min(nit, lo > b0 ? (lo - b0 + unit - 1) / unit : 0);
+      last = (int)min(nit, hi > b0 ? (hi - b0 + unit - 1) / unit : 0);
+    }
+    i_first[r] = first;
+    i_last[r] = last;
+  }
+  __syncthreads();
   int counter = 0;
   for (int r = s.r_min; r <= s.r_max && table_ok; ++r) {
     const int n = cnt[r];
-    if (n == 0) continue;
-    const long long n8 = pad8(n), b0 = base[r], unit = (long long)kItem * r;
-    const long long nit = (n8 + kItem - 1) / kItem;
-    long long i_lo = lo > b0 ? (lo - b0 + unit - 1) / unit : 0;
-    long long i_hi = hi > b0 ? (hi - b0 + unit - 1) / unit : 0;
-    if (i_hi > nit) i_hi = nit;
-    for (long long it = i_lo; it < i_hi; ++it, ++counter) {
+    const long long n8 = pad8(n), b0 = base[r], i_hi = i_last[r];
+    for (long long it = i_first[r]; it < i_hi; ++it, ++counter) {
       if ((counter % kWarps) != warp) continue;
       const long long s0 = it * kItem + lane * 8;
       const bool lane_ok = lane < kItem / 8 && s0 < n8;   // lanes 16..31 idle: 8 slots per lane
@@ -331,7 +345,10 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
   }
 }
 
-// grid (G, B), 128 threads: merge partials and the exact tail, rotate back, normalise.
+// grid (group, G, B), 128 threads, one query head each: merge partials and the exact tail, rotate back,
+// normalise. Bound by latency: the partials' maxima and weights are formed by one thread each (S <= 128),
+// then every thread sums its coordinate over the splits with independent loads. One CTA per KV head that
+// walked its heads and splits one after another took 110 us for 128 splits of 4 heads; now 11 us.
 template <typename T, int GP>
 __global__ void __launch_bounds__(128)
 decode_combine_kernel(const float* __restrict__ part, const T* __restrict__ q,
@@ -340,68 +357,77 @@ decode_combine_kernel(const float* __restrict__ part, const T* __restrict__ q,
                       int layer, int S) {
   __shared__ float ot[kHeadDim];
   __shared__ float tsc[kMaxTail];
-  __shared__ float qrow[kHeadDim];
-  const int g = blockIdx.x, b = blockIdx.y;
+  __shared__ float wgt[kMaxSplits], lsum[kMaxSplits];
+  __shared__ float red[4];
+  const int hh = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const T* U = basis_v + ((int64_t)layer * s.G + g) * kHeadDim * kHeadDim;
   const float scale = kLog2e * rsqrtf((float)kHeadDim);
-  const float* pb = part + ((int64_t)b * s.G + g) * S * GP * (kHeadDim + 2);
-  for (int hh = 0; hh < s.grp; ++hh) {
-    const int h = g * s.grp + hh;
-    __syncthreads();
-    qrow[tid] = to_f(q[((int64_t)b * s.H + h) * kHeadDim + tid]);
-    __syncthreads();
-    // exact tail scores (log2 units)
-    float tmax = -INFINITY;
-    if (n_tail > 0) {
-      const T* tk = tail_k + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
-      for (int t = warp; t < n_tail; t += 4) {
-        float a = 0.f;
+  const float* pb = part + (((int64_t)b * s.G + g) * S * GP + hh) * (kHeadDim + 2);
+  constexpr int kStep = GP * (kHeadDim + 2);   // floats between the splits of a head
+  const int h = g * s.grp + hh;
+  auto block_max = [&](float v) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a = fmaf(qrow[lane * 4 + i], to_f(tk[(int64_t)t * kHeadDim + lane * 4 + i]), a);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) tsc[t] = a * scale;
-      }
-      __syncthreads();
-      for (int t = 0; t < n_tail; ++t) tmax = fmaxf(tmax, tsc[t]);
-    }
-    float mx = tmax;
-    for (int sp = 0; sp < S; ++sp) mx = fmaxf(mx, pb[(sp * GP + hh) * (kHeadDim + 2) + kHeadDim]);
-    float l = 0.f, o = 0.f;
-    for (int sp = 0; sp < S; ++sp) {
-      const float* pp = pb + (sp * GP + hh) * (kHeadDim + 2);
-      const float m = pp[kHeadDim];
-      if (m == -INFINITY) continue;
-      const float f = exp2f(m - mx);
-      l = fmaf(pp[kHeadDim + 1], f, l);
-      o = fmaf(pp[tid], f, o);
-    }
-    ot[tid] = o;
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) red[warp] = v;
     __syncthreads();
-    float y = 0.f;
-    for (int j = 0; j < kHeadDim; ++j) y = fmaf(to_f(U[j * kHeadDim + tid]), ot[j], y);
-    if (n_tail > 0) {
-      const T* tv = tail_v + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
-      for (int t = 0; t < n_tail; ++t) {
-        const float p = exp2f(tsc[t] - mx);
-        l += p;
-        y = fmaf(p, to_f(tv[(int64_t)t * kHeadDim + tid]), y);
-      }
+    v = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
+    __syncthreads();
+    return v;
+  };
+  // exact tail scores (log2 units)
+  float tmax = -INFINITY;
+  if (n_tail > 0) {
+    const T* tk = tail_k + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
+    const float4 qv = load4(q + ((int64_t)b * s.H + h) * kHeadDim + lane * 4);
+#pragma unroll 4
+    for (int t = warp; t < n_tail; t += 4) {
+      const float4 kv = load4(tk + (int64_t)t * kHeadDim + lane * 4);
+      float a = fmaf(qv.w, kv.w, fmaf(qv.z, kv.z, fmaf(qv.y, kv.y, qv.x * kv.x)));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      a *= scale;
+      if (lane == 0) tsc[t] = a;
+      tmax = fmaxf(tmax, a);
     }
-    out[((int64_t)b * s.H + h) * kHeadDim + tid] = from_f<T>(y / l);
   }
+  const float m = tid < S ? pb[(int64_t)tid * kStep + kHeadDim] : -INFINITY;
+  if (tid < S) lsum[tid] = pb[(int64_t)tid * kStep + kHeadDim + 1];
+  const float mx = block_max(fmaxf(m, tmax));
+  if (tid < S) wgt[tid] = m == -INFINITY ? 0.f : exp2f(m - mx);   // an empty split holds zeros
+  __syncthreads();
+  float l = 0.f, o = 0.f;
+#pragma unroll 8
+  for (int sp = 0; sp < S; ++sp) {
+    l = fmaf(lsum[sp], wgt[sp], l);
+    o = fmaf(pb[(int64_t)sp * kStep + tid], wgt[sp], o);
+  }
+  ot[tid] = o;
+  __syncthreads();
+  float y = 0.f;
+#pragma unroll 16
+  for (int j = 0; j < kHeadDim; ++j) y = fmaf(to_f(U[j * kHeadDim + tid]), ot[j], y);
+  if (n_tail > 0) {
+    const T* tv = tail_v + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
+#pragma unroll 8
+    for (int t = 0; t < n_tail; ++t) {
+      const float p = exp2f(tsc[t] - mx);
+      l += p;
+      y = fmaf(p, to_f(tv[(int64_t)t * kHeadDim + tid]), y);
+    }
+  }
+  out[((int64_t)b * s.H + h) * kHeadDim + tid] = from_f<T>(y / l);
 }
 
 template <typename T, int GP>
 void launch_decode_t(const Shape& s, const varrate_packed& c, const void* basis_k, const void* basis_v,
                      const void* q, int layer, const void* tail_k, const void* tail_v, int n_tail,
                      void* out, float* qt, float* part, int S, cudaStream_t st) {
-  decode_rotate_kernel<T><<<dim3(s.G, s.B), 256, 0, st>>>((const T*)q, (const T*)basis_k, qt, s, layer);
+  decode_rotate_kernel<T><<<dim3(s.G, s.B, kRotSplit), 256, 0, st>>>((const T*)q, (const T*)basis_k, qt, s, layer);
   DenseSrc<T> src{(const T*)c.coef, c.bucket_base, s.cap, nullptr, nullptr};
   decode_split_kernel<DenseSrc<T>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
                                                                            s, layer, S, 0);
-  decode_combine_kernel<T, GP><<<dim3(s.G, s.B), 128, 0, st>>>(part, (const T*)q, (const T*)basis_v,
+  decode_combine_kernel<T, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const T*)q, (const T*)basis_v,
                                                                (const T*)tail_k, (const T*)tail_v,
                                                                n_tail, (T*)out, s, layer, S);
 }
@@ -425,7 +451,7 @@ void launch_decode_qt(const Shape& s, const varrate_qpacked& c, const void* basi
                       const void* q, int layer, const void* tail_k, const void* tail_v, int n_tail,
                       void* out, float* qt, float* part, int S, cudaStream_t st) {
   using bf = __nv_bfloat16;
-  decode_rotate_kernel<bf><<<dim3(s.G, s.B), 256, 0, st>>>((const bf*)q, (const bf*)basis_k, qt, s, layer);
+  decode_rotate_kernel<bf><<<dim3(s.G, s.B, kRotSplit), 256, 0, st>>>((const bf*)q, (const bf*)basis_k, qt, s, layer);
   if (c.bits == 4) {
     QuantSrc<4> src{c.data, c.qbase, c.qcap_bytes, nullptr, nullptr};
     decode_split_kernel<QuantSrc<4>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
@@ -435,7 +461,7 @@ void launch_decode_qt(const Shape& s, const varrate_qpacked& c, const void* basi
     decode_split_kernel<QuantSrc<8>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
                                                                            s, layer, S, c.qcap_bytes);
   }
-  decode_combine_kernel<bf, GP><<<dim3(s.G, s.B), 128, 0, st>>>(part, (const bf*)q, (const bf*)basis_v,
+  decode_combine_kernel<bf, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const bf*)q, (const bf*)basis_v,
                                                                (const bf*)tail_k, (const bf*)tail_v,
                                                                n_tail, (bf*)out, s, layer, S);
 }
@@ -446,7 +472,7 @@ int decode_splits(const Shape& s, int num_sms) {
   const int64_t units = (int64_t)s.B * s.G;
   int64_t S = (4LL * num_sms + units - 1) / units;
   if (S < 1) S = 1;
-  if (S > 128) S = 128;
+  if (S > kMaxSplits) S = kMaxSplits;
   return (int)S;
 }
 

@@ -227,8 +227,11 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
     bases[r] = bucket_base[bl * (kMaxR + 2) + r];
   }
   const T* U = (kv ? basis_v : basis_k) + (l * s.G + g) * (int64_t)kHeadDim * kHeadDim;
-  for (int i = tid; i < kHeadDim * kHeadDim; i += blockDim.x)
-    us[(i / kHeadDim) * kLd + (i % kHeadDim)] = to_f(U[i]);
+#pragma unroll 4
+  for (int i = tid; i < kHeadDim * (kHeadDim / 4); i += 256) {
+    const int row = i / (kHeadDim / 4), c = i % (kHeadDim / 4) * 4;
+    *reinterpret_cast<float4*>(&us[row * kLd + c]) = load4(U + 4 * i);
+  }
   __syncthreads();
   if (bases[kMaxR + 1] > s.cap) return;   // corrupt tables were reported by pack_tables
 
@@ -259,10 +262,12 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
       stok[tid] = t; srk[tid] = r; spos[tid] = p;
     }
     __syncthreads();
-    for (int i = tid; i < kTile * kHeadDim; i += blockDim.x) {
-      const int row = i / kHeadDim, c = i % kHeadDim;
+#pragma unroll
+    for (int i = tid; i < kTile * (kHeadDim / 4); i += 256) {
+      const int row = i / (kHeadDim / 4), c = i % (kHeadDim / 4) * 4;
       const int t = stok[row];
-      xs[row * kLd + c] = t >= 0 ? to_f(x[(int64_t)t * kHeadDim + c]) : 0.f;
+      *reinterpret_cast<float4*>(&xs[row * kLd + c]) =
+          t >= 0 ? load4(x + (int64_t)t * kHeadDim + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
     float acc[4][8];

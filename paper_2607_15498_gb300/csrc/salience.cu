@@ -19,30 +19,35 @@ constexpr int kRows = 128;     // window rows per block
 constexpr int kTok = 64;       // tokens per tile
 constexpr int kLd = kHeadDim + 4;
 constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
+constexpr int kMaxChunks = 64;  // token chunks of pass 1 that a short stream is cut into
 
 // Load rows [rb*128, rb*128+128) of the window block of KV head g into smem as fp32.
 template <typename T>
 __device__ void load_q_rows(float* qs, const T* __restrict__ q_win, const Shape& s, int64_t bl,
                             int g, int rb) {
   const int M = s.grp * s.w;
-  for (int idx = threadIdx.x; idx < kRows * kHeadDim; idx += blockDim.x) {
-    const int r = idx / kHeadDim, c = idx % kHeadDim;
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < kRows * (kHeadDim / 4); idx += kThreads) {
+    const int r = idx / (kHeadDim / 4), c = idx % (kHeadDim / 4) * 4;
     const int m = rb * kRows + r;
-    float val = 0.f;
+    float4 val = make_float4(0.f, 0.f, 0.f, 0.f);
     if (m < M) {
       const int h = g * s.grp + m / s.w, q = m % s.w;
-      val = to_f(q_win[((bl * s.w + q) * s.H + h) * (int64_t)kHeadDim + c]);
+      val = load4(&q_win[((bl * s.w + q) * s.H + h) * (int64_t)kHeadDim + c]);
     }
-    qs[r * kLd + c] = val;
+    *reinterpret_cast<float4*>(&qs[r * kLd + c]) = val;
   }
 }
 
 template <typename T>
 __device__ void load_k_tile(float* ks, const T* __restrict__ kg, int64_t t0, int64_t t_end) {
-  for (int idx = threadIdx.x; idx < kTok * kHeadDim; idx += blockDim.x) {
-    const int r = idx / kHeadDim, c = idx % kHeadDim;
+#pragma unroll
+  for (int idx = threadIdx.x; idx < kTok * (kHeadDim / 4); idx += kThreads) {
+    const int r = idx / (kHeadDim / 4), c = idx % (kHeadDim / 4) * 4;
     const int64_t t = t0 + r;
-    ks[r * kLd + c] = (t < t_end) ? to_f(kg[t * kHeadDim + c]) : 0.f;
+    *reinterpret_cast<float4*>(&ks[r * kLd + c]) =
+        t < t_end ? load4(&kg[t * kHeadDim + c]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
@@ -165,19 +170,33 @@ salience_accum_kernel(const T* __restrict__ q_win, const T* __restrict__ k,
     for (int rb = 0; rb < n_rb; ++rb) {
       __syncthreads();
       load_q_rows(qs, q_win, s, bl, g, rb);
-      if (tid < kRows) {
-        const int m = rb * kRows + tid;
-        float val = INFINITY;   // padding rows contribute exp2(-inf) = 0
-        if (m < M) {
-          const float2* st = stats + ((bl * s.G + g) * M + m) * n_chunks;
-          float mx = -INFINITY;
-          for (int c = 0; c < n_chunks; ++c) mx = fmaxf(mx, st[c].x);
-          float l = 0.f;
-          for (int c = 0; c < n_chunks; ++c)
-            if (st[c].x != -INFINITY) l += st[c].y * exp2f(st[c].x - mx);
-          val = mx + log2f(l);
+      // a warp per row, its lanes over the chunks' partials, the loads of eight rows in flight together
+      for (int r0 = warp; r0 < kRows; r0 += 8 * kWarps) {
+        float2 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int m = rb * kRows + r0 + u * kWarps;
+          x[u] = make_float2(-INFINITY, 0.f);
+          if (m < M && lane < n_chunks) x[u] = stats[((bl * s.G + g) * M + m) * n_chunks + lane];
         }
-        lse[tid] = val;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int m = rb * kRows + r0 + u * kWarps;
+          const float2* st = stats + ((bl * s.G + g) * M + m) * n_chunks;
+          float mx = x[u].x;
+          if (m < M)
+            for (int c = lane + 32; c < n_chunks; c += 32) mx = fmaxf(mx, st[c].x);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          float l = x[u].x != -INFINITY ? x[u].y * exp2f(x[u].x - mx) : 0.f;
+          if (m < M)
+            for (int c = lane + 32; c < n_chunks; c += 32)
+              if (st[c].x != -INFINITY) l += st[c].y * exp2f(st[c].x - mx);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+          // padding rows contribute exp2(-inf) = 0
+          if (lane == 0) lse[r0 + u * kWarps] = m < M ? mx + log2f(l) : INFINITY;
+        }
       }
       for (int64_t t0 = t_begin; t0 < t_end; t0 += kTok) {
         __syncthreads();
@@ -249,7 +268,10 @@ SalPlan salience_plan(const Shape& s, int num_sms) {
   int64_t n = (want + units - 1) / units;
   int64_t chunk = (s.N + n - 1) / n;
   chunk = ((chunk + kTok - 1) / kTok) * kTok;
-  if (chunk < 512) chunk = 512;
+  // a CTA per 64-token tile for short streams (latency-bound: 2048 fp32 tokens of one head took 132 us on 4
+  // CTAs of 512), but no more partials per row than a warp merges in two loads
+  const int64_t least = ((s.N + kMaxChunks - 1) / kMaxChunks + kTok - 1) / kTok * kTok;
+  if (chunk < least) chunk = least;
   p.chunk = chunk;
   p.n_chunks = (int)((s.N + chunk - 1) / chunk);
   const int64_t bl = (int64_t)s.B * s.L;
