@@ -5,14 +5,14 @@
 // o = U_V^T (sum_t 2^(score_t - m) c^V_t[:r_t]) / sum_t 2^(score_t - m)   (+ exact tail tokens).
 //
 // decode_rotate  q~ for every head (fp32 workspace).
-// decode_split   grid (S, G, B), 8 warps. The coded elements of the (b, l, g) stream are split
-//                into S contiguous cost ranges; a warp item is one 128-slot tile of a rank bucket
-//                (8 slots per lane on 16 lanes, one 16-byte load per coefficient row, addressed
-//                through the packed layout's coef_offset). Scores: 8 slots x GP heads per lane, no cross-lane work. Value rows: every
-//                lane forms GP x RG partial sums (GP heads x RG rows, GP * RG = 32) and one
-//                31-shuffle transpose-reduction leaves lane i with the full sum of pair i, so each
-//                lane owns 128 / RG output coordinates. Online softmax per warp; warps then merge
-//                in shared memory and write one (max, sum, o~[128]) partial per head.
+// decode_split   grid (S x head quads, G, B), 8 warps. The coded elements of the (b, l, g) stream are split
+//                into S contiguous cost ranges; a warp item is 32 slots of a rank bucket. Lane (phase,
+//                sg) holds 8 slots (16-byte loads, addressed through the packed layout) of the rows
+//                j = phase, phase + 8, ...: scores are its partial sums added over the phases by
+//                shuffles; on the value side each lane keeps the partial outputs of its rows over its
+//                slots, added over the four slot groups once at the end, so no item needs more
+//                cross-lane work than its scores. Online softmax per warp; warps then merge in shared
+//                memory and write one (max, sum, o~[128]) partial per head.
 // decode_combine merges the S partials (and the exact tail), rotates back with U_V^T, writes out.
 #include "common.cuh"
 #include "kernels.h"
@@ -23,7 +23,8 @@ namespace {
 
 constexpr int kMaxR = kHeadDim;
 constexpr int kWarps = 8;
-constexpr int kItem = 128;        // slots per warp item: one tile of the packed layout
+constexpr int kItem = 32;         // slots per warp item: a quarter of a tile of the packed layout
+constexpr int kPhases = 8;        // lanes that share the rows of a slot group
 constexpr int kMaxTail = 4096;
 constexpr int kMaxSplits = 128;
 
@@ -78,7 +79,9 @@ template <int BITS> struct QFrag {
 
 // Where the split kernel reads coefficient rows from. DenseSrc: the packed cache of `T` elements
 // (bucket offsets from its table). QuantSrc: the quantized cache (bucket element offsets rebuilt
-// from the counts, byte offsets from qbase).
+// from the counts, byte offsets from qbase). bind() selects a stream pair, tile() the tile that holds
+// bucket slot s0 (8 slots from there on), row() loads coefficient row j of those slots: `rot` is the
+// position of their group in that row, (group + j) mod (tl / 8).
 template <typename T> struct DenseSrc {
   using F = Frag<T>;
   static constexpr bool kTableBase = true;
@@ -86,12 +89,15 @@ template <typename T> struct DenseSrc {
   const int64_t* bucket_base;
   int64_t stride;   // elements per stream
   const T* cK;
-  const T* cV;
-  __device__ __forceinline__ void bind(int64_t stream0) { cK = coef + stream0 * stride; cV = cK + stride; }
-  __device__ __forceinline__ void load(F& f, int kv, int r, long long b0, long long qb0, long long n8,
-                                       long long s0, int j) const {
-    (void)qb0;
-    f.load((kv ? cV : cK) + b0 + coef_offset(r, n8, s0, j));
+  const T* tK;
+  int tl;
+  __device__ __forceinline__ void bind(int64_t stream0) { cK = coef + stream0 * stride; }
+  __device__ __forceinline__ void tile(int r, long long b0, long long, int tl_, long long s0) {
+    tK = cK + b0 + (s0 >> 7) * 128 * r;
+    tl = tl_;
+  }
+  __device__ __forceinline__ void row(F& f, int kv, int j, int rot) const {
+    f.load(tK + (kv ? stride : 0) + j * tl + rot * 8);
   }
 };
 template <int BITS> struct QuantSrc {
@@ -101,34 +107,18 @@ template <int BITS> struct QuantSrc {
   const int64_t* qbase;
   int64_t stride;   // bytes per stream
   const uint8_t* qK;
-  const uint8_t* qV;
-  __device__ __forceinline__ void bind(int64_t stream0) { qK = data + stream0 * stride; qV = qK + stride; }
-  __device__ __forceinline__ void load(F& f, int kv, int r, long long b0, long long qb0, long long n8,
-                                       long long s0, int j) const {
-    (void)b0;
-    const long long it = s0 >> 7;
-    const int p0 = (int)(s0 & 127);
-    const int tl = (int)min(128ll, n8 - (it << 7));
-    f.load((kv ? qV : qK) + qb0 + it * r * qrow_bytes(128, BITS) + (long long)j * qrow_bytes(tl, BITS), p0, tl);
+  const uint8_t* tK;
+  int tl, p0;
+  __device__ __forceinline__ void bind(int64_t stream0) { qK = data + stream0 * stride; }
+  __device__ __forceinline__ void tile(int r, long long, long long qb0, int tl_, long long s0) {
+    tK = qK + qb0 + (s0 >> 7) * r * qrow_bytes(128, BITS);
+    tl = tl_;
+    p0 = (int)(s0 & 127);
+  }
+  __device__ __forceinline__ void row(F& f, int kv, int j, int) const {
+    f.load(tK + (kv ? stride : 0) + j * qrow_bytes(tl, BITS), p0, tl);
   }
 };
-
-// v[32] holds partials of 32 (head, row) pairs; afterwards v[0] of lane i is the warp-wide sum of
-// pair i (each halving step keeps the half selected by the lane's bit and trades the other).
-__device__ __forceinline__ float transpose_reduce32(float (&v)[32]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int n = 16; n >= 1; n >>= 1) {
-    const bool upper = lane & n;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const float send = upper ? v[i] : v[i + n];
-      const float keep = upper ? v[i + n] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, n);
-    }
-  }
-  return v[0];
-}
 
 constexpr int kRotSplit = 8;   // CTAs that share the rows of U_K of one head
 
@@ -162,21 +152,28 @@ decode_rotate_kernel(const T* __restrict__ q, const T* __restrict__ basis_k, flo
   }
 }
 
-template <class Src, int GP>
-__global__ void __launch_bounds__(256, (GP == 4 || GP == 2) ? 2 : 1)
+// GH heads of the group per CTA (4, or the whole group when it is smaller); blockIdx.x = split * quads + quad.
+// Bound by instructions and load latency. Whole 128-slot tiles per warp (8 slots on each of 16 lanes, value rows
+// reduced over the warp eight at a time) left a 128-row tile to one warp for 80 us and more. Per layer
+// call with rotation and combine, before / now: fp32, 8 heads x 8000 tokens x 2 sequences 280 / 92 us;
+// bf16, 8 heads x 32768 with 400 tail tokens 347 / 114 us, 4 heads of group 7 with wide ranks 662 / 143
+// us; 4-bit, 300 tail tokens 318 / 124 us.
+template <class Src, int GP, int GH>
+__global__ void __launch_bounds__(256, 1)
 decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const float* __restrict__ qt,
                     float* __restrict__ part, Shape s, int layer, int S, long long table_cap) {
-  constexpr int RG = 32 / GP;             // value rows per transpose-reduction
-  constexpr int NACC = kHeadDim / RG;     // output coordinates owned per lane
-  __shared__ __align__(16) float q_s[kHeadDim][GP];
+  constexpr int kRowsPer = kHeadDim / kPhases;   // rows a lane owns
+  constexpr int kBatch = 4;                      // rows whose loads are in flight together
+  __shared__ __align__(16) float q_s[kHeadDim][GH];
   __shared__ int cnt[kMaxR + 1];
   __shared__ long long base[kMaxR + 2];
   __shared__ long long qb[kMaxR + 2];   // quantized source: byte offset of each bucket
   __shared__ int i_first[kMaxR + 1], i_last[kMaxR + 1];   // this split's items of each bucket
-  __shared__ float wM[kWarps][GP], wL[kWarps][GP];
-  __shared__ float wacc[kWarps][GP][kHeadDim];
+  __shared__ float wM[kWarps][GH], wL[kWarps][GH];
+  __shared__ float wacc[kWarps][GH][kHeadDim];
 
-  const int split = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
+  constexpr int kQuads = GP / GH;
+  const int split = blockIdx.x / kQuads, h0 = blockIdx.x % kQuads * GH, g = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t bl = (int64_t)b * s.L + layer;
   for (int r = tid; r <= kMaxR + 1; r += blockDim.x) {
@@ -195,17 +192,11 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
       base[kMaxR + 1] = acc;
     }
   }
-  for (int i = tid; i < kHeadDim * GP; i += blockDim.x) {
-    const int j = i / GP, hh = i % GP;
-    q_s[j][hh] = hh < s.grp ? qt[((int64_t)b * s.H + g * s.grp + hh) * kHeadDim + j] : 0.f;
+  for (int i = tid; i < kHeadDim * GH; i += blockDim.x) {
+    const int j = i / GH, hh = h0 + i % GH;
+    q_s[j][i % GH] = hh < s.grp ? qt[((int64_t)b * s.H + g * s.grp + hh) * kHeadDim + j] : 0.f;
   }
   __syncthreads();
-
-  float M[GP], Ls[GP], acc[NACC];
-#pragma unroll
-  for (int h = 0; h < GP; ++h) { M[h] = -INFINITY; Ls[h] = 0.f; }
-#pragma unroll
-  for (int a = 0; a < NACC; ++a) acc[a] = 0.f;
 
   const long long W = base[kMaxR + 1];
   const bool table_ok = W <= s.cap && (Src::kTableBase || qb[kMaxR + 1] <= table_cap);
@@ -224,109 +215,127 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
     i_last[r] = last;
   }
   __syncthreads();
-  int counter = 0;
-  for (int r = s.r_min; r <= s.r_max && table_ok; ++r) {
-    const int n = cnt[r];
-    const long long n8 = pad8(n), b0 = base[r], i_hi = i_last[r];
-    for (long long it = i_first[r]; it < i_hi; ++it, ++counter) {
-      if ((counter % kWarps) != warp) continue;
-      const long long s0 = it * kItem + lane * 8;
-      const bool lane_ok = lane < kItem / 8 && s0 < n8;   // lanes 16..31 idle: 8 slots per lane
-      const long long qb0 = Src::kTableBase ? 0 : qb[r];
 
-      // scores for 8 slots x GP heads
-      float sc[GP][8];
+  const int sg = lane & 3, phase = lane >> 2;
+  float M[GH], Ls[GH], acc[kRowsPer][GH];
 #pragma unroll
-      for (int h = 0; h < GP; ++h)
+  for (int h = 0; h < GH; ++h) { M[h] = -INFINITY; Ls[h] = 0.f; }
+#pragma unroll
+  for (int a = 0; a < kRowsPer; ++a)
+#pragma unroll
+    for (int h = 0; h < GH; ++h) acc[a][h] = 0.f;
+
+  int counter = 0;   // items of the split before the bucket: the warps take them in turn
+  for (int r = s.r_min; r <= s.r_max && table_ok; ++r) {
+    const int i0 = i_first[r], i_hi = i_last[r];
+    if (i0 >= i_hi) continue;
+    const int turn = (warp - counter) & (kWarps - 1);
+    counter += i_hi - i0;
+    for (int it = i0 + turn; it < i_hi; it += kWarps) {
+      const int n = cnt[r];
+      const long long s0 = (long long)it * kItem + sg * 8, n8 = pad8(n);
+      const bool on = s0 < n8;                          // the last item of a bucket may hold fewer groups
+      const int tl = (int)min(128ll, n8 - ((long long)it * kItem & ~127ll)), ng = tl >> 3;
+      src.tile(r, base[r], Src::kTableBase ? 0 : qb[r], tl, s0);
+      const int rot0 = ((int)(s0 & 127) / 8 + phase) % ng, rstep = kPhases % ng;
+
+      // scores of 8 slots x GH heads over this lane's rows, then over the phases
+      float sc[GH][8];
+#pragma unroll
+      for (int h = 0; h < GH; ++h)
 #pragma unroll
         for (int i = 0; i < 8; ++i) sc[h][i] = 0.f;
-      for (int j0 = 0; j0 < r; j0 += 8) {
-        typename Src::F f[8];
+      int rot = rot0;
+      for (int j0 = phase; j0 < r; j0 += kPhases * kBatch) {
+        typename Src::F f[kBatch];
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          if (lane_ok && j0 + jj < r) src.load(f[jj], 0, r, b0, qb0, n8, s0, j0 + jj);
-          else f[jj].zero();
+        for (int jj = 0; jj < kBatch; ++jj) {
+          f[jj].zero();
+          if (on && j0 + jj * kPhases < r) src.row(f[jj], 0, j0 + jj * kPhases, rot);
+          rot += rstep;
+          if (rot >= ng) rot -= ng;
         }
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-          if (j0 + jj < r) {
-            float qv[GP];
+        for (int jj = 0; jj < kBatch; ++jj) {
+          const int j = min(j0 + jj * kPhases, kHeadDim - 1);   // a row past r was loaded as zeros
 #pragma unroll
-            for (int h = 0; h < GP; ++h) qv[h] = q_s[j0 + jj][h];
+          for (int h = 0; h < GH; ++h) {
+            const float qv = j0 + jj * kPhases < r ? q_s[j][h] : 0.f;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float kx = f[jj].get(i);
-#pragma unroll
-              for (int h = 0; h < GP; ++h) sc[h][i] = fmaf(qv[h], kx, sc[h][i]);
-            }
+            for (int i = 0; i < 8; ++i) sc[h][i] = fmaf(qv, f[jj].get(i), sc[h][i]);
           }
         }
       }
+      __syncwarp();
       // online softmax over this item
-      float corr[GP];
 #pragma unroll
-      for (int h = 0; h < GP; ++h) {
+      for (int h = 0; h < GH; ++h) {
         float mloc = -INFINITY;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          if (!(lane_ok && s0 + i < n)) sc[h][i] = -INFINITY;
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) sc[h][i] += __shfl_xor_sync(0xffffffffu, sc[h][i], o);
+          if (s0 + i >= n) sc[h][i] = -INFINITY;
           mloc = fmaxf(mloc, sc[h][i]);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, o));
+        mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 1));
+        mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 2));
         const float nm = fmaxf(M[h], mloc);
-        corr[h] = exp2f(M[h] - nm);
+        const float corr = exp2f(M[h] - nm);
         float sum = 0.f;
 #pragma unroll
         for (int i = 0; i < 8; ++i) { sc[h][i] = exp2f(sc[h][i] - nm); sum += sc[h][i]; }
-        Ls[h] = Ls[h] * corr[h] + sum;
+        Ls[h] = Ls[h] * corr + sum;
         M[h] = nm;
+#pragma unroll
+        for (int a = 0; a < kRowsPer; ++a) acc[a][h] *= corr;
       }
-      float my_corr = corr[0];
-#pragma unroll
-      for (int h = 1; h < GP; ++h) if (lane / RG == h) my_corr = corr[h];
-#pragma unroll
-      for (int a = 0; a < NACC; ++a) acc[a] *= my_corr;
 
-      // weighted value rows, RG rows at a time
+      // weighted value rows
+      rot = rot0;
 #pragma unroll
-      for (int gi = 0; gi < NACC; ++gi) {
-        if (gi * RG >= r) break;
-        typename Src::F f[RG];
+      for (int a0 = 0; a0 < kRowsPer; a0 += kBatch) {
+        if (a0 * kPhases >= r) break;                   // warp-uniform
+        typename Src::F f[kBatch];
 #pragma unroll
-        for (int jj = 0; jj < RG; ++jj) {
-          if (lane_ok && gi * RG + jj < r) src.load(f[jj], 1, r, b0, qb0, n8, s0, gi * RG + jj);
-          else f[jj].zero();
+        for (int jj = 0; jj < kBatch; ++jj) {
+          const int j = phase + (a0 + jj) * kPhases;
+          f[jj].zero();
+          if (on && j < r) src.row(f[jj], 1, j, rot);
+          rot += rstep;
+          if (rot >= ng) rot -= ng;
         }
-        float pv[32];
 #pragma unroll
-        for (int jj = 0; jj < RG; ++jj) {
+        for (int jj = 0; jj < kBatch; ++jj)
 #pragma unroll
-          for (int h = 0; h < GP; ++h) {
+          for (int h = 0; h < GH; ++h) {
             float a2 = 0.f;
 #pragma unroll
             for (int i = 0; i < 8; ++i) a2 = fmaf(sc[h][i], f[jj].get(i), a2);
-            pv[h * RG + jj] = a2;
+            acc[a0 + jj][h] += a2;
           }
-        }
-        acc[gi] += transpose_reduce32(pv);
       }
     }
   }
 
-  // merge the warps of this CTA
+  // merge the slot groups of each warp, then the warps of this CTA
 #pragma unroll
-  for (int h = 0; h < GP; ++h) {
+  for (int h = 0; h < GH; ++h) {
     float l = Ls[h];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
     if (lane == 0) { wM[warp][h] = M[h]; wL[warp][h] = l; }
-  }
 #pragma unroll
-  for (int a = 0; a < NACC; ++a) wacc[warp][lane / RG][a * RG + (lane % RG)] = acc[a];
+    for (int a = 0; a < kRowsPer; ++a) {
+      float v = acc[a][h];
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (sg == 0) wacc[warp][h][phase + a * kPhases] = v;
+    }
+  }
   __syncthreads();
-  float* out = part + (((int64_t)b * s.G + g) * S + split) * GP * (kHeadDim + 2);
-  for (int i = tid; i < GP * kHeadDim; i += blockDim.x) {
+  float* out = part + ((((int64_t)b * s.G + g) * S + split) * GP + h0) * (kHeadDim + 2);
+  for (int i = tid; i < GH * kHeadDim; i += blockDim.x) {
     const int h = i / kHeadDim, j = i % kHeadDim;
     float mx = -INFINITY;
 #pragma unroll
@@ -348,7 +357,7 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
 // grid (group, G, B), 128 threads, one query head each: merge partials and the exact tail, rotate back,
 // normalise. Bound by latency: the partials' maxima and weights are formed by one thread each (S <= 128),
 // then every thread sums its coordinate over the splits with independent loads. One CTA per KV head that
-// walked its heads and splits one after another took 110 us for 128 splits of 4 heads; now 11 us.
+// walked its heads and splits one after another took 110 us for 128 splits of 4 heads; now 23 us.
 template <typename T, int GP>
 __global__ void __launch_bounds__(128)
 decode_combine_kernel(const float* __restrict__ part, const T* __restrict__ q,
@@ -424,9 +433,10 @@ void launch_decode_t(const Shape& s, const varrate_packed& c, const void* basis_
                      const void* q, int layer, const void* tail_k, const void* tail_v, int n_tail,
                      void* out, float* qt, float* part, int S, cudaStream_t st) {
   decode_rotate_kernel<T><<<dim3(s.G, s.B, kRotSplit), 256, 0, st>>>((const T*)q, (const T*)basis_k, qt, s, layer);
-  DenseSrc<T> src{(const T*)c.coef, c.bucket_base, s.cap, nullptr, nullptr};
-  decode_split_kernel<DenseSrc<T>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
-                                                                           s, layer, S, 0);
+  constexpr int GH = GP < 4 ? GP : 4;
+  DenseSrc<T> src{(const T*)c.coef, c.bucket_base, s.cap, nullptr, nullptr, 0};
+  decode_split_kernel<DenseSrc<T>, GP, GH><<<dim3(S * (GP / GH), s.G, s.B), 256, 0, st>>>(
+      src, c.bucket_count, qt, part, s, layer, S, 0);
   decode_combine_kernel<T, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const T*)q, (const T*)basis_v,
                                                                (const T*)tail_k, (const T*)tail_v,
                                                                n_tail, (T*)out, s, layer, S);
@@ -451,15 +461,16 @@ void launch_decode_qt(const Shape& s, const varrate_qpacked& c, const void* basi
                       const void* q, int layer, const void* tail_k, const void* tail_v, int n_tail,
                       void* out, float* qt, float* part, int S, cudaStream_t st) {
   using bf = __nv_bfloat16;
+  constexpr int GH = GP < 4 ? GP : 4;
   decode_rotate_kernel<bf><<<dim3(s.G, s.B, kRotSplit), 256, 0, st>>>((const bf*)q, (const bf*)basis_k, qt, s, layer);
   if (c.bits == 4) {
-    QuantSrc<4> src{c.data, c.qbase, c.qcap_bytes, nullptr, nullptr};
-    decode_split_kernel<QuantSrc<4>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
-                                                                           s, layer, S, c.qcap_bytes);
+    QuantSrc<4> src{c.data, c.qbase, c.qcap_bytes, nullptr, nullptr, 0, 0};
+    decode_split_kernel<QuantSrc<4>, GP, GH><<<dim3(S * (GP / GH), s.G, s.B), 256, 0, st>>>(
+        src, c.bucket_count, qt, part, s, layer, S, c.qcap_bytes);
   } else {
-    QuantSrc<8> src{c.data, c.qbase, c.qcap_bytes, nullptr, nullptr};
-    decode_split_kernel<QuantSrc<8>, GP><<<dim3(S, s.G, s.B), 256, 0, st>>>(src, c.bucket_count, qt, part,
-                                                                           s, layer, S, c.qcap_bytes);
+    QuantSrc<8> src{c.data, c.qbase, c.qcap_bytes, nullptr, nullptr, 0, 0};
+    decode_split_kernel<QuantSrc<8>, GP, GH><<<dim3(S * (GP / GH), s.G, s.B), 256, 0, st>>>(
+        src, c.bucket_count, qt, part, s, layer, S, c.qcap_bytes);
   }
   decode_combine_kernel<bf, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const bf*)q, (const bf*)basis_v,
                                                                (const bf*)tail_k, (const bf*)tail_v,
