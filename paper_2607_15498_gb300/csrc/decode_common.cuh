@@ -126,6 +126,42 @@ __device__ __forceinline__ Item next_rr(const Tb& sm, Item x, int k) {
   return item_at(sm, k);
 }
 
+// The same with short items apart: the last tile of a bucket with at most kShort slots. Entries of it_pref
+// then hold two prefixes, of the long items in the low 24 bits and of the short ones (at most one a
+// bucket) above them; items are numbered long ones first. A short item's place in its bucket follows
+// from the count, so it_lo stays that of the long ones.
+constexpr int kShort = 32;
+constexpr uint32_t kLongMask = 0x00FFFFFFu;
+
+__device__ __forceinline__ uint32_t split_count(long long i0, long long i1, int n) {
+  const long long n8 = pad8(n), nit = (n8 + ISL - 1) / ISL;
+  const bool has = i1 > i0 && i1 == nit && n8 - (nit - 1) * ISL <= kShort;
+  return (uint32_t)(i1 - i0) - (has ? 1u : 0u) + (has ? 1u << 24 : 0u);
+}
+
+template <class Tb>
+__device__ __forceinline__ Item item_at_split(const Tb& sm, int k, int n_long) {
+  const bool is_long = k < n_long;
+  const int sh = is_long ? 0 : 24;
+  const uint32_t mask = is_long ? kLongMask : 0xFFu, kk = (uint32_t)(is_long ? k : k - n_long);
+  int lo = 0, hi = kMaxR + 1;   // prefix[lo] <= kk < prefix[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if ((((uint32_t)sm.it_pref[mid] >> sh) & mask) <= kk) lo = mid; else hi = mid;
+  }
+  Item x;
+  x.r = lo;
+  x.it = is_long ? sm.it_lo[lo] + (int)(kk - ((uint32_t)sm.it_pref[lo] & kLongMask))
+                 : (int)((pad8(sm.cnt[lo]) - 1) / ISL);
+  return x;
+}
+
+template <int STRIDE, class Tb>
+__device__ __forceinline__ Item next_rr_split(const Tb& sm, Item x, int k, int n_long) {
+  if (k < (int)((uint32_t)sm.it_pref[x.r + 1] & kLongMask)) { x.it += STRIDE; return x; }
+  return item_at_split(sm, k, n_long);
+}
+
 // Rows per chunk of a tile of tl slots, as log2: as many rows as fill one 8 KB stage (32 rows of a
 // full 128-slot tile, 64 of a tile of at most 64 slots, all 128 of a tile of at most 32). The
 // sparse high-rank buckets end in short tiles; reading them in few chunks keeps their items from
