@@ -9,15 +9,21 @@
 //                         shuffle tree, so the value is reproducible), and the anchors copied into a
 //                         dense [B L][2][G][n_ap][d] block (n_ap = anchor count rounded up to 256,
 //                         padding rows zero with norm +inf, so they are never chosen);
-//   anchor_search_tc_kernel  one CTA per 128 tokens of one (sequence, layer): S = Z_tile A^T by
-//                         tcgen05.mma (M = 128 tokens x N = 256 anchors per accumulator, K = D in
+//   anchor_search_tc_kernel  a CTA pair (cta_group::2) per 256 tokens of one (sequence, layer): S = Z_tile A^T
+//                         by tcgen05.mma (M = 256 tokens x N = 256 anchors per accumulator, K = D in
 //                         steps of 64 columns, each step one head half of K or V fed by TMA with a
-//                         128-byte swizzle), both TMEM accumulators in use (512 columns) so that the
+//                         128-byte swizzle: each CTA stages its own 128 tokens and half of the anchors),
+//                         both TMEM accumulators in use (512 columns) so that the
 //                         epilogue of one anchor tile overlaps the products of the next. Epilogue
 //                         thread = token row: it turns its 256 scores into distances and keeps the
 //                         8 smallest (distance, anchor) pairs in registers, in lexicographic order;
 //                         the two epilogue groups (alternate anchor tiles) merge their lists at the
 //                         end and the first c pairs are stored.
+// What bounds the search is what each SM takes in from L2: at 64 bytes a clock, 128 tokens x 256 anchors x 64
+// columns on one CTA need 48 KB, 768 clocks, for 512 clocks of products; half the anchors per CTA make it
+// 32 KB. Before that the epilogue did: an insertion walked the list in a chain of compares, each warp for
+// each lane that inserted. 32768 tokens, 2048 anchors, D = 2048: 387 us on single CTAs and on pairs, 206 us on
+// pairs with the insertion of independent compares (61 % of the tensor pipe's time, 1.7 waves of pairs).
 // A third kernel, anchor_residual_kernel, forms the residuals e_t = z_t - z_bar_t of Eq. 2 from the
 // lists (Algorithm 1, third step).
 // Warp roles of the search kernel: one TMA producer warp, one MMA-issuing warp, eight epilogue
@@ -34,11 +40,11 @@ namespace vr {
 namespace {
 
 constexpr uint32_t kTries = 1u << 22;
-constexpr int AS_TM = 128;                  // tokens per CTA (MMA M)
+constexpr int AS_TM = 128;                  // tokens per CTA (half of the pair's MMA M)
 constexpr int AS_TN = 256;                  // anchors per accumulator (MMA N)
-constexpr int AS_ST = 4;                    // operand stages
+constexpr int AS_ST = 6;                    // operand stages
 constexpr int AS_ABYTES = AS_TM * 128;      // 128 token rows x 64 bf16
-constexpr int AS_BBYTES = AS_TN * 128;      // 256 anchor rows x 64 bf16
+constexpr int AS_BBYTES = AS_TN / 2 * 128;  // this CTA's 128 anchor rows x 64 bf16
 constexpr int AS_SBYTES = AS_ABYTES + AS_BBYTES;
 constexpr int AS_NGRP = 2;                  // epilogue groups of four warps (alternate anchor tiles)
 constexpr int AS_EPI = 4 * AS_NGRP;
@@ -46,7 +52,7 @@ constexpr int AS_THREADS = (AS_EPI + 2) * 32;
 constexpr int AS_LIST = 8;                  // (distance, anchor) pairs kept per token
 
 struct AsSmem {
-  uint64_t full[AS_ST], empty[AS_ST], tfull[AS_NGRP], tempty[AS_NGRP];
+  uint64_t full[AS_ST], empty[AS_ST], tfull[AS_NGRP], tempty[AS_NGRP], drain;
   uint32_t tmem;
   int err;
   float md[AS_TM][AS_LIST];                 // group 1's lists, merged by group 0
@@ -98,6 +104,22 @@ anchor_prep_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __r
   }
 }
 
+// Insert (d, j) where d < bd[s] into a list sorted by distance, j larger than every anchor in it: behind equal
+// distances, so the order stays lexicographic on (distance, anchor). A lane whose d is not below its last
+// entry keeps its list. The eight comparisons are independent: no chain through the list.
+__device__ __forceinline__ void list_insert_next(float (&bd)[AS_LIST], int (&bi)[AS_LIST], float d, int j) {
+  bool lt[AS_LIST];
+#pragma unroll
+  for (int s = 0; s < AS_LIST; ++s) lt[s] = d < bd[s];
+#pragma unroll
+  for (int s = AS_LIST - 1; s > 0; --s) {
+    bd[s] = lt[s - 1] ? bd[s - 1] : lt[s] ? d : bd[s];
+    bi[s] = lt[s - 1] ? bi[s - 1] : lt[s] ? j : bi[s];
+  }
+  bd[0] = lt[0] ? d : bd[0];
+  bi[0] = lt[0] ? j : bi[0];
+}
+
 // Insert (d, j) into the sorted list (bd, bi): lexicographic order on (distance, anchor), so equal
 // distances keep the lower anchor first whatever order the pairs arrive in.
 __device__ __forceinline__ void list_insert(float (&bd)[AS_LIST], int (&bi)[AS_LIST], float d, int j) {
@@ -116,8 +138,9 @@ __device__ __forceinline__ void list_insert(float (&bd)[AS_LIST], int (&bi)[AS_L
 }
 
 // ------------------------------------------------------------------------------ search
-// grid (ceil(N / 128), B * L).
-__global__ void __launch_bounds__(AS_THREADS, 1)
+// grid (2 ceil(N / 256), B * L) in clusters of two along x. The even CTA's full and tempty barriers serve the
+// pair; each CTA has its own empty and tfull barriers, which the pair's commits arrive on.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(AS_THREADS, 1)
 anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_constant__ CUtensorMap tv,
                         const __grid_constant__ CUtensorMap ta, const float* __restrict__ tnorm,
                         const float* __restrict__ anorm, int32_t* __restrict__ idx_out,
@@ -127,21 +150,26 @@ anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_con
   unsigned char* smem = raw_smem + ((1024 - (smem_addr(raw_smem) & 1023)) & 1023);
   AsSmem& sm = *reinterpret_cast<AsSmem*>(smem + AS_ST * AS_SBYTES);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = blockIdx.x & 1;
   const int64_t bl = blockIdx.y;
   const int64_t t0 = (int64_t)blockIdx.x * AS_TM;
+  // the odd CTA of the last pair may have no tokens: it loads its partner's and stores nothing
+  const int64_t t_load = t0 < N ? t0 : t0 - AS_TM;
   const int n_kb = 4 * G;                    // 64-column steps over D = 2 G d
   const int n_at = n_ap / AS_TN;
   const int total = n_at * n_kb;
 
   if (warp == AS_EPI + 1 && lane == 0) {
     for (int i = 0; i < AS_ST; ++i) { mbar_init(&sm.full[i], 1); mbar_init(&sm.empty[i], 1); }
-    for (int i = 0; i < AS_NGRP; ++i) { mbar_init(&sm.tfull[i], 1); mbar_init(&sm.tempty[i], 4); }
+    for (int i = 0; i < AS_NGRP; ++i) { mbar_init(&sm.tfull[i], 1); mbar_init(&sm.tempty[i], 8); }
+    mbar_init(&sm.drain, 1);
     sm.err = 0;
     fence_mbar_init();
   }
-  if (warp == 0) tmem_alloc(&sm.tmem, AS_NGRP * AS_TN);
+  if (warp == 0) tmem_alloc2(&sm.tmem, AS_NGRP * AS_TN);
   tc_fence_before();
   __syncthreads();
+  cluster_barrier();   // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem = sm.tmem;
   const uint32_t stage0 = smem_addr(smem);
@@ -151,40 +179,49 @@ anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_con
   for (int s = 0; s < AS_LIST; ++s) { bd[s] = INFINITY; bi[s] = -1; }
 
   if (warp == AS_EPI) {
-    if (lane == 0) {                                    // TMA producer
-      for (int i = 0; i < total; ++i) {
+    if (lane == 0) {                                    // TMA producer: this CTA's operand halves
+      int i = 0;
+      for (; i < total; ++i) {
         const int at = i / n_kb, kb = i - at * n_kb, st = i % AS_ST;
-        if (!mbar_wait_bounded(&sm.empty[st], ((i / AS_ST) & 1) ^ 1, kTries)) { sm.err = 1; break; }
+        if (!mbar_wait_cluster(&sm.empty[st], ((i / AS_ST) & 1) ^ 1, kTries)) { sm.err = 1; break; }
         const int kv = kb >= 2 * G;
         const int g = (kb >> 1) - kv * G, half = kb & 1;
-        const uint32_t dst = stage0 + st * AS_SBYTES;
-        mbar_arrive_expect_tx(&sm.full[st], AS_SBYTES);
+        const uint32_t dst = stage0 + st * AS_SBYTES, bar = cluster_addr(&sm.full[st], 0);
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[st], 2 * AS_SBYTES);
         // token rows past N read the next stream's rows (or zeros past the tensor): never stored
-        tma_load_2d(dst, kv ? &tv : &tk, 64 * half, (int)((bl * G + g) * N + t0), &sm.full[st]);
-        tma_load_2d(dst + AS_ABYTES, &ta, 64 * half, (int)(((bl * 2 + kv) * G + g) * n_ap + at * AS_TN),
-                    &sm.full[st]);
+        tma_load_2d_pair(dst, kv ? &tv : &tk, 64 * half, (int)((bl * G + g) * N + t_load), bar);
+        tma_load_2d_pair(dst + AS_ABYTES, &ta, 64 * half,
+                         (int)(((bl * 2 + kv) * G + g) * n_ap + at * AS_TN + (int)rank * (AS_TN / 2)), bar);
       }
+      // every copy of the pair has landed before either CTA can end, also after a wait that gave up
+      if (rank == 0)
+        for (int j = max(0, i - AS_ST); j < i; ++j) mbar_wait_cluster(&sm.full[j % AS_ST], (j / AS_ST) & 1, kTries);
     }
   } else if (warp == AS_EPI + 1) {
-    if (lane == 0) {                                    // MMA issuer
-      constexpr uint32_t idesc = idesc_bf16_f32(AS_TM, AS_TN);
+    if (lane == 0 && rank == 0) {                       // MMA issuer of the pair
+      constexpr uint32_t idesc = idesc_bf16_f32(2 * AS_TM, AS_TN);
       bool ok = true;
       for (int at = 0; at < n_at && ok; ++at) {
         const int b = at & 1;
-        if (!mbar_wait_bounded(&sm.tempty[b], ((at >> 1) & 1) ^ 1, kTries)) { sm.err = 1; break; }
+        if (!mbar_wait_cluster(&sm.tempty[b], ((at >> 1) & 1) ^ 1, kTries)) { ok = false; break; }
         tc_fence_after();
         for (int kb = 0; kb < n_kb; ++kb) {
           const int i = at * n_kb + kb, st = i % AS_ST;
-          if (!mbar_wait_bounded(&sm.full[st], (i / AS_ST) & 1, kTries)) { sm.err = 1; ok = false; break; }
+          if (!mbar_wait_cluster(&sm.full[st], (i / AS_ST) & 1, kTries)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a0 = stage0 + st * AS_SBYTES, b0 = a0 + AS_ABYTES;
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks)
-            tc_mma_bf16(tmem + b * AS_TN, sdesc_sw128(a0 + ks * 32), sdesc_sw128(b0 + ks * 32), idesc,
-                        (kb | ks) != 0);
-          tc_commit(&sm.empty[st]);
+            tc_mma2_bf16(tmem + b * AS_TN, sdesc_sw128(a0 + ks * 32), sdesc_sw128(b0 + ks * 32), idesc,
+                         (kb | ks) != 0);
+          tc_commit2(&sm.empty[st]);
         }
-        if (ok) tc_commit(&sm.tfull[b]);
+        if (ok) tc_commit2(&sm.tfull[b]);
+      }
+      if (!ok) {   // the products in flight end before TMEM is freed
+        sm.err = 1;
+        tc_commit2(&sm.drain);
+        mbar_wait_cluster(&sm.drain, 0, kTries);
       }
     }
   } else {                                              // epilogue: one token row, alternate tiles
@@ -196,7 +233,7 @@ anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_con
     bool bad = false;
     for (int at = eg; at < n_at; at += AS_NGRP) {
       const int b = at & 1;
-      if (!bad && !mbar_wait_bounded(&sm.tfull[b], (at >> 1) & 1, kTries)) { sm.err = 1; bad = true; }
+      if (!bad && !mbar_wait_cluster(&sm.tfull[b], (at >> 1) & 1, kTries)) { sm.err = 1; bad = true; }
       tc_fence_after();
       const uint32_t taddr = tmem + b * AS_TN + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
@@ -213,14 +250,15 @@ anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_con
           for (int e = 0; e < 4; ++e) {
             const int jj = q4 * 4 + e;
             const float dd = fmaxf(fmaf(-2.f, sv[jj], nz + nav[e]), 0.f);
-            if (dd < bd[AS_LIST - 1]) list_insert(bd, bi, dd, j0 + jj);
+            // some lane's list takes it (a vote, so that the warp stays together); no-op for the others
+            if (__any_sync(0xffffffffu, dd < bd[AS_LIST - 1])) list_insert_next(bd, bi, dd, j0 + jj);
           }
         }
         __syncwarp();
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.tempty[b]);
+      if (lane == 0) mbar_arrive_cluster(cluster_addr(&sm.tempty[b], 0));
     }
     if (eg == 1) {
 #pragma unroll
@@ -245,59 +283,163 @@ anchor_search_tc_kernel(const __grid_constant__ CUtensorMap tk, const __grid_con
       }
     }
   }
-  if (warp == 0) tmem_dealloc(tmem, AS_NGRP * AS_TN);
   if (tid == 0 && sm.err) raise_status(dev_status, VARRATE_ERR_TIMEOUT);
+  __syncwarp();
+  cluster_barrier();   // no CTA leaves, or frees TMEM, while the other may still signal it or use the pair's TMEM
+  if (warp == 0) tmem_dealloc2(tmem, AS_NGRP * AS_TN);
 }
 
 size_t search_smem_bytes() { return 1024 + (size_t)AS_ST * AS_SBYTES + sizeof(AsSmem); }
 
 // ------------------------------------------------------------------------------ residual
-// Eq. 2: e_t = z_t - mean of the anchors listed for t. grid (ceil(N / 8), B * L), 256 threads: warp w
-// takes token blockIdx.x * 8 + w; lane l owns coordinates 4 l .. 4 l + 3 of every head row. The
-// listed anchors are summed in list order in fp32 (bf16 values are exact in fp32), divided by
-// their count (IEEE division), subtracted from z_t and rounded to bf16.
+// Eq. 2: e_t = z_t - mean of the anchors listed for t. The listed anchors are summed in list order in
+// fp32 (bf16 values are exact in fp32), divided by their count (IEEE division; by a power of two the
+// product with its exact reciprocal is the same number), subtracted from z_t and rounded to bf16.
+// The list of a token: rows[s] = anchor, or n_a (a row of zeros) for a skipped entry; returns the number of valid
+// entries, 0 when there is none or an entry is out of [-1, n_a). C > 0: lists of C entries, else of c <= 8.
+template <int C>
+__device__ __forceinline__ int load_list(const int32_t* __restrict__ p, int c, int n_a, uint32_t (&rows)[C ? C : AS_LIST]) {
+  constexpr int K = C ? C : AS_LIST;
+  int x[K];
+  if constexpr (C == 4) {   // 16-byte aligned
+    const int4 q = __ldg(reinterpret_cast<const int4*>(p));
+    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+  } else {
+#pragma unroll
+    for (int s = 0; s < K; ++s) x[s] = s < c ? __ldg(p + s) : -1;
+  }
+  int m = K;
+  uint32_t worst = 0;
+#pragma unroll
+  for (int s = 0; s < K; ++s) {
+    worst = max(worst, (uint32_t)(x[s] + 1));   // -1 .. n_a - 1 -> 0 .. n_a; anything else is above
+    m += x[s] >> 31;
+    rows[s] = min((uint32_t)x[s], (uint32_t)n_a);
+  }
+  return worst > (uint32_t)n_a ? 0 : m;
+}
+
+// acc + x with x a bf16 (exact in fp32): one mixed-precision add per element, rounded to nearest.
+__device__ __forceinline__ void add8(float (&acc)[8], uint4 u) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n add.rn.f32.bf16 %0, l, %0;\n add.rn.f32.bf16 %1, h, %1;\n}\n"
+        : "+f"(acc[2 * i]), "+f"(acc[2 * i + 1]) : "r"(w[i]));
+}
+
+__device__ __forceinline__ uint4 residual8(uint4 z, float (&acc)[8], int m) {
+  if ((m & (m - 1)) == 0) {
+    const float inv = m == 1 ? 1.f : m == 2 ? 0.5f : m == 4 ? 0.25f : 0.125f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = __fmul_rn(acc[i], inv);
+  } else {
+    const float fm = (float)m;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = __fdiv_rn(acc[i], fm);
+  }
+  const uint32_t w[4] = {z.x, z.y, z.z, z.w};
+  uint32_t o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    o[i] = pack_bf16(__fsub_rn(__uint_as_float(w[i] << 16), acc[2 * i]),
+                     __fsub_rn(__uint_as_float(w[i] & 0xffff0000u), acc[2 * i + 1]));
+  return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+// Slab form: a CTA keeps CW columns of every anchor of one (sequence, layer, head, K-or-V) in shared memory
+// (plus a zero row for skipped entries) and streams its share of the tokens past them, 16 bytes a thread.
+// Read straight from L2 the c listed anchors of every token are c times the bytes of K and V themselves;
+// from shared memory K and V are read once and the residuals written once. Bound by shared-memory reads (rows
+// of 64 bytes: two of them share a wavefront when their parities differ) and instructions. 2 layers x 8
+// heads x 32768 tokens, 4 of 2048 anchors each (538 MB): a warp per token reading L2 248 us, this 141 us.
+// grid (column blocks x splits x 2 G, B L).
+constexpr int RS_THREADS = 1024;
+constexpr int RS_TOK = 2;                    // tokens per thread whose loads are in flight together
+constexpr size_t RS_SMEM = 208 * 1024;       // most shared memory for a slab
+
+template <int CW, int C>
+__global__ void __launch_bounds__(RS_THREADS, 1)
+anchor_residual_slab_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+                            const int32_t* __restrict__ idx, __nv_bfloat16* __restrict__ e,
+                            int32_t* __restrict__ dev_status, int G, int64_t N, int stride, int c, int n_a,
+                            int splits, int64_t share) {
+  constexpr int TPT = CW / 8, TOKS = RS_THREADS / TPT, NCB = kHeadDim / CW;   // threads a token, tokens a step
+  extern __shared__ uint4 slab[];            // [n_a + 1][TPT]
+  const int tid = threadIdx.x, part = tid % TPT;
+  const int cb = blockIdx.x % NCB, rest = blockIdx.x / NCB, split = rest % splits, kvg = rest / splits;
+  const int64_t bl = blockIdx.y;
+  const int kv = kvg >= G, g = kvg - kv * G;
+  const __nv_bfloat16* base = (kv ? v : k) + (bl * G + g) * N * kHeadDim + cb * CW;
+#pragma unroll 4
+  for (int i = tid; i < n_a * TPT; i += RS_THREADS)
+    slab[i] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)(i / TPT) * stride * kHeadDim) + part);
+  if (tid < TPT) slab[n_a * TPT + tid] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  constexpr int K = C ? C : AS_LIST;
+  const int64_t t_end = min(N, (split + 1) * share);
+  for (int64_t t0 = split * share + tid / TPT; t0 < t_end; t0 += TOKS * RS_TOK) {
+    uint4 z[RS_TOK];
+    uint32_t rows[RS_TOK][K];
+    int m[RS_TOK];
+#pragma unroll
+    for (int u = 0; u < RS_TOK; ++u) {
+      const int64_t t = t0 + u * TOKS;
+      if (t < t_end) {
+        z[u] = __ldcs(reinterpret_cast<const uint4*>(base + t * kHeadDim) + part);
+        m[u] = load_list<C>(idx + (bl * N + t) * c, c, n_a, rows[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < RS_TOK; ++u) {
+      const int64_t t = t0 + u * TOKS;
+      if (t >= t_end) break;
+      if (m[u] == 0) {
+        raise_status(dev_status, VARRATE_ERR_CORRUPT);
+        continue;
+      }
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int s = 0; s < K; ++s)
+        if (C || s < c) add8(acc, slab[rows[u][s] * TPT + part]);
+      __stcs(reinterpret_cast<uint4*>(e + ((bl * N + t) * 2 * G + kvg) * kHeadDim + cb * CW) + part,
+             residual8(z[u], acc, m[u]));
+    }
+  }
+}
+
+// Direct form, for more anchors than 16 columns of which fit in shared memory: a warp per token, half a warp
+// per head row (16 bytes a lane), the listed anchors read from L2. grid (ceil(N / 8), B L), 256 threads.
 __global__ void __launch_bounds__(256)
 anchor_residual_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                        const int32_t* __restrict__ idx, __nv_bfloat16* __restrict__ e,
                        int32_t* __restrict__ dev_status, int G, int64_t N, int stride, int c, int n_a) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l16 = lane & 15;
   const int64_t bl = blockIdx.y;
   const int64_t t = (int64_t)blockIdx.x * 8 + warp;
   if (t >= N) return;
-  int ai[AS_LIST];
-  int m = 0;
-  bool bad = false;
-#pragma unroll
-  for (int s = 0; s < AS_LIST; ++s) {
-    ai[s] = s < c ? __ldg(idx + (bl * N + t) * c + s) : -1;
-    if (ai[s] >= n_a || ai[s] < -1) bad = true;
-    if (ai[s] >= 0) ++m;
-  }
-  if (bad || m == 0) {                               // warp-uniform: every lane read the same list
+  uint32_t rows[AS_LIST];
+  const int m = load_list<0>(idx + (bl * N + t) * c, c, n_a, rows);
+  if (m == 0) {                                      // warp-uniform: every lane read the same list
     if (lane == 0) raise_status(dev_status, VARRATE_ERR_CORRUPT);
     return;
   }
-  const float fm = (float)m;
-  for (int kvg = 0; kvg < 2 * G; ++kvg) {
+#pragma unroll 2
+  for (int kvg = lane >> 4; kvg < 2 * G; kvg += 2) {
     const int kv = kvg >= G, g = kvg - kv * G;
     const __nv_bfloat16* base = (kv ? v : k) + (bl * G + g) * N * kHeadDim;
-    const uint2 zu = __ldg(reinterpret_cast<const uint2*>(base + t * kHeadDim) + lane);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    const uint4 z = __ldg(reinterpret_cast<const uint4*>(base + t * kHeadDim) + l16);
+    uint4 u[AS_LIST];
 #pragma unroll
     for (int s = 0; s < AS_LIST; ++s) {
-      if (ai[s] < 0) continue;
-      const uint2 u = __ldg(reinterpret_cast<const uint2*>(base + (int64_t)ai[s] * stride * kHeadDim) + lane);
-      acc[0] += __uint_as_float(u.x << 16);
-      acc[1] += __uint_as_float(u.x & 0xffff0000u);
-      acc[2] += __uint_as_float(u.y << 16);
-      acc[3] += __uint_as_float(u.y & 0xffff0000u);
+      u[s] = make_uint4(0, 0, 0, 0);
+      if (rows[s] < (uint32_t)n_a) u[s] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)rows[s] * stride * kHeadDim) + l16);
     }
-    const float z0 = __uint_as_float(zu.x << 16), z1 = __uint_as_float(zu.x & 0xffff0000u);
-    const float z2 = __uint_as_float(zu.y << 16), z3 = __uint_as_float(zu.y & 0xffff0000u);
-    uint2 o;
-    o.x = pack_bf16(__fsub_rn(z0, __fdiv_rn(acc[0], fm)), __fsub_rn(z1, __fdiv_rn(acc[1], fm)));
-    o.y = pack_bf16(__fsub_rn(z2, __fdiv_rn(acc[2], fm)), __fsub_rn(z3, __fdiv_rn(acc[3], fm)));
-    reinterpret_cast<uint2*>(e + ((bl * N + t) * 2 * G + kvg) * kHeadDim)[lane] = o;
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int s = 0; s < AS_LIST; ++s)
+      if (rows[s] < (uint32_t)n_a) add8(acc, u[s]);
+    reinterpret_cast<uint4*>(e + ((bl * N + t) * 2 * G + kvg) * kHeadDim)[l16] = residual8(z, acc, m);
   }
 }
 
@@ -322,8 +464,44 @@ bool anchor_residual_supported(const Shape& s, int stride, int c) {
          (int64_t)s.B * s.L <= 65535;
 }
 
+namespace {
+
+template <int CW>
+int launch_residual_slab(const Shape& s, const void* k, const void* v, int stride, int c, const int32_t* idx,
+                         void* e_out, int32_t* dev_status, int num_sms, cudaStream_t st) {
+  const int n_a = anchor_count(s.N, stride);
+  const size_t smem = (size_t)(n_a + 1) * CW * 2;
+  auto kernel = c == 4 ? anchor_residual_slab_kernel<CW, 4> : anchor_residual_slab_kernel<CW, 0>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM) != cudaSuccess) return -1;
+  // splits of the tokens that make waves x (steps of a CTA + its slab, read at about twice a step's rate) least
+  constexpr int64_t kStep = RS_THREADS / (CW / 8) * RS_TOK;
+  const int64_t units = (int64_t)s.B * s.L * 2 * s.G * (kHeadDim / CW), steps = (s.N + kStep - 1) / kStep;
+  const double setup = 1.0 + (double)n_a / (2.0 * kStep);
+  int64_t n = 1;
+  double best = 1e300;
+  for (int64_t i = 1; i <= steps && i <= 2 * num_sms; ++i) {
+    const double cost = (double)((units * i + num_sms - 1) / num_sms) * ((double)((steps + i - 1) / i) + setup);
+    if (cost < best * 0.999) { best = cost; n = i; }
+  }
+  const int64_t share = (steps + n - 1) / n * kStep;
+  n = (s.N + share - 1) / share;
+  const dim3 grid((unsigned)(kHeadDim / CW * n * 2 * s.G), (unsigned)((size_t)s.B * s.L));
+  kernel<<<grid, RS_THREADS, smem, st>>>(
+      (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, (__nv_bfloat16*)e_out, dev_status, s.G, s.N, stride, c,
+      n_a, (int)n, share);
+  return 1;
+}
+
+}  // namespace
+
 int launch_anchor_residual(const Shape& s, const void* k, const void* v, int stride, int c,
-                           const int32_t* idx, void* e_out, int32_t* dev_status, cudaStream_t st) {
+                           const int32_t* idx, void* e_out, int32_t* dev_status, int num_sms, cudaStream_t st) {
+  // the widest column block of all anchors (and the zero row) that fits in shared memory
+  const size_t rows = (size_t)anchor_count(s.N, stride) + 1;
+  if (rows * 128 * 2 <= RS_SMEM) return launch_residual_slab<128>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
+  if (rows * 64 * 2 <= RS_SMEM) return launch_residual_slab<64>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
+  if (rows * 32 * 2 <= RS_SMEM) return launch_residual_slab<32>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
+  if (rows * 16 * 2 <= RS_SMEM) return launch_residual_slab<16>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
   anchor_residual_kernel<<<dim3((unsigned)((s.N + 7) / 8), (unsigned)((size_t)s.B * s.L)), 256, 0, st>>>(
       (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, (__nv_bfloat16*)e_out, dev_status, s.G, s.N,
       stride, c, anchor_count(s.N, stride));
@@ -351,13 +529,13 @@ int launch_anchor_search(const Shape& s, const void* k, const void* v, int strid
   const uint64_t rows_a = (uint64_t)bl * 2 * s.G * n_ap;
   CUtensorMap tk, tv, ta;
   if (!make_tmap_rows_bf16(&tk, k, rows_kv, AS_TM) || !make_tmap_rows_bf16(&tv, v, rows_kv, AS_TM) ||
-      !make_tmap_rows_bf16(&ta, anchors, rows_a, AS_TN))
+      !make_tmap_rows_bf16(&ta, anchors, rows_a, AS_TN / 2))
     return -1;
   anchor_prep_kernel<<<dim3((unsigned)((s.N + 7) / 8), (unsigned)bl), 256, 0, st>>>(
       (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, anchors, anorm, tnorm, s.G, s.N, stride, n_a, n_ap);
   const size_t smem = search_smem_bytes();
   cudaFuncSetAttribute(anchor_search_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  anchor_search_tc_kernel<<<dim3((unsigned)((s.N + AS_TM - 1) / AS_TM), (unsigned)bl), AS_THREADS, smem, st>>>(
+  anchor_search_tc_kernel<<<dim3(2 * (unsigned)((s.N + 2 * AS_TM - 1) / (2 * AS_TM)), (unsigned)bl), AS_THREADS, smem, st>>>(
       tk, tv, ta, tnorm, anorm, idx_out, dist_out, dev_status, s.G, s.N, n_ap, c);
   return 2;
 }

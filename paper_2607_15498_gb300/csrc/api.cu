@@ -361,7 +361,8 @@ varrate_status varrate_anchor_residual(const varrate_config* cfg, const void* k,
   if (!aligned16({k, v, idx, e_out, dev_status})) return VARRATE_ERR_ARG;
   const Shape s = make_shape(cfg, cap_elems(cfg));
   if (!vr::anchor_residual_supported(s, stride, c)) return VARRATE_ERR_UNSUPPORTED;
-  vr::launch_anchor_residual(s, k, v, stride, c, idx, e_out, dev_status, (cudaStream_t)stream);
+  if (vr::launch_anchor_residual(s, k, v, stride, c, idx, e_out, dev_status, num_sms(), (cudaStream_t)stream) < 0)
+    return VARRATE_ERR_CUDA;
   return launched();
 }
 

@@ -101,6 +101,6 @@ int launch_anchor_search(const Shape& s, const void* k, const void* v, int strid
                          float* dist_out, int32_t* dev_status, void* ws, cudaStream_t st);
 bool anchor_residual_supported(const Shape& s, int stride, int c);
 int launch_anchor_residual(const Shape& s, const void* k, const void* v, int stride, int c,
-                           const int32_t* idx, void* e_out, int32_t* dev_status, cudaStream_t st);
+                           const int32_t* idx, void* e_out, int32_t* dev_status, int num_sms, cudaStream_t st);
 
 }  // namespace vr
