@@ -24,9 +24,10 @@ namespace vr {
 
 namespace {
 
-constexpr int kThreads = 256;          // few warps: each pass ends in 15 warp sums and two barriers
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kCand = 15;              // water levels per pass
+static_assert(kWarps > kCand, "a warp adds the warps' sums of one level");
 constexpr int kMaxCluster = 8;         // portable cluster size
 constexpr int64_t kMaxCached = 49152;  // normalised saliences kept in shared memory (192 KB)
 
@@ -50,6 +51,12 @@ __device__ __forceinline__ void warp_stats(float& mn, float& mx, float& sum) {
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     sum += __shfl_xor_sync(0xffffffffu, sum, o);
   }
+}
+
+__device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // Offset of the k-th of kCand levels around a guess whose error is expected within `reach` (in units of
@@ -143,11 +150,10 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
   const bool flat = uniform || !(mx > mn);
   const float den = flat ? 1.0f : __fsub_rn(mx, mn);
   // a thread normalises, and reads in every pass, the entries it loaded itself
-  for (int64_t i = tid; i < min(cnt, cached); i += kThreads)
+  for (int64_t i = tid; i < min(cnt, cached); i += kThreads)   // entries past n_cached: normalised when read
     sh_cache[i] = shat_of(uniform ? 0.f : sh_cache[i], mn, den, flat);
-  auto shat = [&](int64_t i) {
-    return i < cached ? sh_cache[i] : shat_of(uniform ? 0.f : sl[t0 + i], mn, den, flat);
-  };
+  const int n_cached = (int)min(cnt, cached);
+  auto shat_far = [&](int64_t i) { return shat_of(uniform ? 0.f : sl[t0 + i], mn, den, flat); };
   const float fmin_r = (float)s.r_min, fmax_r = (float)s.r_max;
   const bool wide = share >= (int64_t(1) << 24);   // a warp's sum may pass 32 bits
 
@@ -172,63 +178,63 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
       guess = lo + (int64_t)((float)span * ((float)(s.Bc - tot_lo) / (float)(tot_hi - tot_lo)));
       reach = max(span / 4, 1u);
     }
-    // level k of this pass, in (lo, hi), not decreasing in k
-    auto level = [&](int k) -> uint32_t {
-      if (even) return min(lo + step * (k + 1), hi - 1);
-      const int64_t b = guess + spread(k, reach) + (k - kCand / 2);
-      return (uint32_t)max((int64_t)lo + 1, min(b, (int64_t)hi - 1));
-    };
+    // level k of this pass, in (lo, hi), not decreasing in k: lane k forms it
+    const int k0 = min(lane, kCand - 1);
+    const int64_t near = guess + spread(k0, reach) + (k0 - kCand / 2);
+    const uint32_t mine = even ? min(lo + step * (k0 + 1), hi - 1)
+                               : (uint32_t)max((int64_t)lo + 1, min(near, (int64_t)hi - 1));
     float lam[kCand];
     uint32_t acc[kCand];
 #pragma unroll
     for (int k = 0; k < kCand; ++k) {
-      lam[k] = __uint_as_float(level(k));
+      lam[k] = __uint_as_float(__shfl_sync(0xffffffffu, mine, k));
       acc[k] = 0;
     }
     uint32_t seen = 0;
-    for (int64_t i = tid; i < cnt; i += kThreads) {
-      const float sh = shat(i);
+    auto add = [&](float sh) {
 #pragma unroll
       for (int k = 0; k < kCand; ++k) acc[k] += rank_bits(lam[k], sh, fmin_r, fmax_r);
       ++seen;
-    }
+    };
+    for (int i = tid; i < n_cached; i += kThreads) add(sh_cache[i]);
+    for (int64_t i = n_cached + tid; i < cnt; i += kThreads) add(shat_far(i));
+    // modulo 2^32 the sums themselves; lane k keeps that of level k
+    unsigned long long w = 0;
+    if (!wide) {
 #pragma unroll
-    for (int k = 0; k < kCand; ++k) {
-      const uint32_t v = acc[k] - seen * kRankBias;   // modulo 2^32: the sum itself
-      unsigned long long w;
-      if (wide) {
-        w = v;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-      } else {
-        w = __reduce_add_sync(0xffffffffu, v);
+      for (int k = 0; k < kCand; ++k) {
+        const uint32_t v = __reduce_add_sync(0xffffffffu, acc[k] - seen * kRankBias);
+        if (lane == k) w = v;
       }
-      if (lane == 0) sm.wsum[k][warp] = w;
-    }
-    __syncthreads();
-    if (tid < kCand * C) {   // thread (candidate, peer)
-      const int k = tid % kCand, c = tid / kCand;
-      unsigned long long w = 0;
+    } else {
 #pragma unroll
-      for (int i = 0; i < kWarps; ++i) w += sm.wsum[k][i];
-      *cluster.map_shared_rank(&sm.tot[pass & 1][rank][k], c) = (long long)w;
+      for (int k = 0; k < kCand; ++k) {
+        const unsigned long long v = warp_sum64(acc[k] - seen * kRankBias);
+        if (lane == k) w = v;
+      }
     }
-    cluster.sync();   // also orders this pass's reads of wsum before the next pass's writes
+    if (lane < kCand) sm.wsum[lane][warp] = w;
+    __syncthreads();
+    if (warp < kCand) {
+      w = lane < kWarps ? sm.wsum[warp][lane] : 0;
+      w = wide ? warp_sum64(w) : __reduce_add_sync(0xffffffffu, (uint32_t)w);
+      if (lane < C) *cluster.map_shared_rank(&sm.tot[pass & 1][rank][warp], lane) = (long long)w;
+    }
+    // also orders this pass's reads of wsum before the next pass's writes
+    if (C > 1) cluster.sync(); else __syncthreads();
     long long total = 0;
-    if (lane < kCand)
-      for (int c = 0; c < C; ++c) total += sm.tot[pass & 1][c][lane];
+    for (int c = 0; c < C; ++c) total += sm.tot[pass & 1][c][k0];
     // the levels do not decrease, so those that fit come first
     const int m = __popc(__ballot_sync(0xffffffffu, lane < kCand && total <= s.Bc));
-    const uint32_t below = m > 0 ? level(m - 1) : lo, above = m < kCand ? level(m) : hi;
-    if (m > 0) tot_lo = __shfl_sync(0xffffffffu, total, m - 1);
-    if (m < kCand) tot_hi = __shfl_sync(0xffffffffu, total, m);
-    lo = below;
-    hi = above;
+    const uint32_t below = __shfl_sync(0xffffffffu, mine, max(m - 1, 0)), above = __shfl_sync(0xffffffffu, mine, min(m, kCand - 1));
+    const long long t_below = __shfl_sync(0xffffffffu, total, max(m - 1, 0)), t_above = __shfl_sync(0xffffffffu, total, min(m, kCand - 1));
+    if (m > 0) { lo = below; tot_lo = t_below; }
+    if (m < kCand) { hi = above; tot_hi = t_above; }
   }
 
   const float lam = __uint_as_float(lo);
   for (int64_t i = tid; i < cnt; i += kThreads)
-    rk[t0 + i] = (uint8_t)(rank_bits(lam, shat(i), fmin_r, fmax_r) - kRankBias);
+    rk[t0 + i] = (uint8_t)(rank_bits(lam, i < n_cached ? sh_cache[i] : shat_far(i), fmin_r, fmax_r) - kRankBias);
   if (rank == 0 && tid == 0 && realized) realized[bl] = tot_lo;
 }
 

@@ -354,78 +354,104 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
   }
 }
 
-// grid (group, G, B), 128 threads, one query head each: merge partials and the exact tail, rotate back,
-// normalise. Bound by latency: the partials' maxima and weights are formed by one thread each (S <= 128),
-// then every thread sums its coordinate over the splits with independent loads. One CTA per KV head that
-// walked its heads and splits one after another took 110 us for 128 splits of 4 heads; now 23 us.
+// grid (group, G, B), 512 threads, one query head each: merge partials and the exact tail, rotate back,
+// normalise. Bound by latency: the weights are formed by one thread per split (S <= 128), then four
+// quarters of the block sum the splits, the basis rows and the tail tokens for all 128 coordinates, with
+// independent loads, and add up through shared memory in a fixed order. One CTA of 128 threads per KV head
+// that walked its heads and splits one after another took 110 us for 128 splits of 4 heads, a CTA of 128
+// threads per head 23 us, this FIGURES.
+constexpr int kCombThreads = 512;
+constexpr int kCombParts = kCombThreads / kHeadDim;
+
 template <typename T, int GP>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kCombThreads)
 decode_combine_kernel(const float* __restrict__ part, const T* __restrict__ q,
                       const T* __restrict__ basis_v, const T* __restrict__ tail_k,
                       const T* __restrict__ tail_v, int n_tail, T* __restrict__ out, Shape s,
                       int layer, int S) {
-  __shared__ float ot[kHeadDim];
+  __shared__ float ot[kCombParts][kHeadDim], yt[kCombParts][kHeadDim];
+  __shared__ float lt[2][kCombParts];                 // softmax sums: of the splits, of the tail
   __shared__ float tsc[kMaxTail];
   __shared__ float wgt[kMaxSplits], lsum[kMaxSplits];
-  __shared__ float red[4];
+  __shared__ float red[kCombThreads / 32];
   const int hh = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int quart = tid / kHeadDim, col = tid % kHeadDim;
   const T* U = basis_v + ((int64_t)layer * s.G + g) * kHeadDim * kHeadDim;
   const float scale = kLog2e * rsqrtf((float)kHeadDim);
   const float* pb = part + (((int64_t)b * s.G + g) * S * GP + hh) * (kHeadDim + 2);
   constexpr int kStep = GP * (kHeadDim + 2);   // floats between the splits of a head
   const int h = g * s.grp + hh;
-  auto block_max = [&](float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    v = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-    __syncthreads();
-    return v;
-  };
   // exact tail scores (log2 units)
-  float tmax = -INFINITY;
+  float mloc = -INFINITY;
   if (n_tail > 0) {
     const T* tk = tail_k + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
     const float4 qv = load4(q + ((int64_t)b * s.H + h) * kHeadDim + lane * 4);
 #pragma unroll 4
-    for (int t = warp; t < n_tail; t += 4) {
+    for (int t = warp; t < n_tail; t += kCombThreads / 32) {
       const float4 kv = load4(tk + (int64_t)t * kHeadDim + lane * 4);
       float a = fmaf(qv.w, kv.w, fmaf(qv.z, kv.z, fmaf(qv.y, kv.y, qv.x * kv.x)));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
       a *= scale;
       if (lane == 0) tsc[t] = a;
-      tmax = fmaxf(tmax, a);
+      mloc = fmaxf(mloc, a);
     }
   }
+  // this thread's part of U_V, in flight while the partials are merged
+  constexpr int kRows = kHeadDim / kCombParts;
+  float u[kRows];
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) u[j] = to_f(U[(quart * kRows + j) * kHeadDim + col]);
   const float m = tid < S ? pb[(int64_t)tid * kStep + kHeadDim] : -INFINITY;
   if (tid < S) lsum[tid] = pb[(int64_t)tid * kStep + kHeadDim + 1];
-  const float mx = block_max(fmaxf(m, tmax));
+  mloc = fmaxf(mloc, m);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, o));
+  if (lane == 0) red[warp] = mloc;
+  __syncthreads();
+  float mx = red[0];
+#pragma unroll
+  for (int w = 1; w < kCombThreads / 32; ++w) mx = fmaxf(mx, red[w]);
   if (tid < S) wgt[tid] = m == -INFINITY ? 0.f : exp2f(m - mx);   // an empty split holds zeros
   __syncthreads();
-  float l = 0.f, o = 0.f;
-#pragma unroll 8
-  for (int sp = 0; sp < S; ++sp) {
-    l = fmaf(lsum[sp], wgt[sp], l);
-    o = fmaf(pb[(int64_t)sp * kStep + tid], wgt[sp], o);
-  }
-  ot[tid] = o;
-  __syncthreads();
-  float y = 0.f;
+  {
+    float l = 0.f, o = 0.f;
 #pragma unroll 16
-  for (int j = 0; j < kHeadDim; ++j) y = fmaf(to_f(U[j * kHeadDim + tid]), ot[j], y);
+    for (int sp = quart; sp < S; sp += kCombParts) {
+      l = fmaf(lsum[sp], wgt[sp], l);
+      o = fmaf(pb[(int64_t)sp * kStep + col], wgt[sp], o);
+    }
+    ot[quart][col] = o;
+    if (col == 0) lt[0][quart] = l;
+  }
+  float y = 0.f, l = 0.f;
   if (n_tail > 0) {
     const T* tv = tail_v + ((int64_t)b * s.G + g) * n_tail * kHeadDim;
 #pragma unroll 8
-    for (int t = 0; t < n_tail; ++t) {
+    for (int t = quart; t < n_tail; t += kCombParts) {
       const float p = exp2f(tsc[t] - mx);
       l += p;
-      y = fmaf(p, to_f(tv[(int64_t)t * kHeadDim + tid]), y);
+      y = fmaf(p, to_f(tv[(int64_t)t * kHeadDim + col]), y);
     }
   }
-  out[((int64_t)b * s.H + h) * kHeadDim + tid] = from_f<T>(y / l);
+  if (col == 0) lt[1][quart] = l;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) {
+    float o = 0.f;
+#pragma unroll
+    for (int i = 0; i < kCombParts; ++i) o += ot[i][quart * kRows + j];
+    y = fmaf(u[j], o, y);
+  }
+  yt[quart][col] = y;
+  __syncthreads();
+  if (quart == 0) {
+    float sum = 0.f, l = 0.f;
+#pragma unroll
+    for (int i = 0; i < kCombParts; ++i) { sum += yt[i][col]; l += lt[0][i] + lt[1][i]; }
+    out[((int64_t)b * s.H + h) * kHeadDim + col] = from_f<T>(sum / l);
+  }
 }
 
 template <typename T, int GP>
@@ -437,7 +463,7 @@ void launch_decode_t(const Shape& s, const varrate_packed& c, const void* basis_
   DenseSrc<T> src{(const T*)c.coef, c.bucket_base, s.cap, nullptr, nullptr, 0};
   decode_split_kernel<DenseSrc<T>, GP, GH><<<dim3(S * (GP / GH), s.G, s.B), 256, 0, st>>>(
       src, c.bucket_count, qt, part, s, layer, S, 0);
-  decode_combine_kernel<T, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const T*)q, (const T*)basis_v,
+  decode_combine_kernel<T, GP><<<dim3(s.grp, s.G, s.B), kCombThreads, 0, st>>>(part, (const T*)q, (const T*)basis_v,
                                                                (const T*)tail_k, (const T*)tail_v,
                                                                n_tail, (T*)out, s, layer, S);
 }
@@ -472,7 +498,7 @@ void launch_decode_qt(const Shape& s, const varrate_qpacked& c, const void* basi
     decode_split_kernel<QuantSrc<8>, GP, GH><<<dim3(S * (GP / GH), s.G, s.B), 256, 0, st>>>(
         src, c.bucket_count, qt, part, s, layer, S, c.qcap_bytes);
   }
-  decode_combine_kernel<bf, GP><<<dim3(s.grp, s.G, s.B), 128, 0, st>>>(part, (const bf*)q, (const bf*)basis_v,
+  decode_combine_kernel<bf, GP><<<dim3(s.grp, s.G, s.B), kCombThreads, 0, st>>>(part, (const bf*)q, (const bf*)basis_v,
                                                                (const bf*)tail_k, (const bf*)tail_v,
                                                                n_tail, (bf*)out, s, layer, S);
 }

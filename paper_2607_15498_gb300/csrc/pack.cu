@@ -215,6 +215,7 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
   float* us = smem;                         // [128][kLd]  U rows
   float* xs = us + kHeadDim * kLd;          // [64][kLd]   gathered tokens, then coefficients
   __shared__ int stok[kTile], srk[kTile], spos[kTile];
+  __shared__ int s_ranks;                   // largest rank of the tile (its last valid slot's)
   __shared__ int n8s[kMaxR + 1];
   __shared__ long long bases[kMaxR + 2];
   const int64_t bl = blockIdx.z;
@@ -260,6 +261,7 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
         p = pos[bl * s.N + t];
       }
       stok[tid] = t; srk[tid] = r; spos[tid] = p;
+      if (sl < s_end && (sl + 1 == s_end || tid == kTile - 1)) s_ranks = r;
     }
     __syncthreads();
 #pragma unroll
@@ -270,11 +272,31 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
           t >= 0 ? load4(x + (int64_t)t * kHeadDim + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
+    const int nj = s_ranks;   // slots come in increasing rank: rows of U from nj on are not needed
     float acc[4][8];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
       for (int i = 0; i < 8; ++i) acc[a][i] = 0.f;
+    if (nj <= 32) {
+#pragma unroll 4
+      for (int c = 0; c < kHeadDim; c += 4) {
+        float4 xv[4], uv[2];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) xv[a] = *reinterpret_cast<const float4*>(&xs[(4 * ts + a) * kLd + c]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) uv[i] = *reinterpret_cast<const float4*>(&us[(tj + 16 * i) * kLd + c]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            acc[a][i] = fmaf(xv[a].x, uv[i].x, acc[a][i]);
+            acc[a][i] = fmaf(xv[a].y, uv[i].y, acc[a][i]);
+            acc[a][i] = fmaf(xv[a].z, uv[i].z, acc[a][i]);
+            acc[a][i] = fmaf(xv[a].w, uv[i].w, acc[a][i]);
+          }
+      }
+    } else
 #pragma unroll 4
     for (int c = 0; c < kHeadDim; c += 4) {
       float4 xv[4], uv[8];
@@ -298,7 +320,7 @@ project_kernel(const T* __restrict__ k, const T* __restrict__ v, const T* __rest
 #pragma unroll
       for (int i = 0; i < 8; ++i) xs[(4 * ts + a) * kLd + tj + 16 * i] = acc[a][i];
     __syncthreads();
-    for (int i = tid; i < kTile * kHeadDim; i += blockDim.x) {
+    for (int i = tid; i < kTile * nj; i += blockDim.x) {
       const int slot = i % kTile, j = i / kTile;
       const int r = srk[slot];
       if (stok[slot] >= 0 && j < r)

@@ -242,6 +242,22 @@ salience_accum_tc_kernel(const __grid_constant__ CUtensorMap tk, const __nv_bflo
       }
       *reinterpret_cast<uint4*>(qb + sw128_offset(row, cidx, npad)) = v;
     }
+    if (n_chunks <= 8) {   // few partials: a thread per row
+      for (int row = tid; row < npad; row += P2_EPI * 32) {
+        float2 x[8];
+        float mx = -INFINITY, l = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          x[c] = make_float2(-INFINITY, 0.f);
+          if (row < M && c < n_chunks) x[c] = stats[((bl * s.G + g) * M + row) * n_chunks + c];
+          mx = fmaxf(mx, x[c].x);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (x[c].x != -INFINITY) l += x[c].y * exp2f(x[c].x - mx);
+        sm.nlse[row] = row < M ? -(mx + log2f(l)) : -INFINITY;
+      }
+    } else
     // a warp per row, its lanes over the chunks' partials, the loads of eight rows in flight together
     for (int r0 = warp; r0 < npad; r0 += 8 * P2_EPI) {
       float2 x[8];
