@@ -823,7 +823,7 @@ bool helper_smem(int which, const void* fn, size_t bytes) {
   return true;
 }
 
-int window_rg(int ntt) { return ntt <= 2 ? 1 : (ntt <= 4 ? 2 : (ntt <= 8 ? 4 : 8)); }
+int window_rg(int ntt) { return ntt <= 2 ? 1 : (ntt <= 4 ? 2 : 8); }   // 8: decode_window_tc.cu
 
 }  // namespace
 
@@ -869,8 +869,7 @@ int launch_decode_window(const Shape& s, const varrate_packed& c, const void* ba
   switch (RG) {
     case 1: rc = launch_window_main<1>(s, c, qf, part, dev_status, layer, ntt, num_sms, st); break;
     case 2: rc = launch_window_main<2>(s, c, qf, part, dev_status, layer, ntt, num_sms, st); break;
-    case 4: rc = launch_window_main<4>(s, c, qf, part, dev_status, layer, ntt, num_sms, st); break;
-    default: rc = launch_window_main<8>(s, c, qf, part, dev_status, layer, ntt, num_sms, st); break;
+    default: rc = launch_window_tc(s, c, qf, part, dev_status, layer, ntt, num_sms, st); break;
   }
   if (rc < 0) return -1;
 
