@@ -359,7 +359,7 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
 // quarters of the block sum the splits, the basis rows and the tail tokens for all 128 coordinates, with
 // independent loads, and add up through shared memory in a fixed order. One CTA of 128 threads per KV head
 // that walked its heads and splits one after another took 110 us for 128 splits of 4 heads, a CTA of 128
-// threads per head 23 us, this FIGURES.
+// threads per head 23 us, this 19 us (cold).
 constexpr int kCombThreads = 512;
 constexpr int kCombParts = kCombThreads / kHeadDim;
 

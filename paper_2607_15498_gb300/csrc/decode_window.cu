@@ -24,8 +24,9 @@
 //     The teams' states merge in shared memory into one partial (m, l, o~[128]) per row, per
 //     (segment, CTA).
 //  3. window_combine_kernel: per (sequence, KV head) and 8 rows, merges the partials of the CTAs
-//     that shared the segment, adds the causal exact tail (scores and values in fp32 on CUDA
-//     cores, 64 tokens at a time, online), rotates o~ back with U_V^T and normalises.
+//     that shared the segment, adds the causal exact tail (on tensor cores, 128 tokens at a time,
+//     online), rotates o~ back with U_V^T and normalises.
+// More than 32 rows run decode_window_tc.cu in the place of the second kernel.
 //
 // Every bounded wait that gives up raises VARRATE_ERR_TIMEOUT; the CTA then streams nothing more,
 // writes empty partials and waits (bounded) for its copies in flight before it exits.
@@ -616,22 +617,30 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
 
 // ------------------------------------------------------------------ 3. combine
 
-constexpr int kTT = 64;                   // tail tokens per step
-constexpr int kKsStride = kHeadDim + 2;   // staged tail keys (odd word stride: no bank conflicts)
-constexpr int kCombRows = 8;              // query rows per combine CTA: one warp each
+constexpr int kTT = 128;                  // tail tokens per step: a 16-token tile per warp
+constexpr int kCombRows = 8;              // query rows per combine CTA
+constexpr int kRowStride = kHeadDim + 8;  // staged bf16 rows (272 bytes: ldmatrix without bank conflicts)
+constexpr int kWStride = kTT + 4;
 
 struct CombineSmem {
-  __nv_bfloat16 us[kHeadDim * kHeadDim];   // U_V[j][col]
-  __nv_bfloat16 ks[kTT * kKsStride];        // tail keys of the step
-  __nv_bfloat16 vs[kTT * kHeadDim];         // tail values of the step
-  float qs[kCombRows][kHeadDim];            // raw query rows (fp32)
-  float os[kCombRows][kHeadDim + 4];        // merged o~ per row
-  float ws[kCombRows][kTT];                 // tail weights of the step
+  alignas(16) __nv_bfloat16 us[kHeadDim * kRowStride];   // U_V[j][col]
+  alignas(16) __nv_bfloat16 ks[kTT * kRowStride];        // tail keys of the step
+  alignas(16) __nv_bfloat16 vs[kTT * kRowStride];        // tail values of the step
+  alignas(16) float os[kCombRows][kHeadDim + 8];         // merged o~ per row
+  float ws[kCombRows][kWStride];                         // tail scores, then tail weights, of the step
+  float fs[kCombRows];                                   // factor of the rows' earlier sums
+  float ls[kCombRows];                                   // softmax normaliser
 };
 
-// grid (B G, ceil(R / 8)), 256 threads: warp w owns row rho = 8 blockIdx.y + w, lane l its columns
-// l + 32 k (k < 4) and, per step of 64 tail tokens, tokens l and l + 32. part slots as written
-// above; out is [B][n_q][H][d].
+// grid (B G, ceil(R / 8)), 256 threads: rows 8 blockIdx.y .. + 7 of one (sequence, KV head). part slots as
+// written above; out is [B][n_q][H][d]. Warp w merges the partials of row w: the maxima and sums one CTA a
+// lane, then the weighted sums with eight 16-byte loads in flight. The tail goes 128 tokens at a time, on
+// tensor cores: scores as m16n8k16 tiles (16 tokens x 8 rows, exact bf16 products, fp32 sums) with the causal
+// cut, the online softmax by row, values as further k-steps of the rotation back,
+//   out^T[col][row] = sum_j U_V[j][col] o~[row][j] + sum_t v_t[col] w[row][t],
+// warp w owning columns 16 w .. 16 w + 15, with o~ and w split hi + lo in bf16. Bound by latency.
+// 8 heads, 19 partials a row: 128 rows and 32 tail tokens 27 us with scalar loops over partials, tail and
+// basis rows, 12 us now; 32 rows and 300 tail tokens 67 / 15 us.
 __global__ void __launch_bounds__(256)
 window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict__ bucket_base,
                       const __nv_bfloat16* __restrict__ basis_v, const __nv_bfloat16* __restrict__ q,
@@ -642,142 +651,188 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
   CombineSmem& cs = *reinterpret_cast<CombineSmem*>(smem_c);
   __shared__ long long segW[64];
   __shared__ long long segP[65];
-  const int tid = threadIdx.x, lr = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, c = lane & 3;
   const long long seg = blockIdx.x;
   const int b = (int)(seg / s.G), g = (int)(seg % s.G);
-  const int R = n_q * s.grp, rows = 8 * ntt;
-  const int rho = kCombRows * blockIdx.y + lr;
-  const bool valid = rho < R;
-  const int iq = valid ? rho / s.grp : 0, h = valid ? rho % s.grp : 0;
-  pdl_trigger();
-  pdl_wait();
-  // U_V of the head (eight 16-byte loads per thread, all in flight) and the query rows
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(basis_v + ((long long)layer * s.G + g) * kHeadDim * kHeadDim);
-    uint4* dst = reinterpret_cast<uint4*>(cs.us);
-    uint4 v[kHeadDim * kHeadDim / 8 / 256];
-#pragma unroll
-    for (int k = 0; k < kHeadDim * kHeadDim / 8 / 256; ++k) v[k] = __ldg(src + tid + 256 * k);
-#pragma unroll
-    for (int k = 0; k < kHeadDim * kHeadDim / 8 / 256; ++k) dst[tid + 256 * k] = v[k];
-    const __nv_bfloat16* qr = q + (((long long)b * n_q + iq) * s.H + (long long)g * s.grp + h) * kHeadDim;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) cs.qs[lr][lane + 32 * k] = valid ? __bfloat162float(qr[lane + 32 * k]) : 0.f;
-  }
-  seg_lengths(bucket_base, s, layer, segW, segP, tid);
-  // merge the partials of the CTAs that shared the segment: the common maximum first, then the
-  // weighted sums (independent loads, four partials at a time)
-  float M = -INFINITY, L = 0.f, o[4], ov[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) { o[k] = 0.f; ov[k] = 0.f; }
-  const long long W = segW[b];
-  if (W > 0 && valid) {
-    const long long T = segP[64];
-    const long long P = segP[b] + g * (W + kSegCost + kSegEnd) + kSegCost;
-    int c0, c1;
-    seg_cta_range([&](int i) { return cut_at(T, i, C); }, T, C, P, W, c0, c1);
-    const float* pr = part + ((c0 + seg) * (long long)rows + rho) * kPartStride;
-    const long long pstride = (long long)rows * kPartStride;
-    const int np = c1 - c0 + 1;
-#pragma unroll 4
-    for (int p = 0; p < np; ++p) M = fmaxf(M, __ldcg(pr + p * pstride + kHeadDim));
-    if (M != -INFINITY) {
-#pragma unroll 4
-      for (int p = 0; p < np; ++p) {
-        const float* pp = pr + p * pstride;
-        const float mp = __ldcg(pp + kHeadDim);
-        const float w = mp == -INFINITY ? 0.f : exp2f(mp - M);
-        L = fmaf(w, __ldcg(pp + kHeadDim + 1), L);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) o[k] = fmaf(w, __ldcg(pp + lane + 32 * k), o[k]);
-      }
-    }
-  }
-  // exact tail, causal: row rho (query iq) sees tail tokens t < n_tail - n_q + iq + 1
-  const int vis = n_tail - n_q + iq + 1;
-  const int last_row = min(R, kCombRows * (int)blockIdx.y + kCombRows) - 1;
-  const int vis_max = n_tail - n_q + last_row / s.grp + 1;   // block-uniform
-  const float scale = kLog2e * rsqrtf((float)kHeadDim);
+  const int R = n_q * s.grp, rows = 8 * ntt, row0 = kCombRows * blockIdx.y;
   const __nv_bfloat16* tk = tail_k + ((long long)b * s.G + g) * n_tail * kHeadDim;
   const __nv_bfloat16* tv = tail_v + ((long long)b * s.G + g) * n_tail * kHeadDim;
-  for (int t0 = 0; t0 < vis_max; t0 += kTT) {
-    __syncthreads();   // previous step's readers of ks / vs (and the loads above) are done
-    for (int e = tid; e < kTT * kHeadDim / 2; e += blockDim.x) {
-      const int t = e / (kHeadDim / 2), i2 = e % (kHeadDim / 2);
-      uint32_t kx = 0u, vx = 0u;
-      if (t0 + t < n_tail) {
-        kx = reinterpret_cast<const uint32_t*>(tk + (long long)(t0 + t) * kHeadDim)[i2];
-        vx = reinterpret_cast<const uint32_t*>(tv + (long long)(t0 + t) * kHeadDim)[i2];
+  pdl_trigger();
+  pdl_wait();
+  // stage `n` 256-byte rows (the rest of `cap` rows as zeros)
+  auto stage = [&](__nv_bfloat16* dst, const __nv_bfloat16* src, int n, int cap) {
+    for (int i = tid; i < cap * 16; i += 256) {
+      const int r = i >> 4, ch = i & 15;
+      const bool in = r < n;
+      cp_async16(smem_addr(dst + r * kRowStride + ch * 8), src + (in ? (long long)r * kHeadDim + ch * 8 : 0), in ? 16 : 0);
+    }
+  };
+  const int last_row = min(R, row0 + kCombRows) - 1;
+  const int vis_max = n_tail - n_q + last_row / s.grp + 1;   // tail tokens some row of the CTA sees
+  stage(cs.us, basis_v + ((long long)layer * s.G + g) * kHeadDim * kHeadDim, kHeadDim, kHeadDim);
+  {
+    const int n = min(kTT, vis_max);
+    stage(cs.ks, tk, n, (n + 15) & ~15);
+    stage(cs.vs, tv, n, (n + 15) & ~15);
+  }
+  cp_async_commit();
+  // query fragments of the tail scores: B[k][n] = q[row n][k]
+  uint32_t qb[kHeadDim / 16][2];
+  {
+    const int rho = min(row0 + g8, R - 1);
+    const __nv_bfloat16* qr = q + (((long long)b * n_q + rho / s.grp) * s.H + (long long)g * s.grp + rho % s.grp) * kHeadDim + 2 * c;
+#pragma unroll
+    for (int ks = 0; ks < kHeadDim / 16; ++ks) {
+      qb[ks][0] = __ldg(reinterpret_cast<const uint32_t*>(qr + 16 * ks));
+      qb[ks][1] = __ldg(reinterpret_cast<const uint32_t*>(qr + 16 * ks + 8));
+    }
+  }
+  seg_lengths(bucket_base, s, layer, segW, segP, tid);
+  // row of this warp (merge and softmax): the partials of the CTAs that shared the segment
+  const int rho = row0 + warp;
+  const bool valid = rho < R;
+  const int vis = valid ? n_tail - n_q + rho / s.grp + 1 : 0;   // causal: tail tokens t < vis
+  float M = -INFINITY, L = 0.f;
+  {
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    const long long W = segW[b];
+    if (W > 0 && valid) {
+      const long long T = segP[64];
+      const long long P = segP[b] + g * (W + kSegCost + kSegEnd) + kSegCost;
+      int c0, c1;
+      seg_cta_range([&](int i) { return cut_at(T, i, C); }, T, C, P, W, c0, c1);
+      const float* pr = part + ((c0 + seg) * (long long)rows + rho) * kPartStride;
+      const long long pstride = (long long)rows * kPartStride;
+      const int np = c1 - c0 + 1;
+      for (int p0 = 0; p0 < np; p0 += 32) {   // the same order for every row: first to last
+        float m = -INFINITY, l = 0.f;
+        if (p0 + lane < np) {
+          m = __ldcg(pr + (p0 + lane) * pstride + kHeadDim);
+          l = __ldcg(pr + (p0 + lane) * pstride + kHeadDim + 1);
+        }
+        float mx = m;
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+        mx = fmaxf(mx, M);
+        if (mx == -INFINITY) continue;
+        const float f = M == -INFINITY ? 0.f : exp2f(M - mx), w = m == -INFINITY ? 0.f : exp2f(m - mx);
+        float lw = l * w;
+#pragma unroll
+        for (int x = 16; x > 0; x >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, x);
+        L = L * f + lw;
+        o.x *= f; o.y *= f; o.z *= f; o.w *= f;
+        M = mx;
+        const int n = min(32, np - p0);
+        for (int k0 = 0; k0 < n; k0 += 8) {
+          float4 v[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (k0 + k < n) v[k] = __ldcg(reinterpret_cast<const float4*>(pr + (p0 + k0 + k) * pstride) + lane);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float wk = __shfl_sync(0xffffffffu, w, (k0 + k) & 31);
+            if (k0 + k < n) {
+              o.x = fmaf(wk, v[k].x, o.x); o.y = fmaf(wk, v[k].y, o.y);
+              o.z = fmaf(wk, v[k].z, o.z); o.w = fmaf(wk, v[k].w, o.w);
+            }
+          }
+        }
       }
-      reinterpret_cast<uint32_t*>(cs.ks + t * kKsStride)[i2] = kx;
-      reinterpret_cast<uint32_t*>(cs.vs + t * kHeadDim)[i2] = vx;
+    }
+    *reinterpret_cast<float4*>(&cs.os[warp][4 * lane]) = o;
+  }
+  const float M0 = M;
+  const float scale = kLog2e * rsqrtf((float)kHeadDim);
+  const int col0 = warp * 16, col = col0 + ((lane >> 3) & 1) * 8, jr = (lane & 7) + ((lane >> 4) & 1) * 8;
+  float d[2][4] = {};   // this warp's 16 columns x 8 rows: sums with the hi and with the lo parts
+  for (int t0 = 0; t0 < vis_max; t0 += kTT) {
+    cp_async_wait<0>();
+    __syncthreads();
+    const int n = min(kTT, vis_max - t0);
+    if (warp * 16 < n) {   // scores of 16 tokens (warp-uniform)
+      float sc[4] = {0.f, 0.f, 0.f, 0.f};
+      const int tr = warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
+#pragma unroll
+      for (int ks = 0; ks < kHeadDim / 16; ++ks) {
+        uint32_t a[4];
+        ldsm_x4(smem_addr(&cs.ks[tr * kRowStride + ks * 16 + (lane >> 4) * 8]), a);
+        mma_bf16_16816(sc, a, qb[ks][0], qb[ks][1]);
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) cs.ws[2 * c + (e & 1)][warp * 16 + g8 + (e >> 1) * 8] = sc[e] * scale;
     }
     __syncthreads();
-    float sc[2] = {0.f, 0.f};
-    for (int i = 0; i < kHeadDim; i += 2) {
-      const float2 qv = *reinterpret_cast<const float2*>(&cs.qs[lr][i]);
+    {   // online softmax of this warp's row
+      float x[kTT / 32], tm = -INFINITY;
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const __nv_bfloat162 kk = *reinterpret_cast<const __nv_bfloat162*>(cs.ks + (lane + 32 * k) * kKsStride + i);
-        sc[k] = fmaf(qv.x, __low2float(kk), fmaf(qv.y, __high2float(kk), sc[k]));
+      for (int k = 0; k < kTT / 32; ++k) {
+        const int t = lane + 32 * k;
+        x[k] = t0 + t < vis ? cs.ws[warp][t] : -INFINITY;
+        tm = fmaxf(tm, x[k]);
       }
-    }
-    float tm = -INFINITY;
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int t = t0 + lane + 32 * k;
-      sc[k] = (valid && t < vis) ? sc[k] * scale : -INFINITY;
-      tm = fmaxf(tm, sc[k]);
-    }
+      for (int o = 16; o > 0; o >>= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, o));
+      const float nm = fmaxf(M, tm);
+      float lt = 0.f;
 #pragma unroll
-    for (int x = 1; x < 32; x <<= 1) tm = fmaxf(tm, __shfl_xor_sync(0xffffffffu, tm, x));
-    const float nm = fmaxf(M, tm);
-    float lt = 0.f;
-    if (nm != -INFINITY) {
-      const float f = M == -INFINITY ? 0.f : exp2f(M - nm);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) { o[k] *= f; ov[k] *= f; }
-      L *= f;
-      M = nm;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const float w = sc[k] == -INFINITY ? 0.f : exp2f(sc[k] - nm);
-        cs.ws[lr][lane + 32 * k] = w;
+      for (int k = 0; k < kTT / 32; ++k) {
+        const float w = x[k] == -INFINITY ? 0.f : exp2f(x[k] - nm);
+        cs.ws[warp][lane + 32 * k] = w;
         lt += w;
       }
-    } else {
 #pragma unroll
-      for (int k = 0; k < 2; ++k) cs.ws[lr][lane + 32 * k] = 0.f;
+      for (int o = 16; o > 0; o >>= 1) lt += __shfl_xor_sync(0xffffffffu, lt, o);
+      const float f = M == -INFINITY ? 0.f : exp2f(M - nm);
+      L = L * f + lt;
+      M = nm;
+      if (lane == 0) cs.fs[warp] = f;
     }
+    __syncthreads();
+    {   // values: 16 tokens per k-step
+      const float f0 = cs.fs[2 * c], f1 = cs.fs[2 * c + 1];
 #pragma unroll
-    for (int x = 1; x < 32; x <<= 1) lt += __shfl_xor_sync(0xffffffffu, lt, x);
-    L += lt;
-    __syncwarp();   // the row's weights were written by this warp
-#pragma unroll 4
-    for (int t = 0; t < kTT; ++t) {
-      const float w = cs.ws[lr][t];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) ov[k] = fmaf(w, __bfloat162float(cs.vs[t * kHeadDim + lane + 32 * k]), ov[k]);
+      for (int h = 0; h < 2; ++h) { d[h][0] *= f0; d[h][1] *= f1; d[h][2] *= f0; d[h][3] *= f1; }
+      for (int ts = 0; ts < (n + 15) / 16; ++ts) {
+        uint32_t a[4], h0, l0, h1, l1;
+        ldsm_x4_trans(smem_addr(&cs.vs[(ts * 16 + jr) * kRowStride + col]), a);
+        const int tb = ts * 16 + 2 * c;
+        split_bf16(cs.ws[g8][tb], cs.ws[g8][tb + 1], h0, l0);
+        split_bf16(cs.ws[g8][tb + 8], cs.ws[g8][tb + 9], h1, l1);
+        mma_bf16_16816(d[0], a, h0, h1);
+        mma_bf16_16816(d[1], a, l0, l1);
+      }
+    }
+    if (t0 + kTT < vis_max) {
+      __syncthreads();   // every reader of the staged tokens and weights is done
+      const int m = min(kTT, vis_max - t0 - kTT);
+      stage(cs.ks, tk + (long long)(t0 + kTT) * kHeadDim, m, (m + 15) & ~15);
+      stage(cs.vs, tv + (long long)(t0 + kTT) * kHeadDim, m, (m + 15) & ~15);
+      cp_async_commit();
     }
   }
-  // rotate the coded part back: out[col] = sum_j U_V[j][col] o~[j] + tail values, over l
-#pragma unroll
-  for (int k = 0; k < 4; ++k) cs.os[lr][lane + 32 * k] = o[k];
+  cp_async_wait<0>();
+  if (lane == 0) {
+    cs.fs[warp] = M0 == -INFINITY ? 0.f : exp2f(M0 - M);   // o~ against the final reference
+    cs.ls[warp] = L;
+  }
   __syncthreads();
-  float y[4];
+  const float fr = cs.fs[g8];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) y[k] = ov[k];
-#pragma unroll 4
-  for (int j = 0; j < kHeadDim; ++j) {
-    const float oj = cs.os[lr][j];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) y[k] = fmaf(__bfloat162float(cs.us[j * kHeadDim + lane + 32 * k]), oj, y[k]);
+  for (int ks = 0; ks < kHeadDim / 16; ++ks) {
+    uint32_t a[4], h0, l0, h1, l1;
+    ldsm_x4_trans(smem_addr(&cs.us[(ks * 16 + jr) * kRowStride + col]), a);
+    const int jb = ks * 16 + 2 * c;
+    split_bf16(cs.os[g8][jb] * fr, cs.os[g8][jb + 1] * fr, h0, l0);
+    split_bf16(cs.os[g8][jb + 8] * fr, cs.os[g8][jb + 9] * fr, h1, l1);
+    mma_bf16_16816(d[0], a, h0, h1);
+    mma_bf16_16816(d[1], a, l0, l1);
   }
-  if (valid) {
-    __nv_bfloat16* dst = out + (((long long)b * n_q + iq) * s.H + (long long)g * s.grp + h) * kHeadDim;
-    const float inv = 1.f / L;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) dst[lane + 32 * k] = __float2bfloat16_rn(y[k] * inv);
+  for (int e = 0; e < 4; ++e) {   // columns col0 + g8 (+ 8), rows 2c, 2c + 1
+    const int lr = 2 * c + (e & 1), r = row0 + lr;
+    if (r < R)
+      out[(((long long)b * n_q + r / s.grp) * s.H + (long long)g * s.grp + r % s.grp) * kHeadDim + col0 + g8 + (e >> 1) * 8] =
+          __float2bfloat16_rn((d[0][e] + d[1][e]) / cs.ls[lr]);
   }
 }
 
