@@ -115,8 +115,8 @@ __device__ __noinline__ void build_qfrag_f16(SegSmem& sm, int tid) {
 // tile and bucket start). Returns false (and issues nothing) when the stream is exhausted.
 template <int BITS>
 __device__ __forceinline__ bool issue_chunk_q(Prod& p, const SegSmem& sm, const uint8_t* cK, const uint8_t* cV,
-                                              uint32_t stage_addr, uint64_t* bar, int total, int lane,
-                                              uint64_t policy) {
+                                              uint32_t stage_addr, uint64_t* bar, int total, int n_long,
+                                              int lane, uint64_t policy) {
   if (p.k >= total) return false;
   const int r = p.item.r;
   const long long n8 = pad8(sm.cnt[r]);
@@ -140,7 +140,7 @@ __device__ __forceinline__ bool issue_chunk_q(Prod& p, const SegSmem& sm, const 
     if (++p.phase == 2) {
       p.phase = 0;
       p.k += NW;
-      if (p.k < total) p.item = next_rr<NW>(sm, p.item, p.k);
+      if (p.k < total) p.item = next_rr_split<NW>(sm, p.item, p.k, n_long);
     }
   }
   return true;
@@ -187,13 +187,33 @@ __device__ __forceinline__ uint4 expand8(uint32_t w0, uint32_t w1, __half2 lo2, 
   return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// Expansion of a tile of fewer than 128 slots, group by group; out of line, so that the main loop's code (with
+// nine copies of dequant_chunk) stays small.
+template <int BITS>
+__device__ __noinline__ void dequant_short(uint32_t src, uint32_t dst, int rows, int j0, int tl, int lane) {
+  const int ng = tl >> 3, qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
+  for (int jr = lane; jr < rows; jr += 32) {
+    const uint32_t row = src + jr * qrow, orow = dst + jr * (tl * 2);
+    int pos = (j0 + jr) % ng;
+    for (int gi = 0; gi < ng; ++gi) {
+      const uint32_t pq = ld_shared_u32(row + pbase + 4 * (gi >> 2));
+      const __half2 ph = *reinterpret_cast<const __half2*>(&pq);
+      const __half2 lo2 = __low2half2(ph), st2 = __high2half2(ph);
+      const uint32_t w0 = ld_shared_u32(row + (BITS == 4 ? 4 : 8) * gi);
+      const uint32_t w1 = BITS == 8 ? ld_shared_u32(row + 8 * gi + 4) : 0u;
+      st_shared_v4(orow + 16 * pos, expand8(w0, w1, lo2, st2, BITS));
+      pos = pos + 1 == ng ? 0 : pos + 1;
+    }
+  }
+}
+
 // Expand `rows` staged quantized rows (tile rows j0 .., tl slots) into fp16 rows at `dst` in the
 // packed layout's order (group g of tile row j at position (g + j) mod (tl / 8)). Lane l takes rows
 // l, l + 32, ...; a full 4-bit row is five 16-byte loads (codes, then the four (lo, step) pairs)
 // and sixteen 16-byte stores, whose banks the row stride (80 bytes) and the rotation spread.
 template <int BITS>
 __device__ __forceinline__ void dequant_chunk(uint32_t src, uint32_t dst, int rows, int j0, int tl, int lane) {
-  const int ng = tl >> 3, qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
+  const int qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
   if (tl == ISL) {   // warp-uniform: full tile, 16-byte loads of four groups' codes at a time
     for (int jr = lane; jr < rows; jr += 32) {
       const uint32_t row = src + jr * qrow, orow = dst + jr * (ISL * 2);
@@ -220,20 +240,8 @@ __device__ __forceinline__ void dequant_chunk(uint32_t src, uint32_t dst, int ro
         }
       }
     }
-  } else {           // a short tile: group by group
-    for (int jr = lane; jr < rows; jr += 32) {
-      const uint32_t row = src + jr * qrow, orow = dst + jr * (tl * 2);
-      const int j = j0 + jr;
-      for (int gi = 0; gi < ng; ++gi) {
-        const uint32_t pq = ld_shared_u32(row + pbase + 4 * (gi >> 2));
-        const __half2 ph = *reinterpret_cast<const __half2*>(&pq);
-        const __half2 lo2 = __low2half2(ph), st2 = __high2half2(ph);
-        const uint32_t w0 = ld_shared_u32(row + (BITS == 4 ? 4 : 8) * gi);
-        const uint32_t w1 = BITS == 8 ? ld_shared_u32(row + 8 * gi + 4) : 0u;
-        const uint4 v = expand8(w0, w1, lo2, st2, BITS);
-        st_shared_v4(orow + 16 * ((gi + j) % ng), v);
-      }
-    }
+  } else {
+    dequant_short<BITS>(src, dst, rows, j0, tl, lane);
   }
 }
 
@@ -370,7 +378,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         long long i0 = 0, i1 = 0;
         if (r >= s.r_min && r <= s.r_max) bucket_range_q<BITS>(sm, r, lo, hi, i0, i1);
         sm.it_lo[r] = (int)i0;
-        sm.it_pref[r + 1] = (int)(i1 - i0);   // counts first, prefixed below
+        sm.it_pref[r + 1] = (int)split_count(i0, i1, sm.cnt[r]);   // counts first, prefixed below
       }
       __syncthreads();
       if (warp == 0) {   // inclusive scan of it_pref[1 .. 129], 5 entries per lane
@@ -410,16 +418,18 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
 #pragma unroll
       for (int t = 0; t < kHeadDim / 16; ++t) oacc[t][0] = oacc[t][1] = oacc[t][2] = oacc[t][3] = 0.f;
 
-      const int total = dead ? 0 : sm.it_pref[kMaxR + 1];
+      // long items first, then the short ones: every warp takes both in turn
+      const int n_long = dead ? 0 : (int)((uint32_t)sm.it_pref[kMaxR + 1] & kLongMask);
+      const int total = dead ? 0 : n_long + (int)((uint32_t)sm.it_pref[kMaxR + 1] >> 24);
       Prod pr;
       pr.k = warp; pr.phase = 0; pr.jc = 0;
-      if (pr.k < total) pr.item = item_at(sm, pr.k);
+      if (pr.k < total) pr.item = item_at_split(sm, pr.k, n_long);
       int cons_k = pr.k;
       Item cons = pr.item;
 #pragma unroll
       for (int i = 0; i < ST; ++i)   // every stage of the ring in flight
         if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + i) % ST) * STQ,
-                        &bars[(n_issued + i) % ST], total, lane, policy)) ++n_pending;
+                        &bars[(n_issued + i) % ST], total, n_long, lane, policy)) ++n_pending;
       int c0, c1;   // the CTAs that share this segment (their partials are merged by the last one)
       seg_cta_range([&](int i) { return cuts[i]; }, T, C, P, W, c0, c1);
       __syncwarp();
@@ -441,10 +451,10 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         ++n_issued;
         --n_pending;
         if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + ST - 1) % ST) * STQ,
-                        &bars[(n_issued + ST - 1) % ST], total, lane, policy)) ++n_pending;
+                        &bars[(n_issued + ST - 1) % ST], total, n_long, lane, policy)) ++n_pending;
       };
 
-      while (cons_k < total && !timed_out) {
+      while (cons_k < n_long && !timed_out) {
         const int r = cons.r;
         const long long n_real = sm.cnt[r] - (long long)cons.it * ISL;   // real slots of this item
         // tile geometry (packed layout, coef_offset): rows of tl slots, 8-slot group g of row j
@@ -614,7 +624,113 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
           __syncwarp();   // the staged rows are read before the next item's first chunk
         }
         cons_k += NW;
-        if (cons_k < total) cons = next_rr<NW>(sm, cons, cons_k);
+        if (cons_k < total) cons = next_rr_split<NW>(sm, cons, cons_k, n_long);
+      }
+      // Short items (at most kShort slots): the same steps on two 16-slot tiles instead of eight, in a loop of
+      // their own as in decode_mma.cu (one chunk each of K and V rows, at 8 bits two past 64 rows). Before / with
+      // it and the out-of-line expansion of short tiles, us per call: 1 sequence, 8 bits, wide ranks 57 / 39; 4
+      // sequences, 4 bits, spread ranks 79 / 67; 8 sequences, 4 bits, nearly equal ranks 85 / 84 (90 with the
+      // expansion inlined nine times: the main loop is held by its code's size).
+      while (cons_k < total && !timed_out) {
+        const int r = cons.r;
+        const int n_real = sm.cnt[r] - cons.it * ISL, tl = (n_real + 7) & ~7, ng = tl >> 3;
+        const uint32_t row_bytes = (uint32_t)tl * 2u;
+        const int lgc = chunk_lg_q(tl, BITS);
+        const int m = lane >> 3, r8 = lane & 7;
+        float sh[2][4] = {}, sl[2][4] = {};
+        for (int j0 = 0; j0 < r; j0 += 1 << lgc) {
+          if (!wait_chunk()) break;
+          const int j1 = min(r, j0 + (1 << lgc));
+          dequant_short<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, j1 - j0, j0, tl, lane);
+          __syncwarp();
+          next_chunk();
+          for (int j16 = j0; j16 < j1; j16 += 16) {
+            const uint4 qf = *reinterpret_cast<const uint4*>(&sm.qfrag[j16 >> 4][lane][0]);
+            const int jrow = (j16 - j0) + (m >> 1) * 8 + r8;
+            const uint32_t row_addr = stg_w + jrow * row_bytes;
+            const int pg = ((m & 1) + j0 + jrow) % ng;
+            uint32_t a[2][4];
+            ldsm_x4_trans(row_addr + 16 * pg, a[0]);
+            ldsm_x4_trans(row_addr + 16 * wrap2(pg, ng), a[1]);
+            if (j16 + 16 > r) {
+              const int jb = j16 + 2 * c;
+              const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
+#pragma unroll
+              for (int mt = 0; mt < 2; ++mt) { a[mt][0] &= m0; a[mt][1] &= m0; a[mt][2] &= m1; a[mt][3] &= m1; }
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+              mma_f16_16816(sh[mt], a[mt], qf.x, qf.y);
+              mma_f16_16816(sl[mt], a[mt], qf.z, qf.w);
+            }
+          }
+          __syncwarp();   // every lane has read the staged rows before the next chunk replaces them
+        }
+        if (timed_out) break;
+        float mloc[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+          const int s0 = mt * 16 + (BITS == 4 ? (g8 >> 1) + 4 * (g8 & 1) : g8);   // the slot at stored position g8
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sh[mt][e] = s0 + (e >> 1) * 8 < n_real ? sh[mt][e] + sl[mt][e] : -INFINITY;
+          mloc[0] = fmaxf(mloc[0], fmaxf(sh[mt][0], sh[mt][2]));
+          mloc[1] = fmaxf(mloc[1], fmaxf(sh[mt][1], sh[mt][3]));
+        }
+        if (!__all_sync(0xffffffffu, mloc[0] <= Mx[0] + kSlack && mloc[1] <= Mx[1] + kSlack)) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) mloc[e] = fmaxf(mloc[e], __shfl_xor_sync(0xffffffffu, mloc[e], o));
+            const float nm = fmaxf(Mx[e], mloc[e]);
+            const float corr = fast_exp2(Mx[e] - nm);
+            Mx[e] = nm;
+            Ls[e] *= corr;
+#pragma unroll
+            for (int t = 0; t < kHeadDim / 16; ++t) { oacc[t][e] *= corr; oacc[t][e + 2] *= corr; }
+          }
+        }
+        const float Mr[2] = {Mx[0] - kPShift, Mx[1] - kPShift};   // weights scaled by 2^kPShift
+        uint32_t pb[2][2];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+          const float p0 = fast_exp2(sh[mt][0] - Mr[0]), p1 = fast_exp2(sh[mt][1] - Mr[1]);
+          const float p2 = fast_exp2(sh[mt][2] - Mr[0]), p3 = fast_exp2(sh[mt][3] - Mr[1]);
+          Ls[0] += p0 + p2;
+          Ls[1] += p1 + p3;
+          pb[mt][0] = movmatrix_trans(pack_f16(p0, p1));
+          pb[mt][1] = movmatrix_trans(pack_f16(p2, p3));
+        }
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {                 // 64 rows: one chunk of 8-bit rows, half a chunk of 4-bit rows
+          if (hf * 64 >= r) break;                       // warp-uniform
+          const int j0 = lgc == 6 ? hf * 64 : 0;         // first staged row
+          if (hf == 0 || lgc == 6) {
+            __syncwarp();
+            if (!wait_chunk()) break;
+            dequant_short<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, min(r - j0, 1 << lgc), j0, tl, lane);
+            __syncwarp();
+            next_chunk();
+          }
+#pragma unroll
+          for (int jt = 4 * hf; jt < 4 * hf + 4; ++jt) {
+            if (jt * 16 >= r) break;
+            const int jrow = (jt * 16 - j0) + (m & 1) * 8 + r8;
+            const uint32_t row_addr = stg_w + jrow * row_bytes;
+            const int pg = ((m >> 1) + j0 + jrow) % ng;
+            uint32_t a[4], b2[4];
+            ldsm_x4(row_addr + 16 * pg, a);
+            ldsm_x4(row_addr + 16 * wrap2(pg, ng), b2);
+            if (jt * 16 + 16 > r) {
+              if (jt * 16 + g8 >= r) { a[0] = a[2] = 0u; b2[0] = b2[2] = 0u; }
+              if (jt * 16 + g8 + 8 >= r) { a[1] = a[3] = 0u; b2[1] = b2[3] = 0u; }
+            }
+            mma_f16_16816(oacc[jt], a, pb[0][0], pb[0][1]);
+            mma_f16_16816(oacc[jt], b2, pb[1][0], pb[1][1]);
+          }
+        }
+        __syncwarp();   // the staged rows are read before the next item's first chunk
+        cons_k += NW;
+        if (cons_k < total) cons = next_rr_split<NW>(sm, cons, cons_k, n_long);
       }
       // drain: never leave bulk copies in flight into this ring (a copy whose wait gave up stays
       // counted in n_pending and is waited for once more before the CTA exits)

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_helpers import O, V, cfg_for, decode_close, decode_errors, f64, gpu_decode, gpu_pack, synth
+from gpu_helpers import O, V, cfg_for, decode_close, decode_errors, f64, gpu_decode, gpu_pack, synth, unpack
 
 pytestmark = pytest.mark.gpu
 
@@ -71,3 +71,30 @@ def test_window_wide_ranks(kind, n, grp, n_q, n_tail):
     got = f64(out)[0]
     for i in range(n_q):
         assert decode_close(got[i], want[i], cfg), (i, decode_errors(got[i], want[i]))
+
+
+@pytest.mark.parametrize("bits, grp, n_tail", [(4, 4, 0), (8, 4, 3), (4, 7, 40), (8, 1, 0)])
+@pytest.mark.parametrize("kind, n", [("wide", 2500), ("edges", 1500), ("ends", 900)])
+def test_decode_quantized_wide_ranks(kind, n, bits, grp, n_tail):
+    """The stored bf16 coefficients are read back, so that both sides quantize the same values."""
+    wl, cfg, packed, bk, bv, _, _, ranks = _cache(kind, n, grp)
+    count, base, pos, _ = O.pack_tables(ranks, 16, 128)
+    stored = [[unpack(packed, 0, 0, g, kv, ranks, count, base, pos) for g in range(2)] for kv in range(2)]
+    ck, cv = (np.stack([O.quantize_coefficients(x.astype(np.float32), ranks, count, pos, bits)[3] for x in side])
+              for side in stored)
+    qp = V.QPackedCache.allocate(cfg, packed, bits)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    V.check(V.varrate_quantize(cfg, packed, qp, status), "varrate_quantize")
+    q = synth.stack_decode_queries(wl, 0, 1)[0]
+    gen = torch.Generator().manual_seed(n_tail)
+    tk, tv = (torch.randn((1, 2, n_tail, 128), generator=gen).to(torch.bfloat16) for _ in range(2))
+    out = torch.empty_like(q, device="cuda")
+    V.check(V.varrate_decode_attn_q(cfg, qp, bk.cuda(), bv.cuda(), q.cuda(), 0, tk.cuda() if n_tail else None,
+                                    tv.cuda() if n_tail else None, n_tail, out, status,
+                                    V.workspace(cfg, V.CALL_DECODE_Q)), "varrate_decode_attn_q")
+    torch.cuda.synchronize()
+    assert int(status.item()) == V.OK
+    want = O.decode_coef(f64(q[0]), ck.astype(np.float64), cv.astype(np.float64), ranks, f64(bk[0]), f64(bv[0]),
+                         *((f64(tk[0]), f64(tv[0])) if n_tail else ()))
+    got = f64(out)[0]
+    assert decode_close(got, want, cfg), decode_errors(got, want)
