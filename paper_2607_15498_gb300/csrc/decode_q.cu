@@ -9,16 +9,23 @@
 //    from the bf16 ones by the bytes of a 128-slot row (qrow(128) per 128 elements), and an item of
 //    rank r spans r * qrow(128) bytes.
 //  - A chunk is a run of quantized rows of one tile (qrow(tl) bytes each: the codes, then (fp16 lo,
-//    fp16 step) per 32-slot group), one 1-D bulk copy into a 4 KB ring stage. Once it lands, the
-//    warp expands it, one row per lane, into its own 8 KB staging buffer as fp16 rows laid out like
-//    the bf16 packed layout (8-slot group g of row j at position (g + j) mod (tl / 8); at 4 bits the
-//    slots inside a group in the order 0 4 1 5 2 6 3 7, see expand8), refills the stage at once and
-//    computes from the staging rows with the bf16 kernel's fragment code.
-//  - Expansion in fp16 half2 arithmetic: a code becomes the fp16 value 1024 + code by a byte
-//    permute and a mask (the exponent of 1024 put above it), 1024 is subtracted exactly, and
-//    code * step + lo is one fused multiply-add rounded once to fp16 (the format's lo and step are
-//    fp16 already); x^ = lo + code * step of the format is therefore held to within an fp16
-//    rounding, finer than the bf16 rounding of the bf16 path.
+//    fp16 step) per 32-slot group), one 1-D bulk copy into a ring stage. The codes become the
+//    tensor-core fragments in registers, straight from the stage: nothing ties the order in which the
+//    MMAs take a tile's slots to the order in memory, so each lane takes runs of slots. For the scores
+//    (m = slots, k = rows) lane group g8 has slots 16 g8 .. 16 g8 + 15 of the lane's four rows, and a
+//    byte permute pairs the codes of two rows; for the output (m = rows, k = slots) lane c has the 32
+//    slots of group c of its two rows, and the pairs are 16 slots apart, which is where the scores'
+//    fragments leave the weights of those slots.
+//  - Expansion in fp16 half2 arithmetic: a code becomes the fp16 value 1024 + code (or 64 + code) by a
+//    mask or a byte permute, the base is subtracted exactly, and code * step + lo is one fused
+//    multiply-add rounded once to fp16 (the format's lo and step are fp16 already); x^ = lo + code *
+//    step of the format is therefore held to within an fp16 rounding, finer than the bf16 rounding of
+//    the bf16 path.
+//  Bound by instructions and their latency at three warps a scheduler. With the rows first expanded into a
+//  staging buffer in shared memory (16 stores and as many matrix loads for 32 rows, and the barrier between
+//  them), 8 sequences of 32768 tokens at 4 bits took 84 us a layer, in fragments 63, and 58 with the rows
+//  past the rank and the groups past the tile zeroed through (lo, step) instead of fragment by fragment;
+//  4 sequences of spread ranks 67 -> 41 us, 1 sequence of wide ranks at 8 bits 39 -> 30.
 //  - The tensor-core tiles are fp16 (mma m16n8k16 f16): q~ split hi + lo in fp16, the softmax
 //    weights P in fp16 scaled by 2^kPShift (weights down to 2^-31 of the running max stay normal
 //    numbers; the partials carry max - kPShift as their reference, so nothing downstream changes).
@@ -41,18 +48,19 @@ static_assert(kSlack + kPShift <= 15, "scaled weights stay below the fp16 range"
 template <int BITS> struct QLine {
   static constexpr long long row = ((128 * BITS / 8 + 4 * 4) + 15) & ~15;   // qrow(128)
   // ring stage: the largest chunk (4 bits: 32 rows x 80, 64 x 48 or 128 x 32 bytes; 8 bits:
-  // 32 rows x 144 or x 80, 64 x 48)
-  static constexpr int stage = BITS == 4 ? 4096 : 4608;
+  // 32 rows x 144, 64 x 80 or x 48)
+  static constexpr int stage = BITS == 4 ? 4096 : 5120;
+  static constexpr int stages = BITS == 4 ? 4 : 3;   // ring stages per warp (192 KB and 180 KB in all)
   static constexpr long long seg_cost = kSegCost * row / ISL;
   static constexpr long long seg_end = kSegEnd * row / ISL;
 };
 static_assert(QLine<4>::row == 80 && QLine<8>::row == 144, "quantized row sizes");
 
 // Rows per chunk (log2): the bf16 kernel's chunking at 4 bits (32 rows of a full tile, 64 of one of
-// at most 64 slots, 128 of one of at most 32); at 8 bits 32 rows of any tile over 32 slots and 64
-// below, so that a chunk fits a stage and its expansion the 8 KB staging buffer.
+// at most 64 slots, 128 of one of at most 32); at 8 bits 32 rows of a tile over 64 slots and 64
+// below, so that a chunk fits a stage.
 __device__ __forceinline__ int chunk_lg_q(int tl, int bits) {
-  return bits == 4 ? chunk_lg(tl) : (tl > 32 ? 5 : 6);
+  return bits == 4 ? chunk_lg(tl) : (tl > 64 ? 5 : 6);
 }
 
 // Items of bucket r inside the byte range [lo, hi) of a quantized stream: [i0, i1). Item i starts
@@ -156,92 +164,137 @@ __device__ __forceinline__ uint32_t ld_shared_u32(uint32_t a) {
   asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(a));
   return v;
 }
-__device__ __forceinline__ void st_shared_v4(uint32_t a, uint4 v) {
-  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+// Codes -> fp16 pairs. A code c becomes the fp16 number 1024 + c (0x6400 | c) or, four bits higher, 64 + c
+// (0x5400 | c << 4), both exact; the base is subtracted exactly and lo + c * step is one fused multiply-add.
+__device__ __forceinline__ uint32_t code_pair(uint32_t t, uint32_t base, uint32_t lo2, uint32_t st2) {
+  const __half2 code = __hsub2(*reinterpret_cast<const __half2*>(&t), *reinterpret_cast<const __half2*>(&base));
+  const __half2 x = __hfma2(code, *reinterpret_cast<const __half2*>(&st2), *reinterpret_cast<const __half2*>(&lo2));
+  return *reinterpret_cast<const uint32_t*>(&x);
 }
-
-// Eight codes (one 8-slot group) -> eight fp16 values lo + code * step, as four half2. A code c
-// becomes the fp16 number 1024 + c (0x6400 | c, exact for c < 1024). At 8 bits half2 p holds slots
-// 2p, 2p + 1; at 4 bits it holds slots p and p + 4 (nibbles p and p + 4 of the word, one mask
-// apiece), so within each group the staged order of slots is 0 4 1 5 2 6 3 7. Nothing depends on
-// the order of slots inside a tile except the mask of padding slots, which maps it back.
-__device__ __forceinline__ uint4 expand8(uint32_t w0, uint32_t w1, __half2 lo2, __half2 st2, int bits) {
-  const __half2 k1024 = __halves2half2(__ushort_as_half(0x6400), __ushort_as_half(0x6400));
-  uint32_t t[4];
-  if (bits == 4) {   // nibble e holds slot e
-#pragma unroll
-    for (int p = 0; p < 4; ++p) t[p] = ((w0 >> (4 * p)) & 0x000F000Fu) | 0x64006400u;
-  } else {           // byte e of (w0, w1) holds slot e
-    t[0] = __byte_perm(w0, 0x64646464u, 0x4140);
-    t[1] = __byte_perm(w0, 0x64646464u, 0x4342);
-    t[2] = __byte_perm(w1, 0x64646464u, 0x4140);
-    t[3] = __byte_perm(w1, 0x64646464u, 0x4342);
-  }
-  uint32_t o[4];
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const __half2 code = __hsub2(*reinterpret_cast<const __half2*>(&t[p]), k1024);
-    const __half2 x = __hfma2(code, st2, lo2);
-    o[p] = *reinterpret_cast<const uint32_t*>(&x);
-  }
-  return make_uint4(o[0], o[1], o[2], o[3]);
+// u: four 4-bit codes in the low half, four in the high half. o[i] = (code i of the low, code i of the high half).
+__device__ __forceinline__ void expand4(uint32_t u, uint32_t lo2, uint32_t st2, uint32_t* o) {
+  const uint32_t v = u >> 8;
+  o[0] = code_pair((u & 0x000F000Fu) | 0x64006400u, 0x64006400u, lo2, st2);
+  o[1] = code_pair((u & 0x00F000F0u) | 0x54005400u, 0x54005400u, lo2, st2);
+  o[2] = code_pair((v & 0x000F000Fu) | 0x64006400u, 0x64006400u, lo2, st2);
+  o[3] = code_pair((v & 0x00F000F0u) | 0x54005400u, 0x54005400u, lo2, st2);
 }
-
-// Expansion of a tile of fewer than 128 slots, group by group; out of line, so that the main loop's code (with
-// nine copies of dequant_chunk) stays small.
+// a, b: four 8-bit codes each. o[i] = (code i of a, code i of b).
+__device__ __forceinline__ void expand8(uint32_t a, uint32_t b, uint32_t lo2, uint32_t st2, uint32_t* o) {
+  const uint32_t u = __byte_perm(a, b, 0x5140), v = __byte_perm(a, b, 0x7362);
+  o[0] = code_pair(__byte_perm(u, 0x64646464u, 0x4140), 0x64006400u, lo2, st2);
+  o[1] = code_pair(__byte_perm(u, 0x64646464u, 0x4342), 0x64006400u, lo2, st2);
+  o[2] = code_pair(__byte_perm(v, 0x64646464u, 0x4140), 0x64006400u, lo2, st2);
+  o[3] = code_pair(__byte_perm(v, 0x64646464u, 0x4342), 0x64006400u, lo2, st2);
+}
+// 16 slots of two streams of codes -> o[x] = (slot x of a, slot x of b); a, b: 16 codes each (BITS / 2 words).
 template <int BITS>
-__device__ __noinline__ void dequant_short(uint32_t src, uint32_t dst, int rows, int j0, int tl, int lane) {
-  const int ng = tl >> 3, qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
-  for (int jr = lane; jr < rows; jr += 32) {
-    const uint32_t row = src + jr * qrow, orow = dst + jr * (tl * 2);
-    int pos = (j0 + jr) % ng;
-    for (int gi = 0; gi < ng; ++gi) {
-      const uint32_t pq = ld_shared_u32(row + pbase + 4 * (gi >> 2));
-      const __half2 ph = *reinterpret_cast<const __half2*>(&pq);
-      const __half2 lo2 = __low2half2(ph), st2 = __high2half2(ph);
-      const uint32_t w0 = ld_shared_u32(row + (BITS == 4 ? 4 : 8) * gi);
-      const uint32_t w1 = BITS == 8 ? ld_shared_u32(row + 8 * gi + 4) : 0u;
-      st_shared_v4(orow + 16 * pos, expand8(w0, w1, lo2, st2, BITS));
-      pos = pos + 1 == ng ? 0 : pos + 1;
+__device__ __forceinline__ void expand16(const uint32_t* a, const uint32_t* b, uint32_t lo2, uint32_t st2, uint32_t* o) {
+#pragma unroll
+  for (int h = 0; h < BITS / 2; ++h) {
+    if (BITS == 4) {
+      expand4(__byte_perm(a[h], b[h], 0x5410), lo2, st2, o + 8 * h);
+      expand4(__byte_perm(a[h], b[h], 0x7632), lo2, st2, o + 8 * h + 4);
+    } else {
+      expand8(a[h], b[h], lo2, st2, o + 4 * h);
     }
   }
 }
-
-// Expand `rows` staged quantized rows (tile rows j0 .., tl slots) into fp16 rows at `dst` in the
-// packed layout's order (group g of tile row j at position (g + j) mod (tl / 8)). Lane l takes rows
-// l, l + 32, ...; a full 4-bit row is five 16-byte loads (codes, then the four (lo, step) pairs)
-// and sixteen 16-byte stores, whose banks the row stride (80 bytes) and the rotation spread.
+// 16 codes of one row at shared address x
 template <int BITS>
-__device__ __forceinline__ void dequant_chunk(uint32_t src, uint32_t dst, int rows, int j0, int tl, int lane) {
-  const int qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
-  if (tl == ISL) {   // warp-uniform: full tile, 16-byte loads of four groups' codes at a time
-    for (int jr = lane; jr < rows; jr += 32) {
-      const uint32_t row = src + jr * qrow, orow = dst + jr * (ISL * 2);
-      const int j = j0 + jr;
-      const uint4 pr = ld_shared_v4(row + pbase);   // (lo, step) of slot groups 0..3 of 32
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {   // 32 slots: four 8-slot groups
-        const uint32_t pq = q == 0 ? pr.x : q == 1 ? pr.y : q == 2 ? pr.z : pr.w;
-        const __half2 ph = *reinterpret_cast<const __half2*>(&pq);
-        const __half2 lo2 = __low2half2(ph), st2 = __high2half2(ph);
-        uint32_t w[8];
-        if (BITS == 4) {
-          const uint4 c4 = ld_shared_v4(row + 16 * q);
-          w[0] = c4.x; w[1] = c4.y; w[2] = c4.z; w[3] = c4.w;
-        } else {
-          const uint4 a = ld_shared_v4(row + 32 * q), b = ld_shared_v4(row + 32 * q + 16);
-          w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int gi = 4 * q + e;
-          const uint4 v = BITS == 4 ? expand8(w[e], 0u, lo2, st2, 4) : expand8(w[2 * e], w[2 * e + 1], lo2, st2, 8);
-          st_shared_v4(orow + 16 * ((gi + j) & 15), v);
-        }
-      }
-    }
+__device__ __forceinline__ void ld_codes16(uint32_t x, uint32_t* w) {
+  if (BITS == 4) {
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(w[0]), "=r"(w[1]) : "r"(x));
   } else {
-    dequant_short<BITS>(src, dst, rows, j0, tl, lane);
+    const uint4 v = ld_shared_v4(x);
+    w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+  }
+}
+// The row of a 16-row tile of V that lane group g8 takes (and 8 rows on): at 4 bits the even groups rows 0 .. 3
+// and the odd ones rows 4 .. 7, so that the two rows of a quarter warp's 16-byte loads are 4 x 80 bytes apart.
+template <int BITS>
+__device__ __forceinline__ int v_row(int g8) { return BITS == 4 ? (g8 >> 1) + 4 * (g8 & 1) : g8; }
+
+// The A fragments of one 16-row step of K against a tile's 128 slots: m16 x k16, m = slots, k = rows. Row g8 of
+// tile mt is slot 16 g8 + 2 mt, row g8 + 8 the slot after it, so a lane's 16 slots are one run of codes in each
+// of its four rows. `row`: the lane's first row (2 c of the step), pq: its group's (lo, step) in that row;
+// left: rows of the item from that row on. The others are whatever the stage held: with (0, 0) for their (lo, step)
+// they are zeros, since a code is a finite number whatever its bits are.
+template <int BITS>
+__device__ __forceinline__ void k_frags(uint32_t row, uint32_t qrow, uint32_t codes, uint32_t pq, int left,
+                                        uint32_t (&a)[ISL / 16][4]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {   // rows 2c, 2c + 1; then 8 rows on
+    const uint32_t r0 = row + 8 * h * qrow, r1 = r0 + qrow;
+    uint32_t w0[BITS / 2], w1[BITS / 2], o[16];
+    ld_codes16<BITS>(r0 + codes, w0);
+    ld_codes16<BITS>(r1 + codes, w1);
+    uint32_t p0 = ld_shared_u32(r0 + pq), p1 = ld_shared_u32(r1 + pq);
+    if (8 * h >= left) p0 = 0u;
+    if (8 * h + 1 >= left) p1 = 0u;
+    expand16<BITS>(w0, w1, __byte_perm(p0, p1, 0x5410), __byte_perm(p0, p1, 0x7632), o);
+#pragma unroll
+    for (int mt = 0; mt < ISL / 16; ++mt) { a[mt][2 * h] = o[2 * mt]; a[mt][2 * h + 1] = o[2 * mt + 1]; }
+  }
+}
+
+// One row's 32 slots of group c: o[x] = (slot 32 c + x, slot 32 c + 16 + x), as the weights' fragments pair them.
+// !on (a row past the rank, a group past the tile): zeros. The weights of slots past the tile are 0 and their codes,
+// of whatever the row holds there, stay within the range of the group's (lo, step).
+template <int BITS>
+__device__ __forceinline__ void v_row32(uint32_t row, uint32_t pbase, int c, bool on, uint32_t (&o)[16]) {
+  uint32_t w0[BITS / 2], w1[BITS / 2];
+  const uint4 x = ld_shared_v4(row + 4 * BITS * c);
+  if (BITS == 4) {
+    w0[0] = x.x; w0[1] = x.y; w1[0] = x.z; w1[1] = x.w;
+  } else {
+    const uint4 y = ld_shared_v4(row + 4 * BITS * c + 16);
+    w0[0] = x.x; w0[1] = x.y; w0[BITS / 2 - 2] = x.z; w0[BITS / 2 - 1] = x.w;
+    w1[0] = y.x; w1[1] = y.y; w1[BITS / 2 - 2] = y.z; w1[BITS / 2 - 1] = y.w;
+  }
+  uint32_t p = ld_shared_u32(row + pbase + 4 * c);
+  if (!on) p = 0u;
+  expand16<BITS>(w0, w1, __byte_perm(p, p, 0x1010), __byte_perm(p, p, 0x3232), o);
+}
+
+// Short tiles (at most 32 slots, one group): row g8 of tile mt of two is slot 4 g8 + 2 mt, row g8 + 8 the one
+// after it; k pairs of the weights are slots 8 c + x and 8 c + 4 + x.
+template <int BITS>
+__device__ __forceinline__ uint32_t ld_codes4(uint32_t x) {
+  if (BITS == 8) return ld_shared_u32(x);
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];\n" : "=h"(v) : "r"(x));
+  return v;
+}
+template <int BITS>
+__device__ __forceinline__ void k_frags_short(uint32_t row, uint32_t qrow, uint32_t codes, uint32_t pbase, int left,
+                                              uint32_t (&a)[2][4]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t r0 = row + 8 * h * qrow, r1 = r0 + qrow;
+    const uint32_t w0 = ld_codes4<BITS>(r0 + codes), w1 = ld_codes4<BITS>(r1 + codes);
+    uint32_t p0 = ld_shared_u32(r0 + pbase), p1 = ld_shared_u32(r1 + pbase);
+    if (8 * h >= left) p0 = 0u;
+    if (8 * h + 1 >= left) p1 = 0u;
+    const uint32_t lo2 = __byte_perm(p0, p1, 0x5410), st2 = __byte_perm(p0, p1, 0x7632);
+    uint32_t o[4];
+    if (BITS == 4) expand4(__byte_perm(w0, w1, 0x5410), lo2, st2, o);
+    else expand8(w0, w1, lo2, st2, o);
+    a[0][2 * h] = o[0]; a[0][2 * h + 1] = o[1];
+    a[1][2 * h] = o[2]; a[1][2 * h + 1] = o[3];
+  }
+}
+template <int BITS>
+__device__ __forceinline__ void v_row_short(uint32_t row, uint32_t pbase, int c, bool on, uint32_t (&o)[4]) {
+  uint32_t p = ld_shared_u32(row + pbase);
+  if (!on) p = 0u;
+  const uint32_t lo2 = __byte_perm(p, p, 0x1010), st2 = __byte_perm(p, p, 0x3232);
+  if (BITS == 4) {
+    expand4(ld_shared_u32(row + 4 * c), lo2, st2, o);
+  } else {
+    uint32_t w[4];
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];\n" : "=r"(w[0]), "=r"(w[1]) : "r"(row + 8 * c));
+    expand8(w[0], w[1], lo2, st2, o);
   }
 }
 
@@ -257,12 +310,12 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
   constexpr long long kSegCostQ = QLine<BITS>::seg_cost, kSegEndQ = QLine<BITS>::seg_end;
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int STQ = QLine<BITS>::stage;
-  unsigned char* ring = smem;   // NW * ST * STQ of quantized chunks, then NW * STAGE of fp16 rows
-  constexpr int kRing = NW * (ST * STQ + STAGE);
-  static_assert(kRing % 16 == 0 && kRing >= NW * ST * STAGE, "SegSmem 16-byte aligned; merge and combine fit");
+  constexpr int SQ = QLine<BITS>::stages;
+  unsigned char* ring = smem;   // NW * SQ * STQ of quantized chunks
+  constexpr int kRing = NW * SQ * STQ;
   SegSmem& sm = *reinterpret_cast<SegSmem*>(smem + kRing);
   // the merge and combine buffers alias the ring (idle while a segment is merged)
-  static_assert(sizeof(Merge) <= (size_t)NW * ST * STAGE, "merge buffers fit in the ring");
+  static_assert(kRing % 16 == 0 && sizeof(Merge) <= kRing && sizeof(CombSmem) <= kRing, "they fit in the ring");
   Merge& mg = *reinterpret_cast<Merge*>(smem);
   __shared__ long long segW[64];                                  // per-sequence stream length
   __shared__ long long segP[65];                                  // start of sequence b on the cost line
@@ -270,7 +323,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
   __shared__ int n_empty;                                         // sequences with no coded tokens
   __shared__ int last_cta;                                        // this CTA closes the segment
   __shared__ uint32_t parity;                                     // counter set of this call
-  __shared__ uint64_t bar_all[NW * ST];                           // one full-barrier per ring stage
+  __shared__ uint64_t bar_all[NW * SQ];                           // one full-barrier per ring stage
   __shared__ uint64_t bar_comb;                                   // U_V copy of a combine
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -282,8 +335,8 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
   // and waits (griddepcontrol.wait) for this grid to finish before it reads anything
   pdl_trigger();
   // self-contained setup first (it may overlap the tail of the preceding grid)
-  if (tid < NW * ST) mbar_init(&bar_all[tid], 1);
-  if (tid == NW * ST) mbar_init(&bar_comb, 1);
+  if (tid < NW * SQ) mbar_init(&bar_all[tid], 1);
+  if (tid == NW * SQ) mbar_init(&bar_comb, 1);
   fence_mbar_init();
   fence_proxy_async_smem();
   pdl_wait();   // everything below reads data written by earlier grids
@@ -409,9 +462,8 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
       // start this warp's loads first: they do not depend on the rotated queries
       const uint8_t* cK = qdata + ((bl * s.G + g) * 2) * qcap;
       const uint8_t* cV = cK + qcap;
-      const uint32_t ring_w = smem_addr(ring) + warp * ST * STQ;
-      const uint32_t stg_w = smem_addr(ring) + NW * ST * STQ + warp * STAGE;   // this warp's fp16 rows
-      uint64_t* bars = &bar_all[warp * ST];
+      const uint32_t ring_w = smem_addr(ring) + warp * SQ * STQ;
+      uint64_t* bars = &bar_all[warp * SQ];
 
       float Mx[2] = {-INFINITY, -INFINITY}, Ls[2] = {0.f, 0.f};
       float oacc[kHeadDim / 16][4];
@@ -427,9 +479,9 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
       int cons_k = pr.k;
       Item cons = pr.item;
 #pragma unroll
-      for (int i = 0; i < ST; ++i)   // every stage of the ring in flight
-        if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + i) % ST) * STQ,
-                        &bars[(n_issued + i) % ST], total, n_long, lane, policy)) ++n_pending;
+      for (int i = 0; i < SQ; ++i)   // every stage of the ring in flight
+        if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + i) % SQ) * STQ,
+                        &bars[(n_issued + i) % SQ], total, n_long, lane, policy)) ++n_pending;
       int c0, c1;   // the CTAs that share this segment (their partials are merged by the last one)
       seg_cta_range([&](int i) { return cuts[i]; }, T, C, P, W, c0, c1);
       __syncwarp();
@@ -438,31 +490,27 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
       build_qfrag_f16(sm, tid);
       __syncthreads();
 
-      // chunk k of this warp (counted over the whole kernel) lives in stage k % ST, phase (k/ST)&1
+      // chunk k of this warp (counted over the whole kernel) lives in stage k % SQ, phase (k / SQ) & 1
 
       auto wait_chunk = [&]() -> bool {
         const uint32_t k = n_issued;
-        if (!mbar_wait_bounded(&bars[k % ST], (k / ST) & 1u, kWaitTries)) { timed_out = true; return false; }
+        if (!mbar_wait_bounded(&bars[k % SQ], (k / SQ) & 1u, kWaitTries)) { timed_out = true; return false; }
         return true;
       };
       auto next_chunk = [&]() {
-        // the consumed stage is free again: refill it with the chunk ST ahead, so that all the
+        // the consumed stage is free again: refill it with the chunk SQ ahead, so that all the
         // other stages stay in flight while the warp computes
         ++n_issued;
         --n_pending;
-        if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + ST - 1) % ST) * STQ,
-                        &bars[(n_issued + ST - 1) % ST], total, n_long, lane, policy)) ++n_pending;
+        if (issue_chunk_q<BITS>(pr, sm, cK, cV, ring_w + ((n_issued + SQ - 1) % SQ) * STQ,
+                        &bars[(n_issued + SQ - 1) % SQ], total, n_long, lane, policy)) ++n_pending;
       };
 
       while (cons_k < n_long && !timed_out) {
         const int r = cons.r;
         const long long n_real = sm.cnt[r] - (long long)cons.it * ISL;   // real slots of this item
-        // tile geometry (packed layout, coef_offset): rows of tl slots, 8-slot group g of row j
-        // stored at position (g + j) mod (tl / 8)
         const int tl = (int)min((long long)ISL, pad8(sm.cnt[r]) - (long long)cons.it * ISL);
-        const int ng = tl >> 3;
-        const bool full_tile = ng == 16;
-        const uint32_t row_bytes = (uint32_t)tl * 2u;
+        const uint32_t qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
         const int lgc = chunk_lg_q(tl, BITS);           // same chunking as the producer
         const int nj = (r + (1 << lgc) - 1) >> lgc;
         float sc[ISL / 16][4];
@@ -473,47 +521,18 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         for (int jc = 0; jc < nj; ++jc) {
           if (!wait_chunk()) break;
           const int j0 = jc << lgc, j1 = min(r, j0 + (1 << lgc));
-          dequant_chunk<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, j1 - j0, j0, tl, lane);
-          __syncwarp();
-          next_chunk();   // the stage is free once its rows are dequantized: refill it now
-          const uint32_t st_addr = stg_w;
-          const int m = lane >> 3, r8 = lane & 7;
+          const uint32_t row0 = ring_w + (n_issued % SQ) * STQ + 2 * c * qrow;
           for (int j16 = j0; j16 < j1; j16 += 16) {
             const uint4 qf = *reinterpret_cast<const uint4*>(&sm.qfrag[j16 >> 4][lane][0]);
-            // this lane's row of the 8x8 matrices: coefficient j, staged at row (j - chunk start)
-            const int jrow = (j16 - j0) + (m >> 1) * 8 + r8;
-            const int j = j0 + jrow;
-            const uint32_t row_addr = st_addr + jrow * row_bytes;
             uint32_t a[ISL / 16][4];
-            // stored position of slot group 2 mt + (m & 1) in row j: (group + j) mod ng; for a full
-            // tile every offset is computed on its own (no chain through the previous one)
-            uint32_t off[ISL / 16];
-            if (full_tile) {
-              const uint32_t o0 = (uint32_t)(((m & 1) + j) & 15) << 4;
-#pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) off[mt] = (o0 + 32u * mt) & 255u;
-            } else {
-              int pg = ((m & 1) + j) % ng;
-#pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) { off[mt] = 16u * pg; pg = wrap2(pg, ng); }
-            }
-#pragma unroll
-            for (int mt = 0; mt < ISL / 16; ++mt) ldsm_x4_trans(row_addr + off[mt], a[mt]);
-            if (j16 + 16 > r) {   // warp-uniform: rows >= r of this k-step are not coefficients
-              // A fragment registers 0, 1 hold rows j16 + 2c (+1), registers 2, 3 rows 8 later
-              const int jb = j16 + 2 * c;
-              const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
-#pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) {
-                a[mt][0] &= m0; a[mt][1] &= m0; a[mt][2] &= m1; a[mt][3] &= m1;
-              }
-            }
+            k_frags<BITS>(row0 + (j16 - j0) * qrow, qrow, 2 * BITS * g8, pbase + 4 * (g8 >> 1), r - j16 - 2 * c, a);
 #pragma unroll
             for (int mt = 0; mt < ISL / 16; ++mt) mma_f16_16816(sc[mt], a[mt], qf.x, qf.y);
 #pragma unroll
             for (int mt = 0; mt < ISL / 16; ++mt) mma_f16_16816(sc[mt], a[mt], qf.z, qf.w);
           }
-          __syncwarp();   // every lane has read the staged rows before the next chunk replaces them
+          __syncwarp();   // every lane has read the stage before it is refilled
+          next_chunk();
         }
         if (timed_out) break;
 
@@ -523,10 +542,9 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
 #pragma unroll
         for (int mt = 0; mt < ISL / 16; ++mt) {
           if (!full_item) {
-            // stored position g8 of an 8-slot group holds slot g8 (8 bits) or g8 / 2 + 4 (g8 % 2) (4 bits)
-            const int s0 = mt * 16 + (BITS == 4 ? (g8 >> 1) + 4 * (g8 & 1) : g8);
+            const int s0 = 16 * g8 + 2 * mt;
             if (s0 >= n_real) { sc[mt][0] = sc[mt][1] = -INFINITY; }
-            if (s0 + 8 >= n_real) { sc[mt][2] = sc[mt][3] = -INFINITY; }
+            if (s0 + 1 >= n_real) { sc[mt][2] = sc[mt][3] = -INFINITY; }
           }
           mloc[0] = fmaxf(mloc[0], fmaxf(sc[mt][0], sc[mt][2]));
           mloc[1] = fmaxf(mloc[1], fmaxf(sc[mt][1], sc[mt][3]));
@@ -555,7 +573,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         }
         float lsum[2] = {0.f, 0.f};
         const float Mr[2] = {Mx[0] - kPShift, Mx[1] - kPShift};   // weights scaled by 2^kPShift
-        uint32_t pb[ISL / 16][2];   // per slot tile: b0, b1 of P^T (bf16)
+        uint32_t pb[ISL / 16][2];   // per slot tile: b0, b1 of P^T
 #pragma unroll
         for (int mt = 0; mt < ISL / 16; ++mt) {
           const float p0 = fast_exp2(sc[mt][0] - Mr[0]), p1 = fast_exp2(sc[mt][1] - Mr[1]);
@@ -571,108 +589,76 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         // ---- V chunks: weighted coefficient rows (rows >= r masked in the A fragment)
         {
           int left = 0;             // rows of the current chunk not used yet
-          int j0 = 0;               // first row of the current chunk
-          uint32_t st_addr = 0;
-          bool ok = true;
-          const int m = lane >> 3, r8 = lane & 7;
+          uint32_t row = 0;         // this lane's row of the next 16-row tile
 #pragma unroll
-          for (int jt = 0; jt < kHeadDim / 16; ++jt) {   // 16-row tile of o~
-            if (jt * 16 >= r) break;                     // warp-uniform
-            if (left == 0) {                             // the tile starts a chunk
-              __syncwarp();   // (jt > 0) the previous chunk's staged rows have been read
-              if (!wait_chunk()) { ok = false; break; }
-              j0 = jt * 16;
-              dequant_chunk<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, min(r - j0, 1 << lgc), j0, tl, lane);
-              __syncwarp();
-              next_chunk();
-              st_addr = stg_w;
+          for (int jp = 0; jp < kHeadDim / 32; ++jp) {   // two 16-row tiles of o~ (chunks are 32 rows or more)
+            if (jp * 32 >= r) break;                     // warp-uniform
+            if (left == 0) {                             // the tiles start a chunk
+              if (!wait_chunk()) break;
+              row = ring_w + (n_issued % SQ) * STQ + v_row<BITS>(g8) * qrow;
               left = 1 << lgc;
             }
-            left -= 16;
-            const int jrow = (jt * 16 - j0) + (m & 1) * 8 + r8;
-            const int j = j0 + jrow;
-            const uint32_t row_addr = st_addr + jrow * row_bytes;
-            const bool keep0 = jt * 16 + g8 < r, keep1 = jt * 16 + g8 + 8 < r;
-            float t1[4] = {0.f, 0.f, 0.f, 0.f};
-            // stored position of slot group 2 kt + (m >> 1) (kt = 0..7) in row j, as in the K loop
-            uint32_t off[ISL / 16];
-            if (full_tile) {
-              const uint32_t o0 = (uint32_t)(((m >> 1) + j) & 15) << 4;
 #pragma unroll
-              for (int kt = 0; kt < ISL / 16; ++kt) off[kt] = (o0 + 32u * kt) & 255u;
-            } else {
-              int pg = ((m >> 1) + j) % ng;
+            for (int jt = 2 * jp; jt < 2 * jp + 2; ++jt) {
+              if (jt * 16 >= r) break;
+              uint32_t o0[16], o1[16];
+              const int left_r = r - jt * 16 - v_row<BITS>(g8);
+              v_row32<BITS>(row, pbase, c, left_r > 0 && 32 * c < tl, o0);
+              v_row32<BITS>(row + 8 * qrow, pbase, c, left_r > 8 && 32 * c < tl, o1);
+              row += 16 * qrow;
+              float t1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-              for (int kt = 0; kt < ISL / 16; ++kt) { off[kt] = 16u * pg; pg = wrap2(pg, ng); }
-            }
-#pragma unroll
-            for (int kt = 0; kt < ISL / 16; kt += 2) {
-              uint32_t a[4], b[4];
-              ldsm_x4(row_addr + off[kt], a);
-              ldsm_x4(row_addr + off[kt + 1], b);
-              if (jt * 16 + 16 > r) {                    // warp-uniform: rows >= r in this tile
-                if (!keep0) { a[0] = a[2] = 0u; b[0] = b[2] = 0u; }
-                if (!keep1) { a[1] = a[3] = 0u; b[1] = b[3] = 0u; }
+              for (int kt = 0; kt < ISL / 16; ++kt) {
+                const uint32_t a[4] = {o0[2 * kt], o1[2 * kt], o0[2 * kt + 1], o1[2 * kt + 1]};
+                mma_f16_16816(kt & 1 ? t1 : oacc[jt], a, pb[kt][0], pb[kt][1]);
               }
-              mma_f16_16816(oacc[jt], a, pb[kt][0], pb[kt][1]);
-              mma_f16_16816(t1, b, pb[kt + 1][0], pb[kt + 1][1]);
-            }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) oacc[jt][e] += t1[e];
+              for (int e = 0; e < 4; ++e) oacc[jt][e] += t1[e];
+            }
+            left -= 32;
+            if (left == 0 || jp * 32 + 32 >= r) {        // the chunk's last rows
+              __syncwarp();   // every lane has read the stage before it is refilled
+              next_chunk();
+              left = 0;
+            }
           }
-          (void)ok;
-          __syncwarp();   // the staged rows are read before the next item's first chunk
         }
         cons_k += NW;
         if (cons_k < total) cons = next_rr_split<NW>(sm, cons, cons_k, n_long);
       }
       // Short items (at most kShort slots): the same steps on two 16-slot tiles instead of eight, in a loop of
       // their own as in decode_mma.cu (one chunk each of K and V rows, at 8 bits two past 64 rows). Before / with
-      // it and the out-of-line expansion of short tiles, us per call: 1 sequence, 8 bits, wide ranks 57 / 39; 4
-      // sequences, 4 bits, spread ranks 79 / 67; 8 sequences, 4 bits, nearly equal ranks 85 / 84 (90 with the
-      // expansion inlined nine times: the main loop is held by its code's size).
+      // it, us per call: 1 sequence, 8 bits, wide ranks 57 / 39; 4 sequences, 4 bits, spread ranks 79 / 67.
       while (cons_k < total && !timed_out) {
         const int r = cons.r;
-        const int n_real = sm.cnt[r] - cons.it * ISL, tl = (n_real + 7) & ~7, ng = tl >> 3;
-        const uint32_t row_bytes = (uint32_t)tl * 2u;
+        const int n_real = sm.cnt[r] - cons.it * ISL, tl = (n_real + 7) & ~7;
+        const uint32_t qrow = qrow_bytes(tl, BITS), pbase = tl * BITS / 8;
         const int lgc = chunk_lg_q(tl, BITS);
-        const int m = lane >> 3, r8 = lane & 7;
         float sh[2][4] = {}, sl[2][4] = {};
         for (int j0 = 0; j0 < r; j0 += 1 << lgc) {
           if (!wait_chunk()) break;
           const int j1 = min(r, j0 + (1 << lgc));
-          dequant_short<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, j1 - j0, j0, tl, lane);
-          __syncwarp();
-          next_chunk();
+          const uint32_t row0 = ring_w + (n_issued % SQ) * STQ + 2 * c * qrow;
           for (int j16 = j0; j16 < j1; j16 += 16) {
             const uint4 qf = *reinterpret_cast<const uint4*>(&sm.qfrag[j16 >> 4][lane][0]);
-            const int jrow = (j16 - j0) + (m >> 1) * 8 + r8;
-            const uint32_t row_addr = stg_w + jrow * row_bytes;
-            const int pg = ((m & 1) + j0 + jrow) % ng;
             uint32_t a[2][4];
-            ldsm_x4_trans(row_addr + 16 * pg, a[0]);
-            ldsm_x4_trans(row_addr + 16 * wrap2(pg, ng), a[1]);
-            if (j16 + 16 > r) {
-              const int jb = j16 + 2 * c;
-              const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
-#pragma unroll
-              for (int mt = 0; mt < 2; ++mt) { a[mt][0] &= m0; a[mt][1] &= m0; a[mt][2] &= m1; a[mt][3] &= m1; }
-            }
+            k_frags_short<BITS>(row0 + (j16 - j0) * qrow, qrow, BITS / 2 * g8, pbase, r - j16 - 2 * c, a);
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
               mma_f16_16816(sh[mt], a[mt], qf.x, qf.y);
               mma_f16_16816(sl[mt], a[mt], qf.z, qf.w);
             }
           }
-          __syncwarp();   // every lane has read the staged rows before the next chunk replaces them
+          __syncwarp();   // every lane has read the stage before it is refilled
+          next_chunk();
         }
         if (timed_out) break;
         float mloc[2] = {-INFINITY, -INFINITY};
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt) {
-          const int s0 = mt * 16 + (BITS == 4 ? (g8 >> 1) + 4 * (g8 & 1) : g8);   // the slot at stored position g8
+          const int s0 = 4 * g8 + 2 * mt;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sh[mt][e] = s0 + (e >> 1) * 8 < n_real ? sh[mt][e] + sl[mt][e] : -INFINITY;
+          for (int e = 0; e < 4; ++e) sh[mt][e] = s0 + (e >> 1) < n_real ? sh[mt][e] + sl[mt][e] : -INFINITY;
           mloc[0] = fmaxf(mloc[0], fmaxf(sh[mt][0], sh[mt][2]));
           mloc[1] = fmaxf(mloc[1], fmaxf(sh[mt][1], sh[mt][3]));
         }
@@ -700,42 +686,40 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
           pb[mt][0] = movmatrix_trans(pack_f16(p0, p1));
           pb[mt][1] = movmatrix_trans(pack_f16(p2, p3));
         }
+        uint32_t row = 0;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {                 // 64 rows: one chunk of 8-bit rows, half a chunk of 4-bit rows
           if (hf * 64 >= r) break;                       // warp-uniform
-          const int j0 = lgc == 6 ? hf * 64 : 0;         // first staged row
           if (hf == 0 || lgc == 6) {
-            __syncwarp();
             if (!wait_chunk()) break;
-            dequant_short<BITS>(ring_w + (n_issued % ST) * STQ, stg_w, min(r - j0, 1 << lgc), j0, tl, lane);
-            __syncwarp();
-            next_chunk();
+            row = ring_w + (n_issued % SQ) * STQ + v_row<BITS>(g8) * qrow;
           }
 #pragma unroll
           for (int jt = 4 * hf; jt < 4 * hf + 4; ++jt) {
             if (jt * 16 >= r) break;
-            const int jrow = (jt * 16 - j0) + (m & 1) * 8 + r8;
-            const uint32_t row_addr = stg_w + jrow * row_bytes;
-            const int pg = ((m >> 1) + j0 + jrow) % ng;
-            uint32_t a[4], b2[4];
-            ldsm_x4(row_addr + 16 * pg, a);
-            ldsm_x4(row_addr + 16 * wrap2(pg, ng), b2);
-            if (jt * 16 + 16 > r) {
-              if (jt * 16 + g8 >= r) { a[0] = a[2] = 0u; b2[0] = b2[2] = 0u; }
-              if (jt * 16 + g8 + 8 >= r) { a[1] = a[3] = 0u; b2[1] = b2[3] = 0u; }
+            uint32_t o0[4], o1[4];
+            const int left_r = r - jt * 16 - v_row<BITS>(g8);
+            v_row_short<BITS>(row, pbase, c, left_r > 0, o0);
+            v_row_short<BITS>(row + 8 * qrow, pbase, c, left_r > 8, o1);
+            row += 16 * qrow;
+#pragma unroll
+            for (int kt = 0; kt < 2; ++kt) {
+              const uint32_t a[4] = {o0[2 * kt], o1[2 * kt], o0[2 * kt + 1], o1[2 * kt + 1]};
+              mma_f16_16816(oacc[jt], a, pb[kt][0], pb[kt][1]);
             }
-            mma_f16_16816(oacc[jt], a, pb[0][0], pb[0][1]);
-            mma_f16_16816(oacc[jt], b2, pb[1][0], pb[1][1]);
+          }
+          if (lgc == 6 || hf == 1 || r <= 64) {          // the chunk's last rows
+            __syncwarp();   // every lane has read the stage before it is refilled
+            next_chunk();
           }
         }
-        __syncwarp();   // the staged rows are read before the next item's first chunk
         cons_k += NW;
         if (cons_k < total) cons = next_rr_split<NW>(sm, cons, cons_k, n_long);
       }
       // drain: never leave bulk copies in flight into this ring (a copy whose wait gave up stays
       // counted in n_pending and is waited for once more before the CTA exits)
       while (n_pending > 0 && !timed_out) {
-        if (!mbar_wait_bounded(&bars[n_issued % ST], (n_issued / ST) & 1u, kWaitTries)) {
+        if (!mbar_wait_bounded(&bars[n_issued % SQ], (n_issued / SQ) & 1u, kWaitTries)) {
           timed_out = true;
           break;
         }
@@ -757,10 +741,10 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
       if (!dead) {
 #pragma unroll
         for (int t = 0; t < kHeadDim / 16; ++t) {
-          mg.acc[warp][2 * c][t * 16 + g8] = oacc[t][0];
-          mg.acc[warp][2 * c + 1][t * 16 + g8] = oacc[t][1];
-          mg.acc[warp][2 * c][t * 16 + g8 + 8] = oacc[t][2];
-          mg.acc[warp][2 * c + 1][t * 16 + g8 + 8] = oacc[t][3];
+          mg.acc[warp][2 * c][t * 16 + v_row<BITS>(g8)] = oacc[t][0];
+          mg.acc[warp][2 * c + 1][t * 16 + v_row<BITS>(g8)] = oacc[t][1];
+          mg.acc[warp][2 * c][t * 16 + v_row<BITS>(g8) + 8] = oacc[t][2];
+          mg.acc[warp][2 * c + 1][t * 16 + v_row<BITS>(g8) + 8] = oacc[t][3];
         }
       }
       if (!dead && tid < kHeadsPad) {
@@ -849,7 +833,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
   if (dead) {
     // last bounded waits for copies that may still be landing in this CTA's shared memory
     for (; n_pending > 0; --n_pending, ++n_issued)
-      if (!mbar_wait_bounded(&bar_all[warp * ST + n_issued % ST], (n_issued / ST) & 1u, kWaitTries)) break;
+      if (!mbar_wait_bounded(&bar_all[warp * SQ + n_issued % SQ], (n_issued / SQ) & 1u, kWaitTries)) break;
     if (n_comb > 0 && tid == 0) mbar_wait_bounded(&bar_comb, (n_comb - 1) & 1u, kWaitTries);
   }
   if (timed_out && lane == 0) raise_status(dev_status, VARRATE_ERR_TIMEOUT);
@@ -864,7 +848,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
 
 size_t decode_q_smem_bytes(int bits) {
   const int stq = bits == 4 ? QLine<4>::stage : QLine<8>::stage;
-  return (size_t)NW * (ST * stq + STAGE) + sizeof(SegSmem);
+  return (size_t)NW * stq * (bits == 4 ? QLine<4>::stages : QLine<8>::stages) + sizeof(SegSmem);
 }
 
 bool decode_q_supported(const Shape& s, int bits, int64_t qcap, int n_tail, int num_sms) {
