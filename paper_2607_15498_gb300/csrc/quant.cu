@@ -18,24 +18,25 @@ namespace vr {
 namespace {
 
 constexpr int kMaxR = kHeadDim;
-constexpr int kGroup = 32;
 
 // grid (2 G, B L, splits), 256 threads: CTA (stream, bl, z) quantizes the z-th share of the tiles of stream
-// (b, l, g, kv); the first CTA of a pair writes qbase. A warp takes one tile at a time, its lanes as rows of
-// ng4 = tl / 8 rounded up to 4: lane (lr, gp) reads the 8 bf16 coefficients of slot group gp of row
-// j = lr, lr + rps, ... (stored at position (gp + j) mod (tl / 8)), the four lanes of a 32-slot group
-// agree on its min and max by shuffles, and each lane writes its 8 codes (one 32-bit word at 4 bits, two
-// at 8 bits); the group's first lane writes (lo, step) and the row's padding bytes are zeroed.
+// (b, l, g, kv); the first CTA of a pair writes qbase. A warp takes one tile at a time and a lane one 32-slot
+// group of a row: lane (lr, qp) reads the (up to) four 8-slot groups of group qp of row j = lr, lr + rps, ...
+// (8-slot group gi is stored at position (gi + j) mod (tl / 8)), finds their min and max as bf16 pairs, and writes
+// the codes (16 bytes at 4 bits, 32 at 8), (lo, step) and its share of the row's zero padding.
 //
-// Bound by instructions. The code is rint(fl((x - lo) / step)); an IEEE division per coefficient took
-// most of them. t = (x - lo) * fl(1 / step) is within 2^-23 of the quotient relatively, and the rounded
-// quotient within 2^-24, so for quotients below 2^b the two are less than 1.5 * 2^(b - 23) apart: when t is
-// farther than 2^(b - 22) from the middle between two codes, both round to the same code. The few lanes
-// with a coefficient nearer than that divide.
-// 16 pairs of 32768 tokens at 8 bits (645 MB read and written): 787 us (of which 41 a serial kernel for the
-// tables) -> 238 us; 32 pairs at 4 bits 1411 -> 484 us.
+// Bound by instructions, and by loads in flight. The code is rint(fl((x - lo) / step)); an IEEE division per
+// coefficient took most of them. With Q = 2^b - 1 and the exact product step Q, t = (x - lo) * fl(1 / (step Q)),
+// saturated to [0, 1], times Q is within 2^-23 of the quotient relatively, and the rounded quotient within
+// 2^-24, so for quotients below 2^b the two are less than 1.5 * 2^(b - 23) apart: when t Q is farther than
+// 2^(b - 22) from the middle between two codes, both round to the same code (and outside [0, Q] both are the
+// end of the range). The few lanes with a coefficient nearer than that divide.
+// A call on 16 pairs of 32768 tokens at 8 bits (645 MB read and written): 804 us (of which 41 a serial kernel
+// for the tables) with a division each, 244 us without, then 205 with a lane per 32-slot group in place of four
+// (no shuffles, a quarter of the work on lo and step) and 169 with pairwise min and max, mixed-precision
+// differences, saturation in place of two clamps and paired fp32 operations; at 4 bits 262 -> 167 us by the last
+// two. More rows in flight per lane cost resident warps: three CTAs of 80 registers 181 us, with two rows 178.
 constexpr uint32_t kBias4 = 0x3F400000u;   // sum over e of 0x4B400000 * 16^e, modulo 2^32
-constexpr int kStepRows = 4;   // row steps per lane whose loads are in flight together
 
 __device__ __forceinline__ int code_exact(float d, float s32, float qmax) {
   int cq = 0;
@@ -43,8 +44,52 @@ __device__ __forceinline__ int code_exact(float d, float s32, float qmax) {
   return min(max(cq, 0), (int)qmax);
 }
 
+// Two fp32 operations as one instruction, each rounded to nearest.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 c;
+  asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(c.x), "=f"(c.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return c;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("{\n .reg .b64 x, y, z;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n mov.b64 z, {%6, %7};\n"
+      " fma.rn.f32x2 x, x, y, z;\n mov.b64 {%0, %1}, x;\n}\n"
+      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return d;
+}
+// min(max(a b, 0), 1), NaN as 0
+__device__ __forceinline__ float mul_sat(float a, float b) {
+  float c;
+  asm("mul.rn.sat.f32 %0, %1, %2;\n" : "=f"(c) : "f"(a), "f"(b));
+  return c;
+}
+// Both bf16 of w (exact in fp32) + a, rounded to nearest.
+__device__ __forceinline__ float2 add_bf2(uint32_t w, float a) {
+  float2 c;
+  asm("{\n .reg .b16 l, h;\n mov.b32 {l, h}, %2;\n add.rn.f32.bf16 %0, l, %3;\n add.rn.f32.bf16 %1, h, %3;\n}\n"
+      : "=f"(c.x), "=f"(c.y) : "r"(w), "f"(a));
+  return c;
+}
+__device__ __forceinline__ __nv_bfloat162 as_bf2(uint32_t w) { return *reinterpret_cast<const __nv_bfloat162*>(&w); }
+
+// The codes of eight coefficients by division, packed as stored. Out of line: the few lanes that need it do not
+// make the others' registers spill.
 template <int BITS>
-__global__ void __launch_bounds__(256)
+__device__ __noinline__ uint2 codes_exact(uint4 x, float lo32, float s32) {
+  const uint32_t w4[4] = {x.x, x.y, x.z, x.w};
+  constexpr float kQmax = (float)((1 << BITS) - 1);
+  uint32_t c[2] = {0, 0};
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float2 d = add_bf2(w4[k >> 1], -lo32);
+    c[k * BITS / 32] |= (uint32_t)code_exact(k & 1 ? d.y : d.x, s32, kQmax) << (k * BITS % 32);
+  }
+  return make_uint2(c[0], c[1]);
+}
+
+template <int BITS>
+__global__ void __launch_bounds__(256, 4)
 quantize_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restrict__ bucket_count,
                 const int64_t* __restrict__ bucket_base, int64_t* __restrict__ qbase,
                 uint8_t* __restrict__ qdata, int32_t* __restrict__ dev_status, Shape s, int64_t qcap) {
@@ -116,79 +161,90 @@ quantize_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restric
     const int r = lo_r;
     const long long i = T - tiles_pre[r];
     const int tl = (int)min(128ll, pad8(cnt[r]) - 128 * i);
-    const int ng = tl >> 3, ng4 = (ng + 3) & ~3;
-    const int rps = ng4 == 16 ? 2 : 32 / ng4;      // rows per step
-    const int lr = ng4 == 16 ? lane >> 4 : lane / ng4, gp = lane - lr * ng4;
+    const int ng = tl >> 3, nq = (ng + 3) >> 2;    // 8-slot groups and 32-slot groups of a row
+    const int rps = 32 / nq;                       // rows per step
+    const int lr = nq == 4 ? lane >> 2 : lane / nq, qp = lane - lr * nq;
     const int qrow = qrow_bytes(tl, BITS);
-    const int raw = tl * BITS / 8 + 4 * ((tl + kGroup - 1) / kGroup);
+    const int raw = tl * BITS / 8 + 4 * nq;
     const __nv_bfloat16* stile = src + base[r] + 128 * i * r;
     uint8_t* qtile = dst + qb[r] + i * (long long)r * qrow_bytes(128, BITS);
-    const bool on = gp < ng && lr < rps;
-    for (int j0 = 0; j0 < r; j0 += rps * kStepRows) {
-      uint4 x[kStepRows];
+    const int n8 = min(4, ng - 4 * qp);            // 8-slot groups of this lane's group
+    for (int j0 = 0; j0 < r; j0 += rps) {
+      uint4 x[4];
+      const int j = j0 + lr;
+      if (lr >= rps || j >= r) continue;
+      const uint4* srow = reinterpret_cast<const uint4*>(stile + j * tl);
+      if (ng == 16) {
 #pragma unroll
-      for (int u = 0; u < kStepRows; ++u) {   // every row's load in flight before the first use
-        const int j = j0 + rps * u + lr;
-        x[u] = make_uint4(0, 0, 0, 0);
-        if (on && j < r)
-          x[u] = __ldcs(reinterpret_cast<const uint4*>(stile + j * tl + 8 * (ng == 16 ? ((gp + j) & 15) : (gp + j) % ng)));
-      }
+        for (int e = 0; e < 4; ++e) x[e] = __ldg(srow + ((4 * qp + e + j) & 15));
+      } else {
+        int pos = (4 * qp + j) % ng;
 #pragma unroll
-      for (int u = 0; u < kStepRows; ++u) {
-        if (j0 + rps * u >= r) break;   // warp-uniform: no row of this step
-        const int j = j0 + rps * u + lr;
-        const bool valid = on && j < r;   // other lanes may still have a row: no early exit
-        float v[8];
-        v[0] = __uint_as_float(x[u].x << 16); v[1] = __uint_as_float(x[u].x & 0xffff0000u);
-        v[2] = __uint_as_float(x[u].y << 16); v[3] = __uint_as_float(x[u].y & 0xffff0000u);
-        v[4] = __uint_as_float(x[u].z << 16); v[5] = __uint_as_float(x[u].z & 0xffff0000u);
-        v[6] = __uint_as_float(x[u].w << 16); v[7] = __uint_as_float(x[u].w & 0xffff0000u);
-        float mn = INFINITY, mx = -INFINITY;
-        if (valid) {
-          mn = fminf(fminf(fminf(v[0], v[1]), fminf(v[2], v[3])), fminf(fminf(v[4], v[5]), fminf(v[6], v[7])));
-          mx = fmaxf(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])), fmaxf(fmaxf(v[4], v[5]), fmaxf(v[6], v[7])));
+        for (int e = 0; e < 4; ++e) {
+          if (e < n8) x[e] = __ldg(srow + pos);
+          pos = pos + 1 == ng ? 0 : pos + 1;
         }
-        // the four lanes of a 32-slot group (gp = 4 q .. 4 q + 3 of the same row)
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        const __half lo = __float2half_rn(mn);
-        const float lo32 = __half2float(lo);
-        // a range beyond the fp16 range saturates the step at the largest finite fp16
-        const __half st = __float2half_rn(fminf(__fdiv_rn(__fsub_rn(mx, lo32), kQmax), 65504.f));
-        const float s32 = __half2float(st);
-        const float inv = s32 != 0.f ? __frcp_rn(s32) : 0.f;
+      }
+      __nv_bfloat162 lo2 = as_bf2(x[0].x), hi2 = lo2;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (e < n8) {
+          const uint32_t w4[4] = {x[e].x, x[e].y, x[e].z, x[e].w};
+#pragma unroll
+          for (int k = 0; k < 4; ++k) { lo2 = __hmin2(lo2, as_bf2(w4[k])); hi2 = __hmax2(hi2, as_bf2(w4[k])); }
+        }
+      }
+      const float2 lf = __bfloat1622float2(lo2), hf = __bfloat1622float2(hi2);
+      const float mn = fminf(fminf(INFINITY, lf.x), lf.y), mx = fmaxf(fmaxf(-INFINITY, hf.x), hf.y);   // NaN: left out
+      const __half lo = __float2half_rn(mn);
+      const float lo32 = __half2float(lo);
+      // a range beyond the fp16 range saturates the step at the largest finite fp16
+      const __half st = __float2half_rn(fminf(__fdiv_rn(__fsub_rn(mx, lo32), kQmax), 65504.f));
+      const float s32 = __half2float(st);
+      const float inv = s32 != 0.f ? __frcp_rn(__fmul_rn(s32, kQmax)) : 0.f;   // the product is exact
+      uint8_t* row = qtile + (long long)j * qrow;
+      uint32_t w[BITS];   // the group's 32 codes
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (e >= n8) break;
+        const uint32_t w4[4] = {x[e].x, x[e].y, x[e].z, x[e].w};
         uint32_t q[8];
         float off = 0.f;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float t = fminf(fmaxf(__fmul_rn(__fsub_rn(v[e], lo32), inv), 0.f), kQmax);   // NaN: code 0
-          const float m = __fadd_rn(t, kMagic);
-          off = fmaxf(off, fabsf(__fsub_rn(t, __fsub_rn(m, kMagic))));
-          q[e] = __float_as_uint(m);   // 0x4B400000 + code
+        for (int k = 0; k < 4; ++k) {
+          const float2 d = add_bf2(w4[k], -lo32);
+          const float2 t = make_float2(mul_sat(d.x, inv), mul_sat(d.y, inv));   // NaN: 0
+          const float2 m = fma2(t, make_float2(kQmax, kQmax), make_float2(kMagic, kMagic));
+          const float2 f = fma2(t, make_float2(-kQmax, -kQmax), add2(m, make_float2(-kMagic, -kMagic)));
+          off = fmaxf(off, fmaxf(fabsf(f.x), fabsf(f.y)));
+          q[2 * k] = __float_as_uint(m.x);   // 0x4B400000 + code
+          q[2 * k + 1] = __float_as_uint(m.y);
         }
-        if (off > kMid) {
+        uint2 c8;
+        if (BITS == 4) {
+          c8.x = q[7];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) q[e] = 0x4B400000u + code_exact(__fsub_rn(v[e], lo32), s32, kQmax);
+          for (int k = 6; k >= 0; --k) c8.x = (c8.x << 4) + q[k];   // the biases add up to kBias4 modulo 2^32
+          c8.x -= kBias4;
+        } else {
+          c8.x = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+          c8.y = __byte_perm(__byte_perm(q[4], q[5], 0x0040), __byte_perm(q[6], q[7], 0x0040), 0x5410);
         }
-        if (lr >= rps || j >= r) continue;
-        uint8_t* row = qtile + (long long)j * qrow;
-        if (on) {
-          if (BITS == 4) {
-            uint32_t w = q[7];
-#pragma unroll
-            for (int e = 6; e >= 0; --e) w = (w << 4) + q[e];   // the biases add up to kBias4 modulo 2^32
-            *reinterpret_cast<uint32_t*>(row + 4 * gp) = w - kBias4;
-          } else {
-            *reinterpret_cast<uint2*>(row + 8 * gp) = make_uint2(
-                __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410),
-                __byte_perm(__byte_perm(q[4], q[5], 0x0040), __byte_perm(q[6], q[7], 0x0040), 0x5410));
-          }
-          if ((gp & 3) == 0) *reinterpret_cast<__half2*>(row + tl * BITS / 8 + 4 * (gp >> 2)) = __halves2half2(lo, st);
+        if (off > kMid) c8 = codes_exact<BITS>(x[e], lo32, s32);
+        w[BITS / 4 * e] = c8.x;
+        if (BITS == 8) w[BITS / 4 * e + BITS / 8] = c8.y;
+        if (n8 < 4) {
+          if (BITS == 4) *reinterpret_cast<uint32_t*>(row + 16 * qp + 4 * e) = c8.x;
+          else *reinterpret_cast<uint2*>(row + 32 * qp + 8 * e) = c8;
         }
-        for (int z0 = raw + gp; z0 < qrow; z0 += ng4) row[z0] = 0;   // zero padding of the row to its 16-byte size
       }
+      if (n8 == 4) {
+        uint4* d = reinterpret_cast<uint4*>(row + 4 * BITS * qp);
+        d[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (BITS == 8) d[1] = make_uint4(w[BITS - 4], w[BITS - 3], w[BITS - 2], w[BITS - 1]);
+      }
+      *reinterpret_cast<__half2*>(row + tl * BITS / 8 + 4 * qp) = __halves2half2(lo, st);
+      for (int z0 = raw + 4 * qp; z0 < qrow; z0 += 4 * nq) *reinterpret_cast<uint32_t*>(row + z0) = 0u;   // to a multiple of 16 bytes
     }
   }
 }
@@ -198,10 +254,10 @@ quantize_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restric
 int launch_quantize(const Shape& s, const varrate_packed& in, const varrate_qpacked& out,
                     int32_t* dev_status, int num_sms, cudaStream_t st) {
   const int64_t pairs = (int64_t)s.B * s.L;
-  // splits of a stream: eight CTAs of eight warps for each SM over all streams (two resident waves), but at
-  // least four full tiles for the eight warps of a CTA
+  // splits of a stream: sixteen CTAs of eight warps for each SM over all streams (four resident waves: 8 of them
+  // 182 us against 176 for the 16 pairs above, 32 no gain), but at least four full tiles for the eight warps of a CTA
   const int64_t streams = 2 * s.G * pairs;
-  int64_t z = (8LL * num_sms + streams - 1) / streams;
+  int64_t z = (16LL * num_sms + streams - 1) / streams;
   const int64_t most = (s.N + 511) / 512;
   if (z > most) z = most;
   const dim3 grid(2 * s.G, (unsigned)pairs, (unsigned)(z < 1 ? 1 : z));
