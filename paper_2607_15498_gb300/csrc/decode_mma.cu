@@ -17,8 +17,11 @@
 // other is in flight (the stage it finishes is refilled with the chunk two ahead), across item
 // boundaries, so loads never wait on arithmetic. The per-row rotation of
 // the 8-slot groups keeps the unpadded staged rows free of shared-memory bank conflicts. Rows >= r
-// of a chunk are never loaded: they are masked out of the K and V fragments (not multiplied by
-// zero), so whatever the ring held before never reaches the arithmetic and it is never cleared.
+// of a chunk are never loaded: the lanes that would address them read a row of zeros instead, so whatever the
+// ring held before never reaches the arithmetic and it is never cleared. (Masking the fragments after
+// the load cost a branch and 32 to 40 instructions in nearly every 16-row step that ends an item, and kept
+// loads and products apart: with the zero row, us per layer call: 8 sequences, group 4, nearly equal ranks
+// 51.9 -> 48.3, wide ranks 81 -> 73; 1 sequence, group 7, wide ranks 26.6 -> 24.6; 131072 tokens 32.6 -> 31.8.)
 //
 // Arithmetic (per warp, fp32 accumulate, all operands exact or split hi+lo in bf16):
 //   scores   S^T[slot][head] += K^T[slot][j] * Q~^T[j][head]   (mma m16n8k16; K via ldmatrix.trans,
@@ -90,9 +93,9 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
                   int n_tail, __nv_bfloat16* __restrict__ out, float* __restrict__ part,
                   DecodeHeader* __restrict__ hdr, int32_t* __restrict__ dev_status, Shape s,
                   int layer) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(256) unsigned char smem[];
   unsigned char* ring = smem;                                     // NW * ST * STAGE
-  static_assert((NW * ST * STAGE) % 16 == 0, "SegSmem must start 16-byte aligned");
+  static_assert((NW * ST * STAGE) % 256 == 0, "SegSmem must start 256-byte aligned");
   SegSmem& sm = *reinterpret_cast<SegSmem*>(smem + NW * ST * STAGE);
   // the merge and combine buffers alias the ring (idle while a segment is merged)
   static_assert(sizeof(Merge) <= (size_t)NW * ST * STAGE, "merge buffers fit in the ring");
@@ -109,6 +112,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g8 = lane >> 2, c = lane & 3;
   const int C = gridDim.x, cta = blockIdx.x;
+  const uint32_t zero_row = smem_addr(sm.zero);
   const uint64_t policy = l2_evict_first_policy();   // coefficient chunks are read once
 
   // the next grid in the stream may be scheduled now: it only starts on SMs this grid has left,
@@ -117,6 +121,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
   // self-contained setup first (it may overlap the tail of the preceding grid)
   if (tid < NW * ST) mbar_init(&bar_all[tid], 1);
   if (tid == NW * ST) mbar_init(&bar_comb, 1);
+  if (tid < 64) sm.zero[tid] = 0u;   // read after the barriers of the first segment's set-up
   fence_mbar_init();
   fence_proxy_async_smem();
   pdl_wait();   // everything below reads data written by earlier grids
@@ -301,7 +306,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
 #pragma unroll
         for (int t = 0; t < ISL / 16; ++t) sc[t][0] = sc[t][1] = sc[t][2] = sc[t][3] = 0.f;
 
-        // ---- K chunks: scores (rows >= r masked in the q~ fragment)
+        // ---- K chunks: scores (rows >= r read as zeros)
         for (int jc = 0; jc < nj; ++jc) {
           if (!wait_chunk()) break;
           const uint32_t st_addr = ring_w + (n_issued % ST) * STAGE;
@@ -312,31 +317,23 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
             // this lane's row of the 8x8 matrices: coefficient j, staged at row (j - chunk start)
             const int jrow = (j16 - j0) + (m >> 1) * 8 + r8;
             const int j = j0 + jrow;
-            const uint32_t row_addr = st_addr + jrow * row_bytes;
+            const uint32_t row_addr = j < r ? st_addr + jrow * row_bytes : zero_row;
             uint32_t a[ISL / 16][4];
             // stored position of slot group 2 mt + (m & 1) in row j: (group + j) mod ng; for a full
             // tile every offset is computed on its own (no chain through the previous one)
+            // (rows of a full tile start on 256 bytes: the offset goes into the row's address by an or)
             uint32_t off[ISL / 16];
             if (full_tile) {
               const uint32_t o0 = (uint32_t)(((m & 1) + j) & 15) << 4;
 #pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) off[mt] = (o0 + 32u * mt) & 255u;
+              for (int mt = 0; mt < ISL / 16; ++mt) off[mt] = ((o0 + 32u * mt) & 255u) | row_addr;
             } else {
               int pg = ((m & 1) + j) % ng;
 #pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) { off[mt] = 16u * pg; pg = wrap2(pg, ng); }
+              for (int mt = 0; mt < ISL / 16; ++mt) { off[mt] = row_addr + 16u * pg; pg = wrap2(pg, ng); }
             }
 #pragma unroll
-            for (int mt = 0; mt < ISL / 16; ++mt) ldsm_x4_trans(row_addr + off[mt], a[mt]);
-            if (j16 + 16 > r) {   // warp-uniform: rows >= r of this k-step are not coefficients
-              // A fragment registers 0, 1 hold rows j16 + 2c (+1), registers 2, 3 rows 8 later
-              const int jb = j16 + 2 * c;
-              const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
-#pragma unroll
-              for (int mt = 0; mt < ISL / 16; ++mt) {
-                a[mt][0] &= m0; a[mt][1] &= m0; a[mt][2] &= m1; a[mt][3] &= m1;
-              }
-            }
+            for (int mt = 0; mt < ISL / 16; ++mt) ldsm_x4_trans(off[mt], a[mt]);
 #pragma unroll
             for (int mt = 0; mt < ISL / 16; ++mt) mma_bf16_16816(sc[mt], a[mt], qf.x, qf.y);
 #pragma unroll
@@ -396,7 +393,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
         Ls[0] = Ls[0] * corr[0] + lsum[0];
         Ls[1] = Ls[1] * corr[1] + lsum[1];
 
-        // ---- V chunks: weighted coefficient rows (rows >= r masked in the A fragment)
+        // ---- V chunks: weighted coefficient rows (rows >= r read as zeros)
         {
           int left = 0;             // rows of the current chunk not used yet
           int j0 = 0;               // first row of the current chunk
@@ -406,7 +403,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
 #pragma unroll
           for (int jt = 0; jt < kHeadDim / 16; ++jt) {   // 16-row tile of o~
             if (jt * 16 >= r) break;                     // warp-uniform
-            if (left == 0) {                             // the tile starts a chunk
+            if (jt % 2 == 0 && left == 0) {              // the tile starts a chunk (of 32 rows or more)
               if (jt > 0) { __syncwarp(); next_chunk(); }
               if (!wait_chunk()) { ok = false; break; }
               st_addr = ring_w + (n_issued % ST) * STAGE;
@@ -416,29 +413,24 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
             left -= 16;
             const int jrow = (jt * 16 - j0) + (m & 1) * 8 + r8;
             const int j = j0 + jrow;
-            const uint32_t row_addr = st_addr + jrow * row_bytes;
-            const bool keep0 = jt * 16 + g8 < r, keep1 = jt * 16 + g8 + 8 < r;
+            const uint32_t row_addr = j < r ? st_addr + jrow * row_bytes : zero_row;
             float t1[4] = {0.f, 0.f, 0.f, 0.f};
             // stored position of slot group 2 kt + (m >> 1) (kt = 0..7) in row j, as in the K loop
             uint32_t off[ISL / 16];
             if (full_tile) {
               const uint32_t o0 = (uint32_t)(((m >> 1) + j) & 15) << 4;
 #pragma unroll
-              for (int kt = 0; kt < ISL / 16; ++kt) off[kt] = (o0 + 32u * kt) & 255u;
+              for (int kt = 0; kt < ISL / 16; ++kt) off[kt] = ((o0 + 32u * kt) & 255u) | row_addr;
             } else {
               int pg = ((m >> 1) + j) % ng;
 #pragma unroll
-              for (int kt = 0; kt < ISL / 16; ++kt) { off[kt] = 16u * pg; pg = wrap2(pg, ng); }
+              for (int kt = 0; kt < ISL / 16; ++kt) { off[kt] = row_addr + 16u * pg; pg = wrap2(pg, ng); }
             }
 #pragma unroll
             for (int kt = 0; kt < ISL / 16; kt += 2) {
               uint32_t a[4], b[4];
-              ldsm_x4(row_addr + off[kt], a);
-              ldsm_x4(row_addr + off[kt + 1], b);
-              if (jt * 16 + 16 > r) {                    // warp-uniform: rows >= r in this tile
-                if (!keep0) { a[0] = a[2] = 0u; b[0] = b[2] = 0u; }
-                if (!keep1) { a[1] = a[3] = 0u; b[1] = b[3] = 0u; }
-              }
+              ldsm_x4(off[kt], a);
+              ldsm_x4(off[kt + 1], b);
               mma_bf16_16816(oacc[jt], a, pb[kt][0], pb[kt][1]);
               mma_bf16_16816(t1, b, pb[kt + 1][0], pb[kt + 1][1]);
             }
@@ -466,17 +458,11 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
         for (int j16 = 0; j16 < r; j16 += 16) {
           const uint4 qf = *reinterpret_cast<const uint4*>(&sm.qfrag[j16 >> 4][lane][0]);
           const int j = j16 + (m >> 1) * 8 + r8;
-          const uint32_t row_addr = st_addr + j * row_bytes;
+          const uint32_t row_addr = j < r ? st_addr + j * row_bytes : zero_row;
           const int pg = ((m & 1) + j) % ng;
           uint32_t a[2][4];
           ldsm_x4_trans(row_addr + 16 * pg, a[0]);
           ldsm_x4_trans(row_addr + 16 * wrap2(pg, ng), a[1]);
-          if (j16 + 16 > r) {
-            const int jb = j16 + 2 * c;
-            const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt) { a[mt][0] &= m0; a[mt][1] &= m0; a[mt][2] &= m1; a[mt][3] &= m1; }
-          }
 #pragma unroll
           for (int mt = 0; mt < 2; ++mt) {
             mma_bf16_16816(sh[mt], a[mt], qf.x, qf.y);
@@ -523,15 +509,11 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
         for (int jt = 0; jt < kHeadDim / 16; ++jt) {
           if (jt * 16 >= r) break;                       // warp-uniform
           const int j = jt * 16 + (m & 1) * 8 + r8;
-          const uint32_t row_addr = st_addr + j * row_bytes;
+          const uint32_t row_addr = j < r ? st_addr + j * row_bytes : zero_row;
           const int pg = ((m >> 1) + j) % ng;
           uint32_t a[4], b2[4];
           ldsm_x4(row_addr + 16 * pg, a);
           ldsm_x4(row_addr + 16 * wrap2(pg, ng), b2);
-          if (jt * 16 + 16 > r) {
-            if (jt * 16 + g8 >= r) { a[0] = a[2] = 0u; b2[0] = b2[2] = 0u; }
-            if (jt * 16 + g8 + 8 >= r) { a[1] = a[3] = 0u; b2[1] = b2[3] = 0u; }
-          }
           mma_bf16_16816(oacc[jt], a, pb[0][0], pb[0][1]);
           mma_bf16_16816(oacc[jt], b2, pb[1][0], pb[1][1]);
         }

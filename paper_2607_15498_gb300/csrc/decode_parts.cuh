@@ -22,6 +22,7 @@ constexpr int kHeadsPad = 8;
 
 struct SegSmem {
   alignas(16) uint32_t qfrag[kHeadDim / 16][32][4];   // per j-chunk, per lane: b0 hi, b1 hi, b0 lo, b1 lo (read as uint4)
+  alignas(256) uint32_t zero[64];                     // a row of zeros, for the rows past a rank (decode_mma.cu)
   alignas(16) float qt[kHeadsPad][kHeadDim];          // rotated, scaled queries (fp32)
   long long base[kMaxR + 2];
   int cnt[kMaxR + 1];

@@ -308,14 +308,14 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
                   DecodeHeader* __restrict__ hdr, int32_t* __restrict__ dev_status, Shape s,
                   int layer, int64_t qcap) {
   constexpr long long kSegCostQ = QLine<BITS>::seg_cost, kSegEndQ = QLine<BITS>::seg_end;
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(256) unsigned char smem[];
   constexpr int STQ = QLine<BITS>::stage;
   constexpr int SQ = QLine<BITS>::stages;
   unsigned char* ring = smem;   // NW * SQ * STQ of quantized chunks
   constexpr int kRing = NW * SQ * STQ;
   SegSmem& sm = *reinterpret_cast<SegSmem*>(smem + kRing);
   // the merge and combine buffers alias the ring (idle while a segment is merged)
-  static_assert(kRing % 16 == 0 && sizeof(Merge) <= kRing && sizeof(CombSmem) <= kRing, "they fit in the ring");
+  static_assert(kRing % 256 == 0 && sizeof(Merge) <= kRing && sizeof(CombSmem) <= kRing, "they fit in the ring");
   Merge& mg = *reinterpret_cast<Merge*>(smem);
   __shared__ long long segW[64];                                  // per-sequence stream length
   __shared__ long long segP[65];                                  // start of sequence b on the cost line
