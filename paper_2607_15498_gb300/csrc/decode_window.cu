@@ -10,7 +10,7 @@
 // launch):
 //  1. window_qfrag_kernel: q~[rho] = U_K q[rho] * log2(e)/sqrt(d) per (sequence, KV head), written
 //     as the score-MMA B fragments (bf16 hi + lo) of each row group (the 16 rows one warp holds).
-//  2. decode_window_kernel<RG>: the coded part. The cost line of decode_common.cuh cuts every
+//  2. decode_window_kernel<RG>, RG = 1 or 2 (at most 16 or 32 rows): the coded part. The cost line of decode_common.cuh cuts every
 //     (sequence, head) stream into equal ranges over a persistent grid. The 8 warps of a CTA form
 //     8 / RG teams of RG warps; a team takes every (8 / RG)-th 128-slot item of the CTA's range and
 //     streams it once into its own shared-memory ring (1-D bulk copies, one per chunk of up to
@@ -18,6 +18,9 @@
 //     its own row group on it (warp rg of a team: n-tiles rg and rg + RG), so the coefficients are
 //     read from HBM once whatever the number of query rows. The last warp of the team to release a
 //     stage (a per-stage shared-memory count) refills it with the chunk SPT ahead.
+//     Rows of a chunk past the rank are read as zeros (a row of them in shared memory), not masked after
+//     the load: windows of 8 queries of group 4 over wide ranks 152 -> 145 us a layer, of 4 over 131072 tokens
+//     58 -> 56.
 //        scores  S^T[slot][row] += K^T[slot][j] Q~^T[j][row]   (m16n8k16, q~ split hi + lo)
 //        softmax online per row, as in the single-query kernel (lazy max with kSlack headroom)
 //        values  O~^T[j][row] += V[j][slot] P^T[slot][row]      (P in bf16)
@@ -52,13 +55,14 @@ template <int RG>
 struct WinCfg {
   static constexpr int NTEAM = NW / RG;
   // ring stages per team: about 160-192 KB of ring in all, next to RG * 8 KB of q~ fragments
-  static constexpr int SPT = RG == 1 ? 3 : (RG == 2 ? 5 : (RG == 4 ? 10 : 16));
+  static constexpr int SPT = RG == 1 ? 3 : 5;
   static constexpr int RING = NTEAM * SPT * STAGE;
   static constexpr int NBAR = NTEAM * SPT;
   static constexpr int ROWS = 16 * RG;                     // query rows a CTA can hold
 };
 
 struct WinTables {
+  alignas(256) uint32_t zero[64];   // a row of zeros, for the rows past a rank
   long long base[kMaxR + 2];
   int cnt[kMaxR + 1];
   int it_lo[kMaxR + 1];
@@ -207,10 +211,10 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
                      int ntt) {
   using Cf = WinCfg<RG>;
   constexpr int NTEAM = Cf::NTEAM, SPT = Cf::SPT;
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(256) unsigned char smem[];
   const uint32_t ring = smem_addr(smem);
   const uint4* qfs = reinterpret_cast<const uint4*>(smem + Cf::RING);
-  static_assert(Cf::RING % 16 == 0 && kQfBytes % 16 == 0, "aligned shared-memory regions");
+  static_assert(Cf::RING % 256 == 0 && kQfBytes % 256 == 0, "aligned shared-memory regions");
   WinTables& sm = *reinterpret_cast<WinTables*>(smem + Cf::RING + RG * kQfBytes);
   static_assert(sizeof(WinMerge<RG>) <= (size_t)Cf::RING, "merge buffers fit in the ring");
   WinMerge<RG>& mg = *reinterpret_cast<WinMerge<RG>*>(smem);
@@ -229,7 +233,10 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
   const bool has_b = rg + RG < ntt;   // warp-uniform: the warp's second n-tile holds rows
   const uint64_t policy = l2_evict_first_policy();
 
+  const uint32_t zero_row = smem_addr(sm.zero);
+
   pdl_trigger();
+  if (tid < 64) sm.zero[tid] = 0u;   // read after the barriers of the first segment's set-up
   if (tid < Cf::NBAR) { mbar_init(&bar[tid], 1); relc[tid] = 0u; iss[tid] = 0u; }
   if (tid == Cf::NBAR) mbar_init(&bar_q, 1);
   fence_mbar_init();
@@ -391,28 +398,22 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
           const uint4 qb = has_b ? qf_w[((j16 >> 4) * 2 + 1) * 32] : make_uint4(0u, 0u, 0u, 0u);
           const int jrow = (j16 - j0) + (m >> 1) * 8 + r8;
           const int j = j0 + jrow;
-          const uint32_t row_addr = st_addr + jrow * row_bytes;
-          uint32_t off[ISL / 16];
+          const uint32_t row_addr = j < r ? st_addr + jrow * row_bytes : zero_row;
+          uint32_t off[ISL / 16];   // rows of a full tile start on 256 bytes
           if (full_tile) {
             const uint32_t o0 = (uint32_t)(((m & 1) + j) & 15) << 4;
 #pragma unroll
-            for (int mt = 0; mt < ISL / 16; ++mt) off[mt] = (o0 + 32u * mt) & 255u;
+            for (int mt = 0; mt < ISL / 16; ++mt) off[mt] = ((o0 + 32u * mt) & 255u) | row_addr;
           } else {
             int pg = ((m & 1) + j) % ng;
 #pragma unroll
-            for (int mt = 0; mt < ISL / 16; ++mt) { off[mt] = 16u * pg; pg = wrap2(pg, ng); }
+            for (int mt = 0; mt < ISL / 16; ++mt) { off[mt] = row_addr + 16u * pg; pg = wrap2(pg, ng); }
           }
-          const bool tail_rows = j16 + 16 > r;   // warp-uniform
-          const int jb = j16 + 2 * c;
-          const uint32_t m0 = keep_rows(0xFFFFFFFFu, jb, r), m1 = keep_rows(0xFFFFFFFFu, jb + 8, r);
 #pragma unroll
           for (int h = 0; h < 2; ++h) {   // slot tiles 4h .. 4h + 3
             uint32_t a[4][4];
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              ldsm_x4_trans(row_addr + off[4 * h + t], a[t]);
-              if (tail_rows) { a[t][0] &= m0; a[t][1] &= m0; a[t][2] &= m1; a[t][3] &= m1; }
-            }
+            for (int t = 0; t < 4; ++t) ldsm_x4_trans(off[4 * h + t], a[t]);
 #pragma unroll
             for (int t = 0; t < 4; ++t) mma_bf16_16816(sc[4 * h + t][0], a[t], qa.x, qa.y);
 #pragma unroll
@@ -489,7 +490,7 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
 #pragma unroll
         for (int jt = 0; jt < kHeadDim / 16; ++jt) {
           if (jt * 16 >= r) break;   // warp-uniform
-          if (left == 0) {
+          if (jt % 2 == 0 && left == 0) {   // chunks are 32 rows or more
             if (jt > 0) release();
             if (!wait_chunk()) { ok = false; break; }
             st_addr = ring_t + (n_cons % SPT) * STAGE;
@@ -499,28 +500,23 @@ decode_window_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __re
           left -= 16;
           const int jrow = (jt * 16 - j0) + (m & 1) * 8 + r8;
           const int j = j0 + jrow;
-          const uint32_t row_addr = st_addr + jrow * row_bytes;
-          const bool keep0 = jt * 16 + g8 < r, keep1 = jt * 16 + g8 + 8 < r;
+          const uint32_t row_addr = j < r ? st_addr + jrow * row_bytes : zero_row;
           uint32_t off[ISL / 16];
           if (full_tile) {
             const uint32_t o0 = (uint32_t)(((m >> 1) + j) & 15) << 4;
 #pragma unroll
-            for (int kt = 0; kt < ISL / 16; ++kt) off[kt] = (o0 + 32u * kt) & 255u;
+            for (int kt = 0; kt < ISL / 16; ++kt) off[kt] = ((o0 + 32u * kt) & 255u) | row_addr;
           } else {
             int pg = ((m >> 1) + j) % ng;
 #pragma unroll
-            for (int kt = 0; kt < ISL / 16; ++kt) { off[kt] = 16u * pg; pg = wrap2(pg, ng); }
+            for (int kt = 0; kt < ISL / 16; ++kt) { off[kt] = row_addr + 16u * pg; pg = wrap2(pg, ng); }
           }
           float t1[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
           for (int kt = 0; kt < ISL / 16; kt += 2) {
             uint32_t a[4], a2[4];
-            ldsm_x4(row_addr + off[kt], a);
-            ldsm_x4(row_addr + off[kt + 1], a2);
-            if (jt * 16 + 16 > r) {
-              if (!keep0) { a[0] = a[2] = 0u; a2[0] = a2[2] = 0u; }
-              if (!keep1) { a[1] = a[3] = 0u; a2[1] = a2[3] = 0u; }
-            }
+            ldsm_x4(off[kt], a);
+            ldsm_x4(off[kt + 1], a2);
             mma_bf16_16816(oacc[jt][0], a, pb[kt][0][0], pb[kt][0][1]);
             mma_bf16_16816(t1[0], a2, pb[kt + 1][0][0], pb[kt + 1][0][1]);
             if (has_b) {
