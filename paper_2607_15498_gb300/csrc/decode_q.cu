@@ -606,14 +606,11 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
               v_row32<BITS>(row, pbase, c, left_r > 0 && 32 * c < tl, o0);
               v_row32<BITS>(row + 8 * qrow, pbase, c, left_r > 8 && 32 * c < tl, o1);
               row += 16 * qrow;
-              float t1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
               for (int kt = 0; kt < ISL / 16; ++kt) {
                 const uint32_t a[4] = {o0[2 * kt], o1[2 * kt], o0[2 * kt + 1], o1[2 * kt + 1]};
-                mma_f16_16816(kt & 1 ? t1 : oacc[jt], a, pb[kt][0], pb[kt][1]);
+                mma_f16_16816(oacc[jt], a, pb[kt][0], pb[kt][1]);
               }
-#pragma unroll
-              for (int e = 0; e < 4; ++e) oacc[jt][e] += t1[e];
             }
             left -= 32;
             if (left == 0 || jp * 32 + 32 >= r) {        // the chunk's last rows
