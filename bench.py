@@ -593,7 +593,7 @@ def sweep_quant(V, wl, dev, peak, stream, decode_steps, bits_list=(4, 8)):
             "decode_gbs": round(gbs, 1), "decode_frac_of_hbm_peak": round(gbs / peak, 4),
             "decode_status": V.status_string(int(status.item())),
             "decode_kernels": "per layer call: one fused kernel reading only the codes and their "
-                              "group parameters, dequantized in each warp's ring into fp16 tiles; "
+                              "group parameters, expanded into fp16 fragments in registers; "
                               "graph-replayed"}
         del g, qp
     res["workload"] = workload_desc(wl)
@@ -637,7 +637,7 @@ def sweep_anchor_search(V, wl, dev, stream, stride=16, c=4):
            "tflops": round(tflops, 1), "frac_of_bf16_peak": round(tflops / tf_peak, 4),
            "status": V.status_string(int(status.item())),
            "kernels": "per call: a norm and anchor-copy pass over K and V, then the tcgen05 search "
-                      "(M = 128 tokens x N = 256 anchors, K = D, TMA-fed); the time and the TFLOP/s "
+                      "(M = 256 tokens of a CTA pair x N = 256 anchors, K = D, TMA-fed); the time and the TFLOP/s "
                       "cover both"}
     del k, v, idx, dist, ws
     torch.cuda.empty_cache()
@@ -678,7 +678,7 @@ def sweep_anchor_residual(V, wl, dev, peak, stream, stride=16, c=4):
     res = {"workload": workload_desc(wl), "stride": stride, "c": c, "ms_per_layer": round(ms / units, 4),
            "bytes_per_layer": int(nbytes // units), "gbs": round(gbs, 1),
            "frac_of_hbm_peak": round(gbs / peak, 4), "status": V.status_string(int(status.item())),
-           "kernels": "one residual kernel per call (a warp per token), on the lists of one search call "
+           "kernels": "one residual kernel per call (anchors in shared memory), on the lists of one search call "
                       "made before the timed calls"}
     del k, v, idx, e
     torch.cuda.empty_cache()

@@ -1,5 +1,5 @@
 // Parts shared by the fused tensor-core decode kernels (bf16 coefficients: decode_mma.cu;
-// group-quantized coefficients dequantized in the ring: decode_q.cu): the warp layout, the
+// group-quantized coefficients expanded in registers: decode_q.cu): the warp layout, the
 // per-segment shared-memory tables, the query rotation, the completion-counting header and the
 // cross-CTA combine.
 #pragma once

@@ -1,6 +1,6 @@
 // Step 4 on a group-quantized cache (Sec. 3.3, "Composability": the stored coefficients are
 // quantized without changing the allocation) — the fused tensor-core decode of decode_mma.cu with
-// the coefficients dequantized inside each warp's ring, so a layer call reads the b-bit codes from
+// the coefficients expanded from each warp's ring, so a layer call reads the b-bit codes from
 // HBM (31.5 % of the bf16 footprint at 4 bits, 56.5 % at 8) and nothing else of the cache.
 //
 // Same work split, cost line, online softmax, merge and combine as the bf16 kernel (the shared
@@ -517,7 +517,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
 #pragma unroll
         for (int t = 0; t < ISL / 16; ++t) sc[t][0] = sc[t][1] = sc[t][2] = sc[t][3] = 0.f;
 
-        // ---- K chunks: scores (rows >= r masked in the q~ fragment)
+        // ---- K chunks: scores (rows >= r as zeros)
         for (int jc = 0; jc < nj; ++jc) {
           if (!wait_chunk()) break;
           const int j0 = jc << lgc, j1 = min(r, j0 + (1 << lgc));
@@ -586,7 +586,7 @@ decode_q_kernel(const uint8_t* __restrict__ qdata, const int32_t* __restrict__ b
         Ls[0] = Ls[0] * corr[0] + lsum[0];
         Ls[1] = Ls[1] * corr[1] + lsum[1];
 
-        // ---- V chunks: weighted coefficient rows (rows >= r masked in the A fragment)
+        // ---- V chunks: weighted coefficient rows (rows >= r as zeros)
         {
           int left = 0;             // rows of the current chunk not used yet
           uint32_t row = 0;         // this lane's row of the next 16-row tile

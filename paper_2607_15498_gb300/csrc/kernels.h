@@ -83,7 +83,7 @@ int launch_decode_window(const Shape& s, const varrate_packed& c, const void* ba
 int launch_quantize(const Shape& s, const varrate_packed& in, const varrate_qpacked& out,
                     int32_t* dev_status, int num_sms, cudaStream_t st);
 // Fused decode on a group-quantized cache (decode_q.cu): the bf16 kernel's work split with the
-// codes dequantized in each warp's ring. Workspace: that of the bf16 fused decode (header, then
+// codes expanded into tensor-core fragments in registers. Workspace: that of the bf16 fused decode (header, then
 // the partials). Shapes it does not take run the general kernels on x^ (launch_decode_q,
 // decode.cu).
 bool decode_q_supported(const Shape& s, int bits, int64_t qcap, int n_tail, int num_sms);
