@@ -111,6 +111,7 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
     return;
   }
 
+  cluster.barrier_arrive();   // this CTA runs: the others may write its shared memory once they have waited
   // min / max over the coded set (exact in any order), and the sum, which only places the first levels
   float mn = INFINITY, mx = -INFINITY, sum = 0.f;
   const bool uniform = (s.mode == VARRATE_UNIFORM) || sl == nullptr;
@@ -124,18 +125,19 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
     }
     warp_stats(mn, mx, sum);
     if (lane == 0) { sm.fred[0][warp] = mn; sm.fred[1][warp] = mx; sm.fred[2][warp] = sum; }
-    __syncthreads();
-    if (warp == 0) {
-      mn = lane < kWarps ? sm.fred[0][lane] : INFINITY;
-      mx = lane < kWarps ? sm.fred[1][lane] : -INFINITY;
-      sum = lane < kWarps ? sm.fred[2][lane] : 0.f;
-      warp_stats(mn, mx, sum);
-      if (lane < C) {
-        float* peer = cluster.map_shared_rank(&sm.mm[0][0], lane) + 3 * rank;
-        peer[0] = mn;
-        peer[1] = mx;
-        peer[2] = sum;
-      }
+  }
+  __syncthreads();
+  cluster.barrier_wait();     // every CTA of the cluster has started
+  if (!uniform && warp == 0) {
+    mn = lane < kWarps ? sm.fred[0][lane] : INFINITY;
+    mx = lane < kWarps ? sm.fred[1][lane] : -INFINITY;
+    sum = lane < kWarps ? sm.fred[2][lane] : 0.f;
+    warp_stats(mn, mx, sum);
+    if (lane < C) {
+      float* peer = cluster.map_shared_rank(&sm.mm[0][0], lane) + 3 * rank;
+      peer[0] = mn;
+      peer[1] = mx;
+      peer[2] = sum;
     }
   }
   cluster.sync();
