@@ -59,6 +59,7 @@ pack_tables_kernel(const uint8_t* __restrict__ ranks, int32_t* __restrict__ buck
   const int64_t w0 = min(c1, c0 + warp * wshare), w1 = min(c1, w0 + wshare);
   const uint8_t* rk = ranks + bl * s.N;
 
+  cluster.barrier_arrive();   // this CTA runs: the others may write its shared memory once they have waited
   for (int i = tid; i < kTabWarps * (kMaxR + 1); i += kTabThreads) (&sm.wcnt[0][0])[i] = 0;
   if (tid == 0) sm.bad = 0;
   __syncthreads();
@@ -74,6 +75,7 @@ pack_tables_kernel(const uint8_t* __restrict__ ranks, int32_t* __restrict__ buck
     }
   }
   __syncthreads();
+  cluster.barrier_wait();     // every CTA of the cluster has started
   if (tid <= kMaxR + 1) {
     int v = tid > kMaxR ? sm.bad : 0;
     if (tid <= kMaxR) {

@@ -24,7 +24,7 @@ def kernel_body(file, kernel):
     raise AssertionError("unbalanced braces")
 
 
-@pytest.mark.parametrize("file, kernel", [("allocate.cu", "allocate_kernel"),
+@pytest.mark.parametrize("file, kernel", [("allocate.cu", "allocate_kernel"), ("pack.cu", "pack_tables_kernel"),
                                           ("anchor_search.cu", "anchor_search_tc_kernel")])
 def test_remote_shared_memory_after_a_cluster_barrier(file, kernel):
     body = kernel_body(file, kernel)
