@@ -624,7 +624,8 @@ struct CombineSmem {
   alignas(16) __nv_bfloat16 vs[kTT * kRowStride];        // tail values of the step
   alignas(16) float os[kCombRows][kHeadDim + 8];         // merged o~ per row
   float ws[kCombRows][kWStride];                         // tail scores, then tail weights, of the step
-  float fs[kCombRows];                                   // factor of the rows' earlier sums
+  float fs[kCombRows];                                   // factor of the rows' earlier sums, of the step
+  float ff[kCombRows];                                   // factor of o~ against the final reference
   float ls[kCombRows];                                   // softmax normaliser
 };
 
@@ -808,11 +809,12 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
   }
   cp_async_wait<0>();
   if (lane == 0) {
-    cs.fs[warp] = M0 == -INFINITY ? 0.f : exp2f(M0 - M);   // o~ against the final reference
+    // not into fs: another warp may still read the last step's factors
+    cs.ff[warp] = M0 == -INFINITY ? 0.f : exp2f(M0 - M);
     cs.ls[warp] = L;
   }
   __syncthreads();
-  const float fr = cs.fs[g8];
+  const float fr = cs.ff[g8];
 #pragma unroll
   for (int ks = 0; ks < kHeadDim / 16; ++ks) {
     uint32_t a[4], h0, l0, h1, l1;

@@ -124,6 +124,28 @@ def test_window_deterministic_and_workspace_reuse(caches):
     assert torch.equal(a, b)
 
 
+def test_window_long_tail_with_early_maximum(caches):
+    """Three steps of the combine over the tail, the first of which raises every row's maximum far above that of the
+    coded part: the factor of the last step differs from that of the coded part in every row. Many runs, equal bits."""
+    c = caches["llama"]
+    wl, cfg = c["wl"], c["cfg"]
+    n_q, n_tail = 8, 300
+    q, tk, tv = _window_inputs(wl, 1, n_q, n_tail, 11)
+    tk[:, :, :n_q * wl.group] = 2 * q.view(wl.batch, n_q, wl.n_kv_heads, wl.group, -1).permute(0, 2, 1, 3, 4).flatten(2, 3)
+    out, st = gpu_window(cfg, c["packed"], c["bk"], c["bv"], q, 1, tk, tv)
+    assert st == V.OK
+    got = f64(out)
+    for b in range(wl.batch):
+        ref = c["refs"][b][1]
+        want = O.decode_window(f64(q[b]), ref["coef_k"], ref["coef_v"], ref["ranks"],
+                               f64(c["bk"][1]), f64(c["bv"][1]), f64(tk[b]), f64(tv[b]))
+        for i in range(n_q):
+            assert decode_close(got[b, i], want[i], cfg), (b, i, decode_errors(got[b, i], want[i]))
+    for _ in range(50):
+        again, st = gpu_window(cfg, c["packed"], c["bk"], c["bv"], q, 1, tk, tv)
+        assert st == V.OK and torch.equal(out, again)
+
+
 def test_window_tail_only():
     """Empty coded set: the whole context is the exact window, plus the exact tail."""
     wl = synth.workload("llama1", n_kv_heads=2, n_ctx=32, window=32, batch=2)

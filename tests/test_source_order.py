@@ -1,5 +1,6 @@
 """Orders that the kernels' sources have to keep and that no run can be relied on to show: another CTA's shared
-memory is written only after a cluster barrier has shown that every CTA of the cluster runs."""
+memory is written only after a cluster barrier has shown that every CTA of the cluster runs, and no shared array
+is written by one warp while another may still read it."""
 import os
 import re
 
@@ -34,3 +35,42 @@ def test_remote_shared_memory_after_a_cluster_barrier(file, kernel):
     assert starts, "no cluster barrier before the first access to another CTA's shared memory"
     # and one that every thread passes: not inside a conditional block
     assert any(before[:s].count("{") == before[:s].count("}") for s in starts)
+
+
+def _accesses(statement):
+    """(array, index, is_write) of the combine's shared arrays in one statement: what stands left of an assignment,
+    or is a destination of `stage`, is written."""
+    left, eq, right = statement.partition(" = ")
+    found = []
+    for part, write in ((left, bool(eq)), (right, False)):
+        for m in re.finditer(r"cs\.(\w+)(?:\[([^\]]*)\])?", part):
+            found.append((m.group(1), m.group(2), write or part[:m.start()].rstrip().endswith("stage(")))
+    return found
+
+
+def test_window_combine_shared_arrays_between_barriers():
+    """Run the source of the combine by statements, its loop over the tail twice, and collect what each stretch
+    between two block barriers touches. A thread-private place (the warp's own row) may be written and read in one
+    stretch; anything else that is written in a stretch may not be read in it. The barrier at the end of the loop's
+    body stands in a condition that holds on every pass but the last."""
+    body = kernel_body("decode_window.cu", "window_combine_kernel")
+    loop = body.index("for (int t0 = 0;")
+    end, depth = body.index("{", loop), 0
+    for end in range(end, len(body)):
+        depth += {"{": 1, "}": -1}.get(body[end], 0)
+        if depth == 0:
+            break
+    head, step, rest = body[:loop], body[body.index("{", loop) + 1:end], body[end + 1:]
+    again = step.index("if (t0 + kTT < vis_max)")
+    stretches = [[]]
+    for text in (head, step, step[:again], rest):
+        for statement in re.split(r"[;{}]", text):
+            if "__syncthreads()" in statement:
+                stretches.append([])
+            else:
+                stretches[-1] += _accesses(statement)
+    assert sum(len(s) for s in stretches) > 20 and len(stretches) > 7
+    for s in stretches:
+        for array, index, _ in (a for a in s if a[2]):
+            others = [(i, w) for x, i, w in s if x == array and i != index]
+            assert not others, f"cs.{array}[{index}] is written while cs.{array}{others} may be in use"
