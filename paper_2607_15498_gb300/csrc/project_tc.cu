@@ -7,7 +7,8 @@
 // (sequence, layer, head, K-or-V) stream and runs three warp roles over a 4-stage ring:
 //   producer (4 warps)   read the tile's tokens from perm (one tile ahead) and copy their rows with 16-byte
 //                        cp.async (two whole rows an instruction) into the 128-byte-swizzled K-major
-//                        layout of the tensor core, three tiles in flight;
+//                        layout of the tensor core; the copies arrive on the stage's barrier themselves
+//                        when they land, so up to four tiles are in flight;
 //   mma (1 thread)       8 x tcgen05.mma (M = 128 slots, N = r rounded up to 16, K = 16) with U (128 x
 //                        128, resident in shared memory) as B, into one of four TMEM accumulators;
 //                        tcgen05.commit frees the stage and hands the accumulator on;
@@ -22,6 +23,9 @@
 // 376 / 95 us (floor 49 us at the copy bandwidth); 1 layer x 8 heads x 32768, 5 % outliers 76 / 48 us; 2 x
 // 8 x 131072, wide 505 / 234 us; 32 x 8 x 32768, ranks within a few units of each other 832 / 894 us. TMA
 // gathers of four rows as the producer: 190, 95, 612 and 2432 us (about 85 cycles a gather on an SM).
+// With the producers waiting for a tile's copies and fencing before they handed it on (the fence also waits for
+// the copies of later tiles) 32 x 8 x 32768 tokens of one rank took 870 us, now 819; ranks from r_min to d 64 x 8 x
+// 16384 1487 / 1396, 16 x 8 x 600 118 / 105 (launch times).
 // Every mbarrier wait is bounded; a timeout raises VARRATE_ERR_TIMEOUT.
 #include "common.cuh"
 #include "kernels.h"
@@ -39,7 +43,6 @@ constexpr int kEpi = 4 * NGRP;             // epilogue warps
 constexpr int NACC = 4;                    // TMEM accumulators of 128 columns (all 512 columns)
 constexpr int kProd = 4;                   // producer warps (32 slots each)
 constexpr int kThreads = (kEpi + kProd + 1) * 32;   // + MMA warp
-constexpr int kAhead = NST - 1;            // tiles whose copies are in flight
 constexpr int STG_BYTES = 32 * TM * 2;     // staging block: 32 coefficient rows
 constexpr uint32_t kWaitTries = 1u << 22;  // bounded mbarrier polls
 
@@ -63,6 +66,12 @@ template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read %0;\n" ::"n"(N) : "memory");
 }
+
+// This thread's copies issued so far arrive on `bar` (counted among its expected arrivals) when they have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // Bucket of tile T, searched upward from r (tiles are visited in increasing order).
 __device__ __forceinline__ int bucket_of(const int* tile_pre, int T, int r) {
@@ -176,16 +185,9 @@ project_tc_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __re
         if (row0 + sub < ni)
           cp_async16(dst + sw128_offset(row0 + sub, lane & 15, TM), src + (int64_t)t * (kHeadDim * 2), 16);
       }
-      cp_async_commit();
-      if (i >= kAhead) {   // the copies of tile i - kAhead have landed: hand it to the tensor core
-        cp_async_wait<kAhead>();
-        fence_proxy_async_smem();
-        mbar_arrive(&sm.full[(i - kAhead) % NST]);
-      }
+      cp_async_arrive(&sm.full[st]);
     }
-    cp_async_wait<0>();     // also after a wait that gave up: nothing is in flight when the block ends
-    fence_proxy_async_smem();
-    for (int j = max(0, i - kAhead); j < i; ++j) mbar_arrive(&sm.full[j % NST]);
+    cp_async_wait_all();    // also after a wait that gave up: nothing is in flight when the block ends
   } else if (warp == kEpi + kProd) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -199,6 +201,7 @@ project_tc_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __re
           mbar_wait_bounded(&sm.drain, 0, kWaitTries);
           break;
         }
+        fence_proxy_async_smem();   // the rows were copied by ordinary (generic) writes
         tc_fence_after();
         r = bucket_of(sm.tile_pre, x0 + i * dx, r);
         const uint32_t idesc = idesc_bf16_f32(TM, (r + 15) & ~15);   // rows of U past r are not needed
