@@ -202,6 +202,7 @@ varrate_status varrate_pack(const varrate_config* cfg, const void* k, const void
   if (!k || !v || !basis_k || !basis_v || !packed_ok(cfg, out)) return VARRATE_ERR_ARG;
   if (!aligned16({k, v, basis_k, basis_v, dev_status})) return VARRATE_ERR_ARG;
   const Shape s = make_shape(cfg, out->cap_elems);
+  if (!vr::pack_ready(s, k, v)) return VARRATE_ERR_CUDA;   // before anything is enqueued
   if (vr::launch_pack(s, k, v, basis_k, basis_v, *out, dev_status, num_sms(), (cudaStream_t)stream) < 0)
     return VARRATE_ERR_CUDA;
   return launched();
@@ -220,6 +221,7 @@ varrate_status varrate_encode(const varrate_config* cfg, const void* q_win, cons
   const size_t need = ws_bytes(cfg, VARRATE_CALL_ENCODE);
   if (ws_bytes_ < need || ws == nullptr) return VARRATE_ERR_WORKSPACE;
   const Shape s = make_shape(cfg, out->cap_elems);
+  if (!vr::pack_ready(s, k, v)) return VARRATE_ERR_CUDA;   // before anything is enqueued
   const int sms = num_sms();
   cudaStream_t cs = (cudaStream_t)stream;
   char* w = static_cast<char*>(ws);

@@ -63,6 +63,8 @@ def _ranks(kind, pairs, n, r_min, rng):
         return np.clip(np.rint(22 + 2 * rng.standard_normal((pairs, n))), r_min, 128).astype(np.int64)
     if kind == "one":
         return np.full((pairs, n), 37)
+    if kind == "mixed":   # pairs that the projection takes by token and by tile in one call
+        return np.concatenate([_ranks(k, 1, n, r_min, rng) for k in ("one", "wide", "ends", "narrow")])[:pairs]
     return np.where(rng.random((pairs, n)) < 0.01, 128, r_min)   # "ends"
 
 
@@ -71,6 +73,15 @@ def _ranks(kind, pairs, n, r_min, rng):
 @pytest.mark.parametrize("n, pairs", [(9, 1), (127, 2), (129, 1), (2049, 3), (4097, 1), (8200, 1), (17001, 1),
                                       (1500, 160)])
 def test_pack_split_edges(n, pairs, kind, dtype):
+    _check_pack(n, pairs, kind, dtype)
+
+
+@pytest.mark.parametrize("n", [700, 5003, 8200])
+def test_pack_mixed_forms(n):
+    _check_pack(n, 4, "mixed", "bf16")
+
+
+def _check_pack(n, pairs, kind, dtype):
     """Tables bit for bit; coefficients within their storage rounding; every element of the buckets
     written (the buffer starts as NaN) and every padding slot zero."""
     if pairs > 100 and (kind != "wide" or dtype == "f32"):
