@@ -622,22 +622,26 @@ struct CombineSmem {
   alignas(16) __nv_bfloat16 us[kHeadDim * kRowStride];   // U_V[j][col]
   alignas(16) __nv_bfloat16 ks[kTT * kRowStride];        // tail keys of the step
   alignas(16) __nv_bfloat16 vs[kTT * kRowStride];        // tail values of the step
-  alignas(16) float os[kCombRows][kHeadDim + 8];         // merged o~ per row
-  float ws[kCombRows][kWStride];                         // tail scores, then tail weights, of the step
+  alignas(16) float os[kHeadDim][kCombRows];             // merged o~, by coordinate
+  alignas(16) float wt[kTT][kCombRows];                  // tail weights of the step, by token
+  float ws[kCombRows][kWStride];                         // tail scores of the step
   float fs[kCombRows];                                   // factor of the rows' earlier sums, of the step
   float ff[kCombRows];                                   // factor of o~ against the final reference
-  float ls[kCombRows];                                   // softmax normaliser
 };
 
 // grid (B G, ceil(R / 8)), 256 threads: rows 8 blockIdx.y .. + 7 of one (sequence, KV head). part slots as
 // written above; out is [B][n_q][H][d]. Warp w merges the partials of row w: the maxima and sums one CTA a
 // lane, then the weighted sums with eight 16-byte loads in flight. The tail goes 128 tokens at a time, on
 // tensor cores: scores as m16n8k16 tiles (16 tokens x 8 rows, exact bf16 products, fp32 sums) with the causal
-// cut, the online softmax by row, values as further k-steps of the rotation back,
-//   out^T[col][row] = sum_j U_V[j][col] o~[row][j] + sum_t v_t[col] w[row][t],
-// warp w owning columns 16 w .. 16 w + 15, with o~ and w split hi + lo in bf16. Bound by latency.
-// 8 heads, 19 partials a row: 128 rows and 32 tail tokens 27 us with scalar loops over partials, tail and
-// basis rows, 12 us now; 32 rows and 300 tail tokens 67 / 15 us.
+// cut, the online softmax by row. Values and the rotation back,
+//   out[row][col] = sum_t w[row][t] v_t[col] + sum_j o~[row][j] U_V[j][col],
+// in fp32: warp w takes every 8th token and basis row for all rows, lane l columns 4 l .. 4 l + 3, and the
+// warps' sums are added at the end.
+// Bound by latency.
+// 8 heads, 19 partials a row, launch times: 128 rows and 32 tail tokens 27 us with scalar loops over partials, tail
+// and basis rows, 12 us now; 32 rows and 300 tail tokens 67 / 17.5 us. With values and rotation as tensor-core steps
+// on o~ and w in two bf16 parts (about 16 bits) 12 and 16.4 us, but whole calls on two layers took longer: 245
+// against 234 us and 112 against 101.
 __global__ void __launch_bounds__(256)
 window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict__ bucket_base,
                       const __nv_bfloat16* __restrict__ basis_v, const __nv_bfloat16* __restrict__ q,
@@ -736,12 +740,29 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
         }
       }
     }
-    *reinterpret_cast<float4*>(&cs.os[warp][4 * lane]) = o;
+    cs.os[4 * lane][warp] = o.x;
+    cs.os[4 * lane + 1][warp] = o.y;
+    cs.os[4 * lane + 2][warp] = o.z;
+    cs.os[4 * lane + 3][warp] = o.w;
   }
   const float M0 = M;
   const float scale = kLog2e * rsqrtf((float)kHeadDim);
-  const int col0 = warp * 16, col = col0 + ((lane >> 3) & 1) * 8, jr = (lane & 7) + ((lane >> 4) & 1) * 8;
-  float d[2][4] = {};   // this warp's 16 columns x 8 rows: sums with the hi and with the lo parts
+  float acc[kCombRows][4] = {};   // this warp's share of the rows' sums, columns 4 lane .. 4 lane + 3
+  auto add_row = [&](const __nv_bfloat16* v, const float (&w)[kCombRows]) {
+    const uint2 u = *reinterpret_cast<const uint2*>(v + 4 * lane);
+    const float x[4] = {__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                        __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u)};
+#pragma unroll
+    for (int r = 0; r < kCombRows; ++r)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[r][i] = fmaf(w[r], x[i], acc[r][i]);
+  };
+  auto load_rows = [&](const float* p, float (&w)[kCombRows]) {
+    const float4 a = *reinterpret_cast<const float4*>(p), c4 = *reinterpret_cast<const float4*>(p + 4);
+    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+    w[4] = c4.x; w[5] = c4.y; w[6] = c4.z; w[7] = c4.w;
+  };
+  static_assert(kCombRows == 8, "a row of weights is two 16-byte loads");
   for (int t0 = 0; t0 < vis_max; t0 += kTT) {
     cp_async_wait<0>();
     __syncthreads();
@@ -774,7 +795,7 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
 #pragma unroll
       for (int k = 0; k < kTT / 32; ++k) {
         const float w = x[k] == -INFINITY ? 0.f : exp2f(x[k] - nm);
-        cs.ws[warp][lane + 32 * k] = w;
+        cs.wt[lane + 32 * k][warp] = w;
         lt += w;
       }
 #pragma unroll
@@ -785,18 +806,17 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
       if (lane == 0) cs.fs[warp] = f;
     }
     __syncthreads();
-    {   // values: 16 tokens per k-step
-      const float f0 = cs.fs[2 * c], f1 = cs.fs[2 * c + 1];
+    {   // values
 #pragma unroll
-      for (int h = 0; h < 2; ++h) { d[h][0] *= f0; d[h][1] *= f1; d[h][2] *= f0; d[h][3] *= f1; }
-      for (int ts = 0; ts < (n + 15) / 16; ++ts) {
-        uint32_t a[4], h0, l0, h1, l1;
-        ldsm_x4_trans(smem_addr(&cs.vs[(ts * 16 + jr) * kRowStride + col]), a);
-        const int tb = ts * 16 + 2 * c;
-        split_bf16(cs.ws[g8][tb], cs.ws[g8][tb + 1], h0, l0);
-        split_bf16(cs.ws[g8][tb + 8], cs.ws[g8][tb + 9], h1, l1);
-        mma_bf16_16816(d[0], a, h0, h1);
-        mma_bf16_16816(d[1], a, l0, l1);
+      for (int r = 0; r < kCombRows; ++r) {
+        const float f = cs.fs[r];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[r][i] *= f;
+      }
+      for (int t = warp; t < n; t += 8) {
+        float w[kCombRows];
+        load_rows(cs.wt[t], w);
+        add_row(&cs.vs[t * kRowStride], w);
       }
     }
     if (t0 + kTT < vis_max) {
@@ -808,29 +828,38 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
     }
   }
   cp_async_wait<0>();
-  if (lane == 0) {
-    // not into fs: another warp may still read the last step's factors
-    cs.ff[warp] = M0 == -INFINITY ? 0.f : exp2f(M0 - M);
-    cs.ls[warp] = L;
-  }
+  // not into fs: another warp may still read the last step's factors
+  if (lane == 0) cs.ff[warp] = M0 == -INFINITY ? 0.f : exp2f(M0 - M);
   __syncthreads();
-  const float fr = cs.ff[g8];
+  {   // rotation back: basis rows warp, warp + 8, ...
+    float f[kCombRows];
 #pragma unroll
-  for (int ks = 0; ks < kHeadDim / 16; ++ks) {
-    uint32_t a[4], h0, l0, h1, l1;
-    ldsm_x4_trans(smem_addr(&cs.us[(ks * 16 + jr) * kRowStride + col]), a);
-    const int jb = ks * 16 + 2 * c;
-    split_bf16(cs.os[g8][jb] * fr, cs.os[g8][jb + 1] * fr, h0, l0);
-    split_bf16(cs.os[g8][jb + 8] * fr, cs.os[g8][jb + 9] * fr, h1, l1);
-    mma_bf16_16816(d[0], a, h0, h1);
-    mma_bf16_16816(d[1], a, l0, l1);
+    for (int r = 0; r < kCombRows; ++r) f[r] = cs.ff[r];
+#pragma unroll 4
+    for (int j = warp; j < kHeadDim; j += 8) {
+      float w[kCombRows];
+      load_rows(cs.os[j], w);
+#pragma unroll
+      for (int r = 0; r < kCombRows; ++r) w[r] *= f[r];
+      add_row(&cs.us[j * kRowStride], w);
+    }
   }
+  float4* sums = reinterpret_cast<float4*>(cs.ks);   // [warp][row][lane]: the keys are done with
+  static_assert(sizeof(cs.ks) >= 8 * kCombRows * 32 * sizeof(float4), "the warps' sums fit");
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {   // columns col0 + g8 (+ 8), rows 2c, 2c + 1
-    const int lr = 2 * c + (e & 1), r = row0 + lr;
-    if (r < R)
-      out[(((long long)b * n_q + r / s.grp) * s.H + (long long)g * s.grp + r % s.grp) * kHeadDim + col0 + g8 + (e >> 1) * 8] =
-          __float2bfloat16_rn((d[0][e] + d[1][e]) / cs.ls[lr]);
+  for (int r = 0; r < kCombRows; ++r) sums[(warp * kCombRows + r) * 32 + lane] = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
+  __syncthreads();
+  if (valid) {
+    float4 y = sums[warp * 32 + lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+      const float4 x = sums[(k * kCombRows + warp) * 32 + lane];
+      y.x += x.x; y.y += x.y; y.z += x.z; y.w += x.w;
+    }
+    uint2 u;
+    u.x = pack_bf16(y.x / L, y.y / L);
+    u.y = pack_bf16(y.z / L, y.w / L);
+    *reinterpret_cast<uint2*>(out + (((long long)b * n_q + rho / s.grp) * s.H + (long long)g * s.grp + rho % s.grp) * kHeadDim + 4 * lane) = u;
   }
 }
 

@@ -146,6 +146,44 @@ def test_window_long_tail_with_early_maximum(caches):
         assert st == V.OK and torch.equal(out, again)
 
 
+def _nearly_cancelling_tail(seed):
+    """One query, four tail tokens: the first two values cancel to 2^-9, the third what is left to 2^-18, and the fourth
+    adds a result of 2^-12 of their size. The cached token has no weight to speak of."""
+    rng = np.random.default_rng(seed)
+    bf = lambda x: torch.as_tensor(x).to(torch.bfloat16).double().numpy()
+    q = bf(rng.standard_normal(128))
+    tk = bf(rng.uniform(0.0, 0.3, (4, 1)) * q * np.sqrt(128) / (q @ q))
+    w = np.exp(tk @ q / np.sqrt(128))
+    tv = np.zeros((4, 128))
+    tv[0] = bf(rng.standard_normal(128))
+    tv[1] = bf(-w[0] * tv[0] / w[1])
+    tv[2] = bf(-(w[:2] @ tv[:2]) / w[2])
+    tv[3] = bf(2.0 ** -12 * rng.standard_normal(128))
+    k = bf(-40 * q * np.sqrt(128) / (q @ q))[None]
+    return q, tk, tv, k, w
+
+
+@pytest.mark.parametrize("seed", [8, 12, 14, 15])   # two parts miss the bar by 2.7 to 4 times there
+def test_window_tail_sums_are_fp32(vlib, seed):
+    """Weights and values of the exact tail are multiplied and added in fp32. Bar: half a bf16 step of the result (2^-8) and
+    2^-21 of sum p |v| (exp2f is within 2 ulp, 2^-22, and so are the four-term sums; two bf16 parts of a weight would
+    be within 2^-18 each and miss it)."""
+    q, tk, tv, k, w = _nearly_cancelling_tail(seed)
+    cfg = V.make_config(1, 1, 1, 1, budget_frac=1.0, window=1)
+    t = lambda x: torch.as_tensor(x).to(torch.bfloat16)
+    eye = torch.eye(128).to(torch.bfloat16)[None, None]
+    kv = t(k).view(1, 1, 1, 1, 128)
+    packed, st = gpu_pack(cfg, np.full((1, 1, 1), 128), kv, kv, eye, eye)
+    assert st == V.OK
+    # the last of the four is the query's own token
+    out, st = gpu_window(cfg, packed, eye, eye, t(q).view(1, 1, 1, 128), 0, t(tk).view(1, 1, 4, 128), t(tv).view(1, 1, 4, 128))
+    assert st == V.OK
+    p = w / w.sum()
+    want = p @ tv
+    bar = 2.0 ** -8 * 1.01 * np.abs(want) + 2.0 ** -21 * (p @ np.abs(tv))
+    assert (np.abs(f64(out).reshape(128) - want) <= bar).all()
+
+
 def test_window_tail_only():
     """Empty coded set: the whole context is the exact window, plus the exact tail."""
     wl = synth.workload("llama1", n_kv_heads=2, n_ctx=32, window=32, batch=2)

@@ -72,5 +72,5 @@ def test_window_combine_shared_arrays_between_barriers():
     assert sum(len(s) for s in stretches) > 20 and len(stretches) > 7
     for s in stretches:
         for array, index, _ in (a for a in s if a[2]):
-            others = [(i, w) for x, i, w in s if x == array and i != index]
-            assert not others, f"cs.{array}[{index}] is written while cs.{array}{others} may be in use"
+            read = [i for x, i, written in s if x == array and i != index and not written]
+            assert not read, f"cs.{array}[{index}] is written while cs.{array}{read} may be read"
