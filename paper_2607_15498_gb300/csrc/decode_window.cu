@@ -636,7 +636,7 @@ struct CombineSmem {
 // cut, the online softmax by row. Values and the rotation back,
 //   out[row][col] = sum_t w[row][t] v_t[col] + sum_j o~[row][j] U_V[j][col],
 // in fp32: warp w takes every 8th token and basis row for all rows, lane l columns 4 l .. 4 l + 3, and the
-// warps' sums are added at the end.
+// warps' sums are added at the end. A row leaves out the tokens after its own (their values may be anything).
 // Bound by latency.
 // 8 heads, 19 partials a row, launch times: 128 rows and 32 tail tokens 27 us with scalar loops over partials, tail
 // and basis rows, 12 us now; 32 rows and 300 tail tokens 67 / 17.5 us. With values and rotation as tensor-core steps
@@ -747,6 +747,7 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
   }
   const float M0 = M;
   const float scale = kLog2e * rsqrtf((float)kHeadDim);
+  const int vis_min = n_tail - n_q + row0 / s.grp + 1;   // tail tokens every row of the CTA sees
   float acc[kCombRows][4] = {};   // this warp's share of the rows' sums, columns 4 lane .. 4 lane + 3
   auto add_row = [&](const __nv_bfloat16* v, const float (&w)[kCombRows]) {
     const uint2 u = *reinterpret_cast<const uint2*>(v + 4 * lane);
@@ -813,10 +814,27 @@ window_combine_kernel(const float* __restrict__ part, const int64_t* __restrict_
 #pragma unroll
         for (int i = 0; i < 4; ++i) acc[r][i] *= f;
       }
-      for (int t = warp; t < n; t += 8) {
+      const int whole = min(n, vis_min - t0);   // at most 7 tokens of the last rows' own come after these
+      int t = warp;
+      for (; t < whole; t += 8) {
         float w[kCombRows];
         load_rows(cs.wt[t], w);
         add_row(&cs.vs[t * kRowStride], w);
+      }
+      for (; t < n; t += 8) {   // a value that a row does not see may be infinite: not multiplied by a zero weight
+        float w[kCombRows], keep[kCombRows][4];
+        load_rows(cs.wt[t], w);
+#pragma unroll
+        for (int r = 0; r < kCombRows; ++r)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) keep[r][i] = acc[r][i];
+        add_row(&cs.vs[t * kRowStride], w);
+#pragma unroll
+        for (int r = 0; r < kCombRows; ++r) {
+          const bool sees = t0 + t < n_tail - n_q + (row0 + r) / s.grp + 1;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[r][i] = sees ? acc[r][i] : keep[r][i];
+        }
       }
     }
     if (t0 + kTT < vis_max) {

@@ -111,6 +111,22 @@ def test_window_is_causal(caches):
     assert not torch.equal(out[:, i + 1:], out2[:, i + 1:])
 
 
+def test_window_is_causal_for_values_that_are_not_finite(caches):
+    """Keys and values after a query's own position may be anything: infinite and NaN ones leave the queries before them
+    as they are (queries 8 and 9, the last finite one and the next, share a block of 8 rows)."""
+    c = caches["llama"]
+    n_q, n_tail, i = 16, 40, 8
+    q, tk, tv, out = _check(c, 0, n_q, n_tail)
+    pos = n_tail - n_q + i
+    tk2, tv2 = tk.clone(), tv.clone()
+    tk2[:, :, pos + 1:] = float("nan")
+    tv2[:, :, pos + 1::2], tv2[:, :, pos + 2::2] = float("inf"), float("nan")
+    out2, st = gpu_window(c["cfg"], c["packed"], c["bk"], c["bv"], q, 0, tk2, tv2)
+    assert st == V.OK
+    assert torch.equal(out[:, : i + 1], out2[:, : i + 1])
+    assert not torch.isfinite(out2[:, i + 1:]).any()
+
+
 def test_window_deterministic_and_workspace_reuse(caches):
     """Two calls on one workspace (garbage-filled first: it is scratch) give identical outputs."""
     c = caches["llama"]
