@@ -1,4 +1,4 @@
-// Step 4 for a window of new tokens, bf16, more than 64 query rows per KV head: the coded part on the
+// Step 4 for a window of new tokens, bf16, more than 32 query rows per KV head: the coded part on the
 // 5th-generation tensor cores (the same mathematics, cost line, q~ fragments and partials as
 // decode_window.cu, whose first and last kernels run around this one).
 //

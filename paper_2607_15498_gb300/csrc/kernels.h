@@ -72,7 +72,7 @@ int launch_decode(const Shape& s, const varrate_packed& cache, const void* basis
 // on the cost line, then merge + causal exact tail + U_V^T per (sequence, KV head). The workspace
 // holds the q~ fragments and the per-(segment, CTA) partials, sized for kWindowMaxRows query rows.
 constexpr int kWindowMaxRows = 128;   // n_q * group
-// more than 64 rows: the coded part on tcgen05 (decode_window_tc.cu); returns -1 if the launch failed
+// more than 32 rows: the coded part on tcgen05 (decode_window_tc.cu); returns -1 if the launch failed
 int launch_window_tc(const Shape& s, const varrate_packed& c, const uint4* qf, float* part, int32_t* dev_status,
                      int layer, int ntt, int num_sms, cudaStream_t st);
 size_t decode_window_ws_bytes(const Shape& s, int num_sms);
