@@ -261,7 +261,8 @@ int64_t varrate_qpacked_cap_bytes(const varrate_config* cfg, int32_t bits);
 /* Quantize a bf16 packed cache (every stream of every (sequence, layer)) into `out` (layout above):
  * fills out->qbase from in->bucket_count and writes the codes and group parameters. out->bits is 4
  * or 8 and out->bucket_count must be in->bucket_count. A table that does not fit in->cap_elems or
- * out->qcap_bytes raises VARRATE_ERR_CORRUPT in *dev_status and leaves that (b, l) unwritten.
+ * out->qcap_bytes raises VARRATE_ERR_CORRUPT in *dev_status, leaves the codes of that (b, l) unwritten
+ * and marks it in out->qbase, so that decode reads it as empty (the exact tail alone).
  * dtype must be VARRATE_BF16 (VARRATE_ERR_UNSUPPORTED otherwise). No workspace. */
 varrate_status varrate_quantize(const varrate_config* cfg, const varrate_packed* in,
                                 varrate_qpacked* out, int32_t* dev_status, void* stream);

@@ -137,10 +137,12 @@ quantize_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restric
     }
   }
   __syncthreads();
+  // a table that does not fit the buffers (corrupt ranks upstream) is skipped, and marked so that decode skips it too
+  const bool fits = base[kMaxR + 1] <= s.cap && qb[kMaxR + 1] <= qcap;
   if (blockIdx.x == 0 && z == 0)
-    for (int r = tid; r <= kMaxR + 1; r += blockDim.x) qbase[bl * (kMaxR + 2) + r] = qb[r];
-  // a table that does not fit the buffers (corrupt ranks upstream) is skipped
-  if (base[kMaxR + 1] > s.cap || qb[kMaxR + 1] > qcap) {
+    for (int r = tid; r <= kMaxR + 1; r += blockDim.x)
+      qbase[bl * (kMaxR + 2) + r] = fits || r <= kMaxR ? qb[r] : INT64_MAX;
+  if (!fits) {
     if (tid == 0 && blockIdx.x == 0 && z == 0) raise_status(dev_status, VARRATE_ERR_CORRUPT);
     return;
   }

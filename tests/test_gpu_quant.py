@@ -319,3 +319,46 @@ def test_quantized_decode_full_size():
     blind = uniform_weight_output(dict(coef_v=deq[1], ranks=ranks), f64(bv[0]), wl.group)
     assert not decode_close(blind, want, cfg), decode_errors(blind, want)
     print(f"llama32 4-bit fused: worst relative / absolute error {decode_errors(got, want)}")
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+def test_quantized_decode_skips_a_corrupt_table(bits):
+    """Ranks out of range in a cache that held a valid encode before: its counts still look valid, but the quantized
+    cache marks the layer and decode (fused, and the general kernels past 256 tail tokens) attends to the tail alone."""
+    wl = synth.workload("llama1", n_kv_heads=2, n_ctx=1024, n_layers=2)
+    k, v, qw, bk, bv = synth.stack_inputs(wl)
+    cfg = cfg_for(wl)
+    packed = V.PackedCache.allocate(cfg, "cuda")
+    qp = V.QPackedCache.allocate(cfg, packed, bits)
+    packed.ranks.fill_(20)
+    packed.ranks[..., -wl.window:] = 128
+    ws = V.workspace(cfg, V.CALL_DECODE_Q)
+    gen = torch.Generator().manual_seed(1)
+    q = synth.stack_decode_queries(wl, 0, 1)[0]
+
+    def encode():
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        V.check(V.varrate_pack(cfg, k.cuda(), v.cuda(), bk.cuda(), bv.cuda(), packed, status), "varrate_pack")
+        packed_status = int(status.item())
+        status.zero_()
+        V.check(V.varrate_quantize(cfg, packed, qp, status), "varrate_quantize")
+        return packed_status, int(status.item())
+
+    def decode(layer, tk, tv):
+        out = torch.empty_like(q, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        V.check(V.varrate_decode_attn_q(cfg, qp, bk.cuda(), bv.cuda(), q.cuda(), layer, tk.cuda(), tv.cuda(), tk.shape[2],
+                                        out, status, ws), "varrate_decode_attn_q")
+        assert int(status.item()) == V.OK
+        return f64(out)[0]
+
+    assert encode() == (V.OK, V.OK)
+    tails = [torch.randn((2, 1, 2, n, 128), generator=gen).to(torch.bfloat16) for n in (7, 300)]
+    before = [decode(1, *t) for t in tails]
+    packed.ranks[0, 0, 100] = 3      # below r_min
+    assert encode() == (V.ERR_CORRUPT, V.ERR_CORRUPT)
+    for t, b in zip(tails, before):
+        want = O.attention(f64(q[0]), f64(t[0][0]), f64(t[1][0]))
+        got = decode(0, *t)
+        assert decode_close(got, want, cfg), decode_errors(got, want)
+        np.testing.assert_array_equal(decode(1, *t), b)
