@@ -129,7 +129,7 @@ __device__ __forceinline__ Item next_rr(const Tb& sm, Item x, int k) {
 // The same with short items apart: the last tile of a bucket with at most kShort slots. Entries of it_pref
 // then hold two prefixes, of the long items in the low 24 bits and of the short ones (at most one a
 // bucket) above them; items are numbered long ones first. A short item's place in its bucket follows
-// from the count, so it_lo stays that of the long ones.
+// from the count, so it_lo stays that of the long ones. The entries are unsigned: 128 short items make 2^31.
 constexpr int kShort = 32;
 constexpr uint32_t kLongMask = 0x00FFFFFFu;
 
@@ -147,18 +147,18 @@ __device__ __forceinline__ Item item_at_split(const Tb& sm, int k, int n_long) {
   int lo = 0, hi = kMaxR + 1;   // prefix[lo] <= kk < prefix[hi]
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if ((((uint32_t)sm.it_pref[mid] >> sh) & mask) <= kk) lo = mid; else hi = mid;
+    if (((sm.it_pref[mid] >> sh) & mask) <= kk) lo = mid; else hi = mid;
   }
   Item x;
   x.r = lo;
-  x.it = is_long ? sm.it_lo[lo] + (int)(kk - ((uint32_t)sm.it_pref[lo] & kLongMask))
+  x.it = is_long ? sm.it_lo[lo] + (int)(kk - (sm.it_pref[lo] & kLongMask))
                  : (int)((pad8(sm.cnt[lo]) - 1) / ISL);
   return x;
 }
 
 template <int STRIDE, class Tb>
 __device__ __forceinline__ Item next_rr_split(const Tb& sm, Item x, int k, int n_long) {
-  if (k < (int)((uint32_t)sm.it_pref[x.r + 1] & kLongMask)) { x.it += STRIDE; return x; }
+  if (k < (int)(sm.it_pref[x.r + 1] & kLongMask)) { x.it += STRIDE; return x; }
   return item_at_split(sm, k, n_long);
 }
 

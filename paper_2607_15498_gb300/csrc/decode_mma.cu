@@ -216,23 +216,23 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
         long long i0 = 0, i1 = 0;
         if (r >= s.r_min && r <= s.r_max) bucket_range(sm, r, lo, hi, i0, i1);
         sm.it_lo[r] = (int)i0;
-        sm.it_pref[r + 1] = (int)split_count(i0, i1, sm.cnt[r]);   // counts first, prefixed below
+        sm.it_pref[r + 1] = split_count(i0, i1, sm.cnt[r]);   // counts first, prefixed below
       }
       __syncthreads();
       if (warp == 0) {   // inclusive scan of it_pref[1 .. 129], 5 entries per lane
         __syncwarp();
         constexpr int kPer = (kMaxR + 1 + 31) / 32;
-        int v[kPer], acc = 0;
+        uint32_t v[kPer], acc = 0;
 #pragma unroll
         for (int e = 0; e < kPer; ++e) {
           const int r = lane * kPer + e;
-          acc += r <= kMaxR ? sm.it_pref[r + 1] : 0;
+          acc += r <= kMaxR ? sm.it_pref[r + 1] : 0u;
           v[e] = acc;
         }
-        int excl = acc;
+        uint32_t excl = acc;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, excl, o);
+          const uint32_t y = __shfl_up_sync(0xffffffffu, excl, o);
           if (lane >= o) excl += y;
         }
         excl -= acc;
@@ -256,8 +256,8 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ coef, const int32_t* __restr
       for (int t = 0; t < kHeadDim / 16; ++t) oacc[t][0] = oacc[t][1] = oacc[t][2] = oacc[t][3] = 0.f;
 
       // long items first, then the short ones: every warp takes both in turn
-      const int n_long = dead ? 0 : (int)((uint32_t)sm.it_pref[kMaxR + 1] & kLongMask);
-      const int total = dead ? 0 : n_long + (int)((uint32_t)sm.it_pref[kMaxR + 1] >> 24);
+      const int n_long = dead ? 0 : (int)(sm.it_pref[kMaxR + 1] & kLongMask);
+      const int total = dead ? 0 : n_long + (int)(sm.it_pref[kMaxR + 1] >> 24);
       Prod pr;
       pr.k = warp; pr.phase = 0; pr.jc = 0;
       if (pr.k < total) pr.item = item_at_split(sm, pr.k, n_long);

@@ -27,7 +27,7 @@ struct SegSmem {
   long long base[kMaxR + 2];
   int cnt[kMaxR + 1];
   int it_lo[kMaxR + 1];     // first item of bucket r inside this CTA's cost range
-  int it_pref[kMaxR + 2];   // exclusive prefix of the per-bucket item counts
+  uint32_t it_pref[kMaxR + 2];   // exclusive prefix of the per-bucket item counts (split_count)
 };
 static_assert(offsetof(SegSmem, qfrag) % 16 == 0, "qfrag is read with 16-byte loads");
 

@@ -98,3 +98,41 @@ def test_decode_quantized_wide_ranks(kind, n, bits, grp, n_tail):
                          *((f64(tk[0]), f64(tv[0])) if n_tail else ()))
     got = f64(out)[0]
     assert decode_close(got, want, cfg), decode_errors(got, want)
+
+
+@pytest.mark.parametrize("bits", [0, 4, 8])
+def test_decode_every_rank_a_short_tile(bits):
+    """Every rank from 1 to 128 holds 8 tokens, and there are more (sequence, head) pairs than thread blocks, so that
+    one block takes all 128 short tiles of a pair: the largest count that the item table holds."""
+    wl = synth.workload("llama1", n_ctx=1024, n_kv_heads=8, group=2, batch=32, window=3, budget_frac=1.0, r_min=1)
+    cfg = cfg_for(wl)
+    ranks = 1 + np.random.default_rng(0).permutation(1024) % 128
+    gen = torch.Generator().manual_seed(0)
+    k, v = (torch.randn((32, 1, 8, 1024, 128), generator=gen).to(torch.bfloat16) for _ in range(2))
+    u = torch.linalg.qr(torch.randn((2, 1, 8, 128, 128), generator=gen))[0].to(torch.bfloat16).contiguous()
+    packed, st = gpu_pack(cfg, np.tile(ranks, (32, 1, 1)), k, v, u[0], u[1])
+    assert st == V.OK
+    q = torch.randn((32, 16, 128), generator=gen).to(torch.bfloat16)
+    if bits:
+        count, base, pos, _ = O.pack_tables(ranks, 1, 128)
+        qp = V.QPackedCache.allocate(cfg, packed, bits)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        V.check(V.varrate_quantize(cfg, packed, qp, status), "varrate_quantize")
+        dev = torch.empty_like(q, device="cuda")
+        V.check(V.varrate_decode_attn_q(cfg, qp, u[0].cuda(), u[1].cuda(), q.cuda(), 0, None, None, 0, dev, status,
+                                        V.workspace(cfg, V.CALL_DECODE_Q)), "varrate_decode_attn_q")
+        assert int(status.item()) == V.OK
+        out = f64(dev)
+    else:
+        out, st = gpu_decode(cfg, packed, u[0], u[1], q, 0)
+        assert st == V.OK
+    for b in (0, 13, 31):
+        if bits:
+            ck, cv = (np.stack([O.quantize_coefficients(unpack(packed, b, 0, g, kv, ranks, count, base, pos).astype(np.float32),
+                                                        ranks, count, pos, bits)[3] for g in range(8)]).astype(np.float64)
+                      for kv in range(2))
+        else:
+            ck, cv = (np.stack([O.truncate(O.project(f64(x[b, 0, g]), f64(w[0, g])), ranks) for g in range(8)])
+                      for x, w in ((k, u[0]), (v, u[1])))
+        want = O.decode_coef(f64(q[b]), ck, cv, ranks, f64(u[0][0]), f64(u[1][0]))
+        assert decode_close(out[b], want, cfg), (b, decode_errors(out[b], want))
