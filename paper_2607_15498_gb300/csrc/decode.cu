@@ -281,10 +281,11 @@ decode_split_kernel(Src src, const int32_t* __restrict__ bucket_count, const flo
         mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 1));
         mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 2));
         const float nm = fmaxf(M[h], mloc);
-        const float corr = exp2f(M[h] - nm);
+        const float ref = nm == -INFINITY ? 0.f : nm;     // every score so far is -inf: weights 0, not NaN
+        const float corr = exp2f(M[h] - ref);
         float sum = 0.f;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) { sc[h][i] = exp2f(sc[h][i] - nm); sum += sc[h][i]; }
+        for (int i = 0; i < 8; ++i) { sc[h][i] = exp2f(sc[h][i] - ref); sum += sc[h][i]; }
         Ls[h] = Ls[h] * corr + sum;
         M[h] = nm;
 #pragma unroll

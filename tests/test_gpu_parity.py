@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_helpers import (O, V, cfg_for, coef_tol, decode_close, decode_errors, f64, gpu_allocate,
+from gpu_helpers import (O, V, cfg_for, coef_index, coef_tol, decode_close, decode_errors, f64, gpu_allocate,
                          gpu_decode, gpu_encode, gpu_pack, oracle_layer, salience_close, synth,
                          unpack)
 
@@ -326,6 +326,36 @@ def test_empty_coded_set_decodes_exactly():
     q = synth.stack_decode_queries(wl, 0, 1)[0]
     out, _ = gpu_decode(cfg, r["packed"], bk, bv, q, 0)
     assert np.abs(out[0] - O.attention(f64(q[0]), f64(k[0, 0]), f64(v[0, 0]))).max() <= 1e-5
+
+
+@pytest.mark.parametrize("dtype, n_tail", [("f32", 0), ("bf16", 300)])
+def test_general_decode_of_items_with_no_finite_score(dtype, n_tail):
+    """Runs of 32 tokens (items of the general kernels) whose scores are all -inf have weight 0, also where a warp or
+    its block goes on to other items (20 sequences of 8 heads leave few splits)."""
+    n, G = 700, 8
+    wl = synth.workload("llama1", n_ctx=n, n_kv_heads=G, group=1, batch=20, window=3, budget_frac=1.0, r_min=16, dtype=dtype)
+    cfg = cfg_for(wl)
+    ranks = np.full(n, 16)
+    k, v, _, bk, bv = synth.stack_inputs(wl)
+    packed, st = gpu_pack(cfg, np.tile(ranks, (20, 1, 1)), k, v, bk, bv)
+    assert st == V.OK
+    q = synth.stack_decode_queries(wl, 0, 1)[0]
+    out = (np.arange(n) // 32) % 3 == 0
+    at = torch.as_tensor(coef_index(0, 16, 704, np.arange(n)[out], 0)).cuda()
+    sign = np.sign([[f64(bk[0, g, 0]) @ f64(q[b, g]) for g in range(G)] for b in range(20)])   # of q~[0]
+    for b in range(20):
+        for g in range(G):
+            packed.coef[b, 0, g, 0, at] = -sign[b, g] * float("inf")
+    gen = torch.Generator().manual_seed(n_tail)
+    tk, tv = (torch.randn((20, G, n_tail, 128), generator=gen).to(synth.torch_dtype(wl)) for _ in range(2))
+    got, st = gpu_decode(cfg, packed, bk, bv, q, 0, *((tk, tv) if n_tail else ()))
+    assert st == V.OK and np.isfinite(got).all()
+    for b in (0, 7, 19):
+        ck, cv = (np.stack([O.truncate(O.project(f64(x[b, 0, g]), f64(u[0, g])), ranks) for g in range(G)])
+                  for x, u in ((k, bk), (v, bv)))
+        want = O.decode_coef(f64(q[b]), ck[:, ~out], cv[:, ~out], ranks[~out], f64(bk[0]), f64(bv[0]),
+                             *((f64(tk[b]), f64(tv[b])) if n_tail else ()))
+        assert decode_close(got[b], want, cfg), decode_errors(got[b], want)
 
 
 # ------------------------------------------------------------------- encode end to end
