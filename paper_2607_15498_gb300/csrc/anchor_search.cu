@@ -32,6 +32,8 @@
 #include <cudaTypedefs.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -296,14 +298,17 @@ size_t search_smem_bytes() { return 1024 + (size_t)AS_ST * AS_SBYTES + sizeof(As
 // fp32 (bf16 values are exact in fp32), divided by their count (IEEE division; by a power of two the
 // product with its exact reciprocal is the same number), subtracted from z_t and rounded to bf16.
 // The list of a token: rows[s] = anchor, or n_a (a row of zeros) for a skipped entry; returns the number of valid
-// entries, 0 when there is none or an entry is out of [-1, n_a). C > 0: lists of C entries, else of c <= 8.
-template <int C>
-__device__ __forceinline__ int load_list(const int32_t* __restrict__ p, int c, int n_a, uint32_t (&rows)[C ? C : AS_LIST]) {
-  constexpr int K = C ? C : AS_LIST;
+// entries, 0 when there is none or an entry is out of [-1, n_a). K entries are formed, of which c are in the list
+// (K = c = 2 or 4: one load, aligned to the list).
+template <int K>
+__device__ __forceinline__ int load_list(const int32_t* __restrict__ p, int c, int n_a, uint32_t (&rows)[K]) {
   int x[K];
-  if constexpr (C == 4) {   // 16-byte aligned
+  if constexpr (K == 4) {
     const int4 q = __ldg(reinterpret_cast<const int4*>(p));
     x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+  } else if constexpr (K == 2) {
+    const int2 q = __ldg(reinterpret_cast<const int2*>(p));
+    x[0] = q.x; x[1] = q.y;
   } else {
 #pragma unroll
     for (int s = 0; s < K; ++s) x[s] = s < c ? __ldg(p + s) : -1;
@@ -351,8 +356,10 @@ __device__ __forceinline__ uint4 residual8(uint4 z, float (&acc)[8], int m) {
 // (plus a zero row for skipped entries) and streams its share of the tokens past them, 16 bytes a thread.
 // Read straight from L2 the c listed anchors of every token are c times the bytes of K and V themselves;
 // from shared memory K and V are read once and the residuals written once. Bound by shared-memory reads (rows
-// of 64 bytes: two of them share a wavefront when their parities differ) and instructions. 2 layers x 8
-// heads x 32768 tokens, 4 of 2048 anchors each (538 MB): a warp per token reading L2 248 us, this 141 us.
+// of 64 bytes: two of them share a wavefront when their parities differ) and instructions: the length of the lists
+// C is a constant (any length in one form, eight entries tested each, took 72 to 102 us at lengths 1 to 8 where this
+// takes 56 to 86). 2 layers x 8 heads x 32768 tokens, 4 of 2048 anchors each (538 MB): a warp per token
+// reading L2 248 us, this 117 us.
 // grid (column blocks x splits x 2 G, B L).
 constexpr int RS_THREADS = 1024;
 constexpr int RS_TOK = 2;                    // tokens per thread whose loads are in flight together
@@ -362,7 +369,7 @@ template <int CW, int C>
 __global__ void __launch_bounds__(RS_THREADS, 1)
 anchor_residual_slab_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                             const int32_t* __restrict__ idx, __nv_bfloat16* __restrict__ e,
-                            int32_t* __restrict__ dev_status, int G, int64_t N, int stride, int c, int n_a,
+                            int32_t* __restrict__ dev_status, int G, int64_t N, int stride, int n_a,
                             int splits, int64_t share) {
   constexpr int TPT = CW / 8, TOKS = RS_THREADS / TPT, NCB = kHeadDim / CW;   // threads a token, tokens a step
   extern __shared__ uint4 slab[];            // [n_a + 1][TPT]
@@ -376,18 +383,17 @@ anchor_residual_slab_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bflo
     slab[i] = __ldg(reinterpret_cast<const uint4*>(base + (int64_t)(i / TPT) * stride * kHeadDim) + part);
   if (tid < TPT) slab[n_a * TPT + tid] = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  constexpr int K = C ? C : AS_LIST;
   const int64_t t_end = min(N, (split + 1) * share);
   for (int64_t t0 = split * share + tid / TPT; t0 < t_end; t0 += TOKS * RS_TOK) {
     uint4 z[RS_TOK];
-    uint32_t rows[RS_TOK][K];
+    uint32_t rows[RS_TOK][C];
     int m[RS_TOK];
 #pragma unroll
     for (int u = 0; u < RS_TOK; ++u) {
       const int64_t t = t0 + u * TOKS;
       if (t < t_end) {
         z[u] = __ldcs(reinterpret_cast<const uint4*>(base + t * kHeadDim) + part);
-        m[u] = load_list<C>(idx + (bl * N + t) * c, c, n_a, rows[u]);
+        m[u] = load_list<C>(idx + (bl * N + t) * C, C, n_a, rows[u]);
       }
     }
 #pragma unroll
@@ -400,17 +406,18 @@ anchor_residual_slab_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bflo
       }
       float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int s = 0; s < K; ++s)
-        if (C || s < c) add8(acc, slab[rows[u][s] * TPT + part]);
+      for (int s = 0; s < C; ++s) add8(acc, slab[rows[u][s] * TPT + part]);
       __stcs(reinterpret_cast<uint4*>(e + ((bl * N + t) * 2 * G + kvg) * kHeadDim + cb * CW) + part,
              residual8(z[u], acc, m[u]));
     }
   }
 }
 
-// Direct form, for more anchors than 16 columns of which fit in shared memory: a warp per token, half a warp
-// per head row (16 bytes a lane), the listed anchors read from L2. grid (ceil(N / 8), B L), 256 threads.
-__global__ void __launch_bounds__(256)
+// Direct form, for more anchors or fewer tokens than the slab form is for: a warp per token, half a warp per head row
+// (16 bytes a lane), the listed anchors read from L2, all of a row's in flight together. Bound by that latency: at 64
+// registers four CTAs share an SM; at 78 (three) 8 heads x 32768 tokens, lists of 7 at stride 5, took 127 us, now 93 (134
+// with a whole warp per head row, 8 bytes a lane). grid (ceil(N / 8), B L), 256 threads.
+__global__ void __launch_bounds__(256, 4)
 anchor_residual_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                        const int32_t* __restrict__ idx, __nv_bfloat16* __restrict__ e,
                        int32_t* __restrict__ dev_status, int G, int64_t N, int stride, int c, int n_a) {
@@ -419,7 +426,7 @@ anchor_residual_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16*
   const int64_t t = (int64_t)blockIdx.x * 8 + warp;
   if (t >= N) return;
   uint32_t rows[AS_LIST];
-  const int m = load_list<0>(idx + (bl * N + t) * c, c, n_a, rows);
+  const int m = load_list<AS_LIST>(idx + (bl * N + t) * c, c, n_a, rows);
   if (m == 0) {                                      // warp-uniform: every lane read the same list
     if (lane == 0) raise_status(dev_status, VARRATE_ERR_CORRUPT);
     return;
@@ -466,12 +473,12 @@ bool anchor_residual_supported(const Shape& s, int stride, int c) {
 
 namespace {
 
-template <int CW>
-int launch_residual_slab(const Shape& s, const void* k, const void* v, int stride, int c, const int32_t* idx,
+template <int CW, int C>
+int launch_residual_slab(const Shape& s, const void* k, const void* v, int stride, const int32_t* idx,
                          void* e_out, int32_t* dev_status, int num_sms, cudaStream_t st) {
   const int n_a = anchor_count(s.N, stride);
   const size_t smem = (size_t)(n_a + 1) * CW * 2;
-  auto kernel = c == 4 ? anchor_residual_slab_kernel<CW, 4> : anchor_residual_slab_kernel<CW, 0>;
+  auto kernel = anchor_residual_slab_kernel<CW, C>;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM) != cudaSuccess) return -1;
   // splits of the tokens that make waves x (steps of a CTA + its slab, read at about twice a step's rate) least
   constexpr int64_t kStep = RS_THREADS / (CW / 8) * RS_TOK;
@@ -487,8 +494,8 @@ int launch_residual_slab(const Shape& s, const void* k, const void* v, int strid
   n = (s.N + share - 1) / share;
   const dim3 grid((unsigned)(kHeadDim / CW * n * 2 * s.G), (unsigned)((size_t)s.B * s.L));
   kernel<<<grid, RS_THREADS, smem, st>>>(
-      (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, (__nv_bfloat16*)e_out, dev_status, s.G, s.N, stride, c,
-      n_a, (int)n, share);
+      (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, (__nv_bfloat16*)e_out, dev_status, s.G, s.N, stride, n_a,
+      (int)n, share);
   return 1;
 }
 
@@ -496,12 +503,30 @@ int launch_residual_slab(const Shape& s, const void* k, const void* v, int strid
 
 int launch_anchor_residual(const Shape& s, const void* k, const void* v, int stride, int c,
                            const int32_t* idx, void* e_out, int32_t* dev_status, int num_sms, cudaStream_t st) {
-  // the widest column block of all anchors (and the zero row) that fits in shared memory
+  // Slabs where 32 columns of all anchors (and the zero row) fit and there are some 24 thousand rows of K to stream
+  // past them; at 32 columns, lists of 8 read too many rows of shared memory. Slab / direct in us, 8 heads: 32768
+  // tokens, stride 64 (128 columns) lists of 1 52 / 75, 4 55 / 79, 8 64 / 83; stride 16 (32 columns) 1 56 / 76, 3 64 / 89,
+  // 4 62 / 81, 7 86 / 89, 8 95 / 83; 2000 tokens 4 12.7 / 10.0, 4000 tokens 12.4 / 14.7. With 16 columns (stride 5 to 8)
+  // slabs took 79 to 170 us where direct takes 76 to 94.
   const size_t rows = (size_t)anchor_count(s.N, stride) + 1;
-  if (rows * 128 * 2 <= RS_SMEM) return launch_residual_slab<128>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
-  if (rows * 64 * 2 <= RS_SMEM) return launch_residual_slab<64>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
-  if (rows * 32 * 2 <= RS_SMEM) return launch_residual_slab<32>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
-  if (rows * 16 * 2 <= RS_SMEM) return launch_residual_slab<16>(s, k, v, stride, c, idx, e_out, dev_status, num_sms, st);
+  const int cw = rows * 256 <= RS_SMEM ? 128 : rows * 128 <= RS_SMEM ? 64 : rows * 64 <= RS_SMEM ? 32 : 0;
+  if (cw && !(cw == 32 && c == AS_LIST) && (int64_t)s.B * s.L * s.G * s.N >= 24576) {
+    auto launch = [&](auto C) {
+      return cw == 128 ? launch_residual_slab<128, C()>(s, k, v, stride, idx, e_out, dev_status, num_sms, st)
+             : cw == 64 ? launch_residual_slab<64, C()>(s, k, v, stride, idx, e_out, dev_status, num_sms, st)
+                        : launch_residual_slab<32, C()>(s, k, v, stride, idx, e_out, dev_status, num_sms, st);
+    };
+    switch (c) {
+      case 1: return launch(std::integral_constant<int, 1>());
+      case 2: return launch(std::integral_constant<int, 2>());
+      case 3: return launch(std::integral_constant<int, 3>());
+      case 4: return launch(std::integral_constant<int, 4>());
+      case 5: return launch(std::integral_constant<int, 5>());
+      case 6: return launch(std::integral_constant<int, 6>());
+      case 7: return launch(std::integral_constant<int, 7>());
+      default: return launch(std::integral_constant<int, 8>());
+    }
+  }
   anchor_residual_kernel<<<dim3((unsigned)((s.N + 7) / 8), (unsigned)((size_t)s.B * s.L)), 256, 0, st>>>(
       (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, idx, (__nv_bfloat16*)e_out, dev_status, s.G, s.N,
       stride, c, anchor_count(s.N, stride));

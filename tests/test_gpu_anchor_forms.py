@@ -62,6 +62,20 @@ def test_search_pair_edges(n, stride, c, tied):
 @pytest.mark.parametrize("c", [1, 3, 4, 8])
 @pytest.mark.parametrize("n, stride", [(700, 3), (830, 1), (831, 1), (1663, 1), (3327, 1), (6655, 1), (6656, 1)])
 def test_residual_forms(n, stride, c):
+    _check_residual(n, stride, c, [])
+
+
+# 831 and 832 anchors: 128 and 64 columns; 1663 and 1664: 64 and 32; 3327 and 3328: 32 columns and the direct form. With
+# 12287 tokens of two heads the slabs are not worth their set-up, with 12288 they are.
+@pytest.mark.parametrize("c", range(1, 9))
+@pytest.mark.parametrize("n, stride", [(12465, 15), (12466, 15), (13304, 8), (13305, 8), (13308, 4), (13309, 4),
+                                       (12287, 16), (12288, 16)])
+def test_residual_slab_forms(n, stride, c):
+    _check_residual(n, stride, c, [0, 5000, n - 1])
+
+
+def _check_residual(n, stride, c, bad):
+    """`bad`: tokens whose lists are out of range (every other one by its last entry, the rest empty)."""
     k, v = _kv(n, 2, n + c)
     n_a = -(-n // stride)
     gen = torch.Generator().manual_seed(c)
@@ -69,17 +83,22 @@ def test_residual_forms(n, stride, c):
     if c > 1:
         idx[torch.rand(idx.shape, generator=gen) < 0.15] = -1
         idx[..., 0] = torch.where((idx >= 0).any(-1), idx[..., 0], n_a - 1)
+    for i, t in enumerate(bad):
+        idx[0, 0, t, -1 if i % 2 == 0 else slice(None)] = n_a if i % 2 == 0 else -1
     cfg = V.make_config(1, 2, 4, n, window=8, dtype=V.BF16)
     e = torch.full((1, 1, n, 512), float("nan"), dtype=torch.bfloat16, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     V.check(V.varrate_anchor_residual(cfg, k.cuda(), v.cuda(), stride, c, idx.cuda(), e, status),
             "varrate_anchor_residual")
     torch.cuda.synchronize()
-    assert int(status.item()) == V.OK
+    assert int(status.item()) == (V.ERR_CORRUPT if bad else V.OK)
+    good = torch.ones(n, dtype=torch.bool)
+    good[bad] = False
+    assert torch.isnan(e[0, 0].cpu()[~good]).all()
     z = _joint(k, v)[0].float()
-    a, li = z[::stride], idx[0, 0].long()
+    a, li = z[::stride], idx[0, 0].long().where(good[:, None], 0)
     acc = torch.zeros_like(z)
     for s in range(c):
         acc += torch.where(li[:, s:s + 1] >= 0, a[li[:, s].clamp(min=0)], 0.0)
     want = (z - acc / (li >= 0).sum(-1, keepdim=True).float()).to(torch.bfloat16)
-    np.testing.assert_array_equal(e[0, 0].cpu().view(torch.int16).numpy(), want.view(torch.int16).numpy())
+    np.testing.assert_array_equal(e[0, 0].cpu()[good].view(torch.int16).numpy(), want[good].view(torch.int16).numpy())
