@@ -31,8 +31,8 @@ static_assert(kWarps > kCand, "a warp adds the warps' sums of one level");
 constexpr int kMaxCluster = 8;         // portable cluster size
 constexpr int64_t kMaxCached = 49152;  // normalised saliences kept in shared memory (192 KB)
 
-__device__ __forceinline__ float shat_of(float s, float mn, float den, bool flat) {
-  const float v = flat ? 1.0f : __fdiv_rn(__fsub_rn(s, mn), den);
+__device__ __forceinline__ float shat_of(float s, float mn, float den) {
+  const float v = __fdiv_rn(__fsub_rn(s, mn), den);
   return v == v ? v : 0.f;   // NaN salience: rank r_min, as x = r_min gives
 }
 
@@ -104,6 +104,8 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
     if (rank == 0 && tid == 0) raise_status(dev_status, VARRATE_FLOOR_BINDS);
   } else if (s.Bc >= (int64_t)s.r_max * n) {
     mode_fixed = s.r_max;
+  } else if (sl == nullptr || s.mode == VARRATE_UNIFORM) {
+    mode_fixed = (int)(s.Bc / n);   // all s_hat are 1: the largest lambda that fits gives every token floor(B_c / n)
   }
   if (mode_fixed >= 0) {   // uniform over the cluster: no barrier is skipped by part of it
     for (int64_t i = tid; i < cnt; i += kThreads) rk[t0 + i] = (uint8_t)mode_fixed;
@@ -114,21 +116,18 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
   cluster.barrier_arrive();   // this CTA runs: the others may write its shared memory once they have waited
   // min / max over the coded set (exact in any order), and the sum, which only places the first levels
   float mn = INFINITY, mx = -INFINITY, sum = 0.f;
-  const bool uniform = (s.mode == VARRATE_UNIFORM) || sl == nullptr;
-  if (!uniform) {
-    for (int64_t i = tid; i < cnt; i += kThreads) {
-      const float v = sl[t0 + i];
-      if (i < cached) sh_cache[i] = v;
-      mn = fminf(mn, v);
-      mx = fmaxf(mx, v);
-      sum += v;
-    }
-    warp_stats(mn, mx, sum);
-    if (lane == 0) { sm.fred[0][warp] = mn; sm.fred[1][warp] = mx; sm.fred[2][warp] = sum; }
+  for (int64_t i = tid; i < cnt; i += kThreads) {
+    const float v = sl[t0 + i];
+    if (i < cached) sh_cache[i] = v;
+    mn = fminf(mn, v);
+    mx = fmaxf(mx, v);
+    sum += v;
   }
+  warp_stats(mn, mx, sum);
+  if (lane == 0) { sm.fred[0][warp] = mn; sm.fred[1][warp] = mx; sm.fred[2][warp] = sum; }
   __syncthreads();
   cluster.barrier_wait();     // every CTA of the cluster has started
-  if (!uniform && warp == 0) {
+  if (warp == 0) {
     mn = lane < kWarps ? sm.fred[0][lane] : INFINITY;
     mx = lane < kWarps ? sm.fred[1][lane] : -INFINITY;
     sum = lane < kWarps ? sm.fred[2][lane] : 0.f;
@@ -141,21 +140,24 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
     }
   }
   cluster.sync();
-  if (!uniform) {
-    mn = INFINITY; mx = -INFINITY; sum = 0.f;
-    for (int c = 0; c < C; ++c) {
-      mn = fminf(mn, sm.mm[c][0]);
-      mx = fmaxf(mx, sm.mm[c][1]);
-      sum += sm.mm[c][2];
-    }
+  mn = INFINITY; mx = -INFINITY; sum = 0.f;
+  for (int c = 0; c < C; ++c) {
+    mn = fminf(mn, sm.mm[c][0]);
+    mx = fmaxf(mx, sm.mm[c][1]);
+    sum += sm.mm[c][2];
   }
-  const bool flat = uniform || !(mx > mn);
-  const float den = flat ? 1.0f : __fsub_rn(mx, mn);
+  if (!(mx > mn)) {   // a constant salience is the uniform case (the same for the whole cluster)
+    const int r = (int)(s.Bc / n);
+    for (int64_t i = tid; i < cnt; i += kThreads) rk[t0 + i] = (uint8_t)r;
+    if (rank == 0 && tid == 0 && realized) realized[bl] = (int64_t)r * n;
+    return;
+  }
+  const float den = __fsub_rn(mx, mn);
   // a thread normalises, and reads in every pass, the entries it loaded itself
   for (int64_t i = tid; i < min(cnt, cached); i += kThreads)   // entries past n_cached: normalised when read
-    sh_cache[i] = shat_of(uniform ? 0.f : sh_cache[i], mn, den, flat);
+    sh_cache[i] = shat_of(sh_cache[i], mn, den);
   const int n_cached = (int)min(cnt, cached);
-  auto shat_far = [&](int64_t i) { return shat_of(uniform ? 0.f : sl[t0 + i], mn, den, flat); };
+  auto shat_far = [&](int64_t i) { return shat_of(sl[t0 + i], mn, den); };
   const float fmin_r = (float)s.r_min, fmax_r = (float)s.r_max;
   const bool wide = share >= (int64_t(1) << 24);   // a warp's sum may pass 32 bits
 
@@ -163,11 +165,11 @@ allocate_kernel(const float* __restrict__ sal, uint8_t* __restrict__ ranks,
   // pattern after the largest finite value stand in at the start. Any levels that bracket it closer give
   // the same answer. The first pass spreads them around the level that would spend the budget if no
   // rank met r_max; then the totals at both ends interpolate a guess (the total is close to linear in
-  // a narrow bracket), and every other pass cuts the bracket evenly, to a sixteenth, which bounds the
+  // a narrow bracket), and every third pass cuts the bracket evenly, to a sixteenth, which bounds the
   // number of passes whatever the salience looks like.
   uint32_t lo = 0, hi = 0x7F800000u;
   long long tot_lo = (long long)s.r_min * n, tot_hi = (long long)s.r_max * n;
-  const float mean = flat ? 1.f : (sum / (float)n - mn) / den;
+  const float mean = (sum / (float)n - mn) / den;
   const float first = ((float)((double)s.Bc / (double)n) - fmin_r + 0.5f) / mean;
   for (int pass = 0; hi - lo > 1; ++pass) {
     const uint32_t span = hi - lo, step = (span + kCand) / (kCand + 1);

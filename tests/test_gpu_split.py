@@ -32,6 +32,18 @@ def test_allocation_split_edges(n_coded, pairs):
     _check(np.exp(1.2 * rng.standard_normal((pairs, n_coded))), wl)
 
 
+@pytest.mark.parametrize("n_coded, pairs", [(1, 1), (700, 2), (2049, 1), (9000, 3), (3000, 160)])
+@pytest.mark.parametrize("budget", [0.2, 0.31, 0.74])
+def test_allocation_of_a_constant_salience(n_coded, pairs, budget):
+    """Constant and absent (uniform mode) salience: no search, on one block and on clusters."""
+    wl = synth.workload("llama1", n_ctx=n_coded + 5, window=5, n_layers=pairs, budget_frac=budget)
+    for sal in (np.full((pairs, n_coded), 0.25), np.full((pairs, n_coded), np.nan)):
+        got = _check(np.where(np.isnan(sal), 1.0, sal), wl)
+        ranks, _, _ = gpu_allocate(cfg_for(wl), sal)
+        np.testing.assert_array_equal(ranks, got)
+    _check(np.random.default_rng(1).random((pairs, n_coded)), wl, mode=O.UNIFORM)
+
+
 def test_allocation_more_tokens_than_shared_memory_holds():
     # 8 CTAs of 52501 tokens, of which 49152 are held normalised; one pair alone on a CTA as well
     wl = synth.workload("llama1", n_ctx=420_008, window=8, budget_frac=0.2)
