@@ -242,49 +242,18 @@ salience_accum_tc_kernel(const __grid_constant__ CUtensorMap tk, const __nv_bflo
       }
       *reinterpret_cast<uint4*>(qb + sw128_offset(row, cidx, npad)) = v;
     }
-    if (n_chunks <= 8) {   // few partials: a thread per row
-      for (int row = tid; row < npad; row += P2_EPI * 32) {
-        float2 x[8];
-        float mx = -INFINITY, l = 0.f;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          x[c] = make_float2(-INFINITY, 0.f);
-          if (row < M && c < n_chunks) x[c] = stats[((bl * s.G + g) * M + row) * n_chunks + c];
-          mx = fmaxf(mx, x[c].x);
-        }
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (x[c].x != -INFINITY) l += x[c].y * exp2f(x[c].x - mx);
-        sm.nlse[row] = row < M ? -(mx + log2f(l)) : -INFINITY;
-      }
-    } else
-    // a warp per row, its lanes over the chunks' partials, the loads of eight rows in flight together
-    for (int r0 = warp; r0 < npad; r0 += 8 * P2_EPI) {
-      float2 x[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int row = r0 + u * P2_EPI;
-        x[u] = make_float2(-INFINITY, 0.f);
-        if (row < M && lane < n_chunks) x[u] = stats[((bl * s.G + g) * M + row) * n_chunks + lane];
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int row = r0 + u * P2_EPI;
-        if (row >= npad) break;                            // warp-uniform
+    for (int row = tid; row < npad; row += P2_EPI * 32) {
+      float val = -INFINITY;
+      if (row < M) {
         const float2* st = stats + ((bl * s.G + g) * M + row) * n_chunks;
-        float mx = x[u].x;
-        if (row < M)
-          for (int c = lane + 32; c < n_chunks; c += 32) mx = fmaxf(mx, st[c].x);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float l = x[u].x != -INFINITY ? x[u].y * exp2f(x[u].x - mx) : 0.f;
-        if (row < M)
-          for (int c = lane + 32; c < n_chunks; c += 32)
-            if (st[c].x != -INFINITY) l += st[c].y * exp2f(st[c].x - mx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-        if (lane == 0) sm.nlse[row] = row < M ? -(mx + log2f(l)) : -INFINITY;
+        float mx = -INFINITY;
+        for (int c = 0; c < n_chunks; ++c) mx = fmaxf(mx, st[c].x);
+        float l = 0.f;
+        for (int c = 0; c < n_chunks; ++c)
+          if (st[c].x != -INFINITY) l += st[c].y * exp2f(st[c].x - mx);
+        val = -(mx + log2f(l));
       }
+      sm.nlse[row] = val;
     }
   }
   if (warp == P2_EPI + 1 && lane == 0) {
@@ -401,7 +370,10 @@ bool salience_tc_supported(const Shape& s) {
 }
 
 // Chunks (CTAs) per unit of work that make waves x (tiles of a CTA + its set-up, counted in tiles) least: with
-// few units one wave of equal CTAs, with many units no more CTAs than their set-up is worth.
+// few units one wave of equal CTAs, with many units no more CTAs than their set-up is worth. A set-up counts as 5
+// tiles of 256 tokens in pass 1 (160 units of 8192 tokens in 1, 2, 3, 4, 6 CTAs each: 195, 186, 185, 190, 201 us for the
+// whole call; 256 of 32768 in 1, 2, 4: 743, 747, 740) and 12 tiles of 128 in pass 2 (160 of 8192 in 1, 2, 3, 4: 191, 181,
+// 182, 187; 256 of 8192 217, 231, 241, 248; 160 of 32768 585, 523, 505, 499; 320 of 32768 965, 909, 902, 901).
 static int best_split(int64_t units, int64_t tiles, double setup, int num_sms) {
   int best_n = 1;
   double best = 1e300;
@@ -418,13 +390,12 @@ SalPlan salience_tc_plan(const Shape& s, int num_sms) {
   p.n_rb = (s.grp * s.w + 127) / 128;
   const int64_t pairs = (int64_t)s.B * s.L * s.G;
   const int64_t tiles = (s.N + P1_TN - 1) / P1_TN;
-  const int n = best_split(pairs * p.n_rb, tiles, 3.0, num_sms);
+  const int n = best_split(pairs * p.n_rb, tiles, 5.0, num_sms);
   p.chunk = (tiles + n - 1) / n * P1_TN;
   p.n_chunks = (int)((s.N + p.chunk - 1) / p.chunk);
   const int64_t tiles2 = s.n_coded > 0 ? (s.n_coded + P2_TM - 1) / P2_TM : 1;
-  // pass 2 pays more per CTA (the lse of every window row): with a wave of units or more it keeps to two
-  // CTAs each (256 units of 32k tokens: 361 us with 2, 395 us with 4; pass 1 366 us with 2, 353 us with 4)
-  const int n2 = pairs >= 2 * num_sms ? 1 : pairs >= num_sms ? 2 : best_split(pairs, tiles2, 12.0, num_sms);
+  // pass 2 pays more per CTA: the window rows and the lse of each
+  const int n2 = best_split(pairs, tiles2, 12.0, num_sms);
   p.chunk2 = (tiles2 + n2 - 1) / n2 * P2_TM;
   p.n_chunks2 = (int)((s.n_coded + p.chunk2 - 1) / p.chunk2);
   return p;
