@@ -46,24 +46,6 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
                      __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
 }
 
-// Eight consecutive elements starting at a 16-byte (bf16) / 32-byte (fp32) aligned address,
-// streamed (read once: evict-first in L2, no L1 allocation).
-__device__ __forceinline__ void load8_stream(const __nv_bfloat16* p, float (&f)[8]) {
-  uint4 u = __ldcs(reinterpret_cast<const uint4*>(p));
-  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = __uint_as_float(w[i] << 16);
-    f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
-  }
-}
-__device__ __forceinline__ void load8_stream(const float* p, float (&f)[8]) {
-  float4 a = __ldcs(reinterpret_cast<const float4*>(p));
-  float4 b = __ldcs(reinterpret_cast<const float4*>(p) + 1);
-  f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
-  f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
-}
-
 __device__ __forceinline__ int64_t pad8(int64_t n) { return (n + 7) & ~int64_t(7); }
 
 // Bytes of one quantized coefficient row of a tile of tl slots (tl a multiple of 8): the codes

@@ -177,12 +177,6 @@ __device__ __forceinline__ int wrap2(int x, int n) {
   return x;
 }
 
-// Keep the bf16 halves of `w` whose row index (lo half: j, hi half: j + 1) is below r.
-__device__ __forceinline__ uint32_t keep_rows(uint32_t w, int j, int r) {
-  const uint32_t m = (j < r ? 0x0000FFFFu : 0u) | (j + 1 < r ? 0xFFFF0000u : 0u);
-  return w & m;
-}
-
 // Per-sequence stream length segW[b] (equal for every head of the sequence; a table outside
 // [0, cap] counts as empty) and cost-line start segP[b] of sequence b, whose G segments take
 // kSegCost + segW[b] + kSegEnd elements each (an empty sequence takes none); segP[64] = T, the
