@@ -21,9 +21,9 @@
 // So the tensor work of one chain runs under the softmax of the other.
 // At the end of a segment the chains merge into one partial (max, sum, o~[128]) per row.
 // Bound by the two chains' latency: for a 128-slot item of rank 32 the issue of its 4 score and 8 value
-// products takes 730 + 660 cycles and its softmax 2,500 of a period of 5,200 per chain. 8 heads x 131072 tokens,
-// 128 rows: 215 us with mma.sync (decode_window.cu), 99 us here; 64 rows 113 / 93 us; 24 rows 65 / 98 us, which is
-// why up to 32 rows stay there (wide ranks, where most tiles are short: 128 rows 590 / 124 us).
+// products takes 730 + 660 cycles and its softmax 2,500 of a period of 5,200 per chain. Launch times, 8 heads x
+// 131072 tokens, 128 rows: 215 us with mma.sync (eight row groups in decode_window.cu), 97 us here; wide ranks, where
+// most tiles are short, 590 / 124 us. Where the line between the two kernels lies stands at window_rg.
 // Set aside: both groups' products from one issuing thread 125 us; weights kept in registers until the reference
 // is known to stay (one pass over the scores) 175 us, with 536 bytes spilled; two threads per row 103 us.
 // Every wait is bounded; one that gives up raises VARRATE_ERR_TIMEOUT, the CTA then streams nothing more and

@@ -52,7 +52,7 @@ def test_decode_wide_ranks(kind, n, dtype, grp, n_tail):
     assert decode_close(out[0], want, cfg), decode_errors(out[0], want)
 
 
-# rows per KV head: 32 (CUDA-core-fed kernel), 36, 64, 65, 120, 126 and 128 (tcgen05 kernel); tails past one
+# rows per KV head: 32 (the mma.sync kernel), 36, 64, 65, 120, 126 and 128 (tcgen05 kernel); tails past one
 # 128-token step of the combine
 @pytest.mark.parametrize("grp, n_q, n_tail", [(4, 8, 150), (4, 9, 9), (8, 8, 129), (5, 13, 128), (8, 15, 257), (7, 18, 40), (4, 32, 32)])
 @pytest.mark.parametrize("kind, n", [("wide", 9000), ("edges", 1500), ("ends", 4000)])

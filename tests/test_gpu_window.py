@@ -2,7 +2,7 @@
 within the window), through the C ABI.
 
 Bars: the decode bars of gpu_helpers.py per output row (one window query and head). The cases cover
-every row-group size of the kernel (n_q * group rows in 1, 2, 4 and 8 groups of 16), a partial
+both kernels (n_q * group rows in one and two groups of 16, and more than 32 rows), a partial
 second n-tile (group 7), a window that is the whole tail, tails past 256 tokens, an empty coded set,
 and causality: changing tail tokens after query i's position leaves queries 0..i bit-identical."""
 import numpy as np
@@ -83,13 +83,13 @@ def _check(c, layer, n_q, n_tail, seed=5):
     return q, tk, tv, out
 
 
-# llama group 4: n_q = 1, 4 -> one row group; 8 -> two; 16 -> four; 32 -> eight (128 rows)
+# llama group 4: n_q = 1, 4 -> one row group; 8 -> two; 16, 32 (64 and 128 rows) -> the tcgen05 kernel
 @pytest.mark.parametrize("n_q,n_tail", [(1, 1), (4, 37), (8, 8), (16, 160), (32, 32), (32, 300)])
 def test_window_matches_oracle_llama(caches, n_q, n_tail):
     _check(caches["llama"], 1, n_q, n_tail)
 
 
-# group 7: 3 queries = 21 rows (two row groups, the second with one n-tile), 18 queries = 126 rows
+# group 7: 3 queries = 21 rows (two row groups, the second with one n-tile), 5 = 35 and 18 = 126 rows (tcgen05)
 @pytest.mark.parametrize("n_q,n_tail", [(3, 40), (18, 18), (5, 257)])
 def test_window_matches_oracle_group7(caches, n_q, n_tail):
     _check(caches["qwen_g7"], 0, n_q, n_tail)
